@@ -19,112 +19,249 @@ namespace {
 // ---------------------------------------------------------------- Philox4x64-10
 // Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy as 1, 2, 3"
 // (SC 2011): 10 rounds of two 64x64->128 multiplications, Weyl key schedule.
-__device__ __forceinline__ void philox4x64_10(uint64_t &x0, uint64_t &x1, uint64_t &x2, uint64_t &x3,
-                                              uint64_t k0, uint64_t k1) {
-    const uint64_t M0 = 0xD2E7470EE14C6C93ULL, M1 = 0xCA5A826395121157ULL;
-    const uint64_t W0 = 0x9E3779B97F4A7C15ULL, W1 = 0xBB67AE8584CAA73BULL;
+// One round maps (x0, x1, x2, x3) to (hi(M1 x2) ^ x1 ^ k0, lo(M1 x2),
+// hi(M0 x0) ^ x3 ^ k1, lo(M0 x0)).  The counter is (shot, block, 0, 0), so
+// with one shot per lane the products of the first three rounds that do not
+// see the block (round 0: M0 shot; round 1: M1 x2; round 2: M0 x0) are the
+// same for all blocks of the shot and are computed once (PhiloxShot).
+constexpr uint64_t kPhiloxM0 = 0xD2E7470EE14C6C93ULL, kPhiloxM1 = 0xCA5A826395121157ULL;
+constexpr uint64_t kPhiloxW0 = 0x9E3779B97F4A7C15ULL, kPhiloxW1 = 0xBB67AE8584CAA73BULL;
+
+// 64 x 64 -> 128 bit product (both halves from one expression: the compiler
+// shares the partial products; a chain of 32 x 32 -> 64 multiply-adds written
+// out was a third slower).
+__device__ __forceinline__ void mul_wide64(uint64_t a, uint64_t m, uint64_t &hi, uint64_t &lo) {
+    hi = __umul64hi(a, m);
+    lo = a * m;
+}
+
+struct PhiloxShot {
+    uint64_t lo_shot;          // lo(M0 shot): x3 after round 0
+    uint64_t x1_r1;            // x1 after round 1
+    uint64_t hi0_r2, lo0_r2;   // M0 x0 of round 2
+};
+
+__device__ __forceinline__ PhiloxShot philox_shot(uint64_t shot, uint64_t seed) {
+    PhiloxShot s;
+    uint64_t hi;
+    mul_wide64(shot, kPhiloxM0, hi, s.lo_shot);          // round 0 (keys seed, 0): x2 = hi
+    uint64_t hi1;
+    mul_wide64(hi, kPhiloxM1, hi1, s.x1_r1);             // round 1: x0 = hi1 ^ 0 ^ (seed + W0)
+    mul_wide64(hi1 ^ (seed + kPhiloxW0), kPhiloxM0, s.hi0_r2, s.lo0_r2);
+    return s;
+}
+
+// The four words of `block` of the shot.
+__device__ __forceinline__ void philox_block(const PhiloxShot &s, uint64_t block, uint64_t seed, uint64_t (&u)[4]) {
+    uint64_t hi, lo;
+    // round 0: x0 = block ^ seed; round 1: x2 = hi(M0 x0) ^ lo_shot ^ W1, x3 = lo(M0 x0)
+    mul_wide64(block ^ seed, kPhiloxM0, hi, lo);
+    const uint64_t x2r1 = hi ^ s.lo_shot ^ kPhiloxW1, x3r1 = lo;
+    // round 2
+    mul_wide64(x2r1, kPhiloxM1, hi, lo);
+    uint64_t x0 = hi ^ s.x1_r1 ^ (seed + 2 * kPhiloxW0), x1 = lo;
+    uint64_t x2 = s.hi0_r2 ^ x3r1 ^ (2 * kPhiloxW1), x3 = s.lo0_r2;
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint64_t hi0 = __umul64hi(M0, x0), lo0 = M0 * x0;
-        const uint64_t hi1 = __umul64hi(M1, x2), lo1 = M1 * x2;
-        const uint64_t y0 = hi1 ^ x1 ^ k0, y2 = hi0 ^ x3 ^ k1;
-        x0 = y0;
-        x1 = lo1;
-        x2 = y2;
-        x3 = lo0;
-        k0 += W0;
-        k1 += W1;
+    for (int r = 3; r < 10; ++r) {
+        uint64_t h0, l0, h1, l1;
+        mul_wide64(x0, kPhiloxM0, h0, l0);
+        mul_wide64(x2, kPhiloxM1, h1, l1);
+        x0 = h1 ^ x1 ^ (seed + (uint64_t)r * kPhiloxW0);
+        x1 = l1;
+        x2 = h0 ^ x3 ^ ((uint64_t)r * kPhiloxW1);
+        x3 = l0;
     }
+    u[0] = x0;
+    u[1] = x1;
+    u[2] = x2;
+    u[3] = x3;
 }
 
-__device__ __forceinline__ uint32_t anti_code(uint32_t a, uint32_t b) {
-    return (a != 0u) & (b != 0u) & (a != b);
+// Transpose of a 32 x 32 bit matrix held one row per lane: bit c of lane r
+// becomes bit r of lane c.
+__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
+    constexpr uint32_t mask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        const int k = 16 >> s;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
+        x = (lane & k) ? (x & ~mask[s]) | ((y & ~mask[s]) >> k) : (x & mask[s]) | ((y & mask[s]) << k);
+    }
+    return x;
 }
 
-// One thread per (shot, block of 4 qubits).
-__global__ void sample_errors_kernel(int N, int B, uint64_t seed, uint64_t shot0, uint64_t tx, uint64_t ty,
-                                     uint64_t tz, uint8_t *err) {
-    const int nblk = (N + 3) / 4;
-    const long total = (long)B * nblk;
-    for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const long b = idx / nblk;
-        const int blk = (int)(idx - b * nblk);
-        uint64_t x0 = shot0 + (uint64_t)b, x1 = (uint64_t)blk, x2 = 0, x3 = 0;
-        philox4x64_10(x0, x1, x2, x3, seed, 0);
-        const uint64_t u[4] = {x0, x1, x2, x3};
+// Which planes of a qubit's two-bit code enter <., p>: the code's parity
+// with mask m(p), m(X) = 2, m(Y) = 1, m(Z) = 3 (codes 0 I, 1 X, 2 Y, 3 Z: bit
+// 1 is the Z part, bit 0 ^ bit 1 the X part), on words of 32 shots.
+__device__ __forceinline__ uint32_t anti_word(uint2 c, uint32_t p) {
+    return (p == 2u || p == 3u ? c.x : 0u) ^ (p == 1u || p == 3u ? c.y : 0u);
+}
+
+// XOR over a check's qubits of anti_word (planes: one uint2 per qubit).
+__device__ __forceinline__ uint32_t check_word(const uint16_t *chk_slot, const uint8_t *chk_pauli, int i,
+                                               const uint2 *planes) {
+    const uint32_t cp = chk_pauli[i];
+    const uint2 s = *reinterpret_cast<const uint2 *>(chk_slot + 4 * i);
+    const uint32_t sl[4] = {s.x & 0xFFFFu, s.x >> 16, s.y & 0xFFFFu, s.y >> 16};
+    uint32_t w = 0;
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+        if (sl[n] != kNoSlot) {
+            const uint32_t p = (cp >> (2 * n)) & 3u;
+            const uint2 c = planes[sl[n] >> 2];
+            w ^= p == 2u ? c.x : p == 1u ? c.y : c.x ^ c.y;
+        }
+    return w;
+}
+
+// Errors and syndromes of 32 consecutive shots per CTA.  Lane s of every warp
+// is shot s; the warps share the shot's blocks of four qubits.  A block's codes go to
+// shared memory one word per (shot, block), and warp votes turn them into bit
+// planes (one word per qubit and code bit, bit s = shot s), from which a
+// thread forms one check's syndrome for all 32 shots with four loads; 32 x 32
+// bit transposes give the packed words.  Errors and syndromes of the tile are
+// contiguous in memory and leave in 32-bit stores.
+// Bound: the Philox multiplications (15 of the 20 per block are left per
+// shot).  The two kernels this replaces (errors, then syndromes from the errors
+// in memory, a byte load per edge) took 305 + 431 us for 10^6 planar d = 7 shots.
+// Shared memory: codes [32][cw] | planes uint2[N] | syn [32][W].
+__global__ void sample_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli, int N, int M, int W, int B,
+                              uint64_t seed, uint64_t shot0, uint64_t tx, uint64_t ty, uint64_t tz, uint8_t *err,
+                              uint32_t *syn) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    const int nblk = (N + 3) / 4, cw = nblk | 1;  // odd row stride: lanes (shots) hit distinct banks
+    uint32_t *codes = reinterpret_cast<uint32_t *>(smem);
+    uint2 *planes = reinterpret_cast<uint2 *>(codes + 32 * cw);
+    uint32_t *words = reinterpret_cast<uint32_t *>(planes + N);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const long b0 = 32L * blockIdx.x;
+    const int cnt = B - b0 < 32 ? (int)(B - b0) : 32;
+
+    const PhiloxShot ps = philox_shot(shot0 + (uint64_t)(b0 + lane), seed);
+    for (int blk = warp; blk < nblk; blk += nwarps) {
+        uint64_t u[4];
+        philox_block(ps, (uint64_t)blk, seed, u);
+        uint32_t word = 0;
+        uint2 mine = make_uint2(0u, 0u);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-            const int j = 4 * blk + l;
-            if (j < N) err[b * N + j] = u[l] < tx ? 1 : u[l] < ty ? 2 : u[l] < tz ? 3 : 0;
+            // thresholds tx <= ty <= tz: X below tx, Y below ty, Z below tz
+            const bool bx = u[l] < tx, by = u[l] < ty, bz = u[l] < tz;
+            const uint32_t code = bx ? 1u : by ? 2u : bz ? 3u : 0u;
+            word |= code << (8 * l);
+            // bit 0 of the code: X or Z; bit 1: Y or Z
+            const uint32_t vx = __ballot_sync(0xffffffffu, bx), vy = __ballot_sync(0xffffffffu, by),
+                           vz = __ballot_sync(0xffffffffu, bz);
+            if (lane == l) mine = make_uint2(vx | (vz & ~vy), vz & ~vx);
+        }
+        codes[lane * cw + blk] = word;
+        if (lane < 4 && 4 * blk + lane < N) planes[4 * blk + lane] = mine;
+    }
+    __syncthreads();
+
+    for (int i0 = 32 * warp; i0 < M; i0 += 32 * nwarps) {
+        const int i = i0 + lane;
+        const uint32_t w = warp_transpose32(i < M ? check_word(chk_slot, chk_pauli, i, planes) : 0u, lane);
+        words[lane * W + (i0 >> 5)] = w;
+    }
+    // the tile's errors: byte o is qubit o % N of shot o / N (o < 2^16 and
+    // N <= 2^11, so the product with ceil(2^32 / N) gives o / N exactly)
+    uint8_t *e = err + b0 * N;
+    const uint8_t *cb = reinterpret_cast<const uint8_t *>(codes);
+    const uint32_t inv = 0xFFFFFFFFu / (uint32_t)N + 1u;
+    const int bytes = cnt * N;
+    int done = 0;
+    if ((reinterpret_cast<uintptr_t>(e) & 3u) == 0 && N >= 4) {
+        done = bytes & ~3;
+        for (int o = 4 * threadIdx.x; o < done; o += 4 * blockDim.x) {
+            const int s = (int)__umulhi((uint32_t)o, inv), j = o - s * N;
+            const uint32_t *row = codes + s * cw + (j >> 2);
+            uint32_t v = __funnelshift_r(row[0], row[1], 8 * (j & 3));
+            const int left = N - j;  // codes of this shot from j on
+            if (left < 4) v = (v & ((1u << (8 * left)) - 1u)) | (codes[(s + 1) * cw] << (8 * left));
+            *reinterpret_cast<uint32_t *>(e + o) = v;
         }
     }
-}
-
-// One warp per (shot, 32-check word); lane l computes check 32 w + l.
-__global__ void syndrome_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli, int N, int M, int W, int B,
-                                const uint8_t *err, uint32_t *syn) {
-    const long gw = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (gw >= (long)B * W) return;
-    const long b = gw / W;
-    const int w = (int)(gw - b * W);
-    const int i = 32 * w + lane;
-    uint32_t bit = 0;
-    if (i < M) {
-        const uint32_t cp = chk_pauli[i];
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const uint32_t sl = chk_slot[4 * i + n];
-            if (sl != kNoSlot) bit ^= anti_code(err[b * N + (sl >> 2)], (cp >> (2 * n)) & 3u);
-        }
+    for (int o = done + threadIdx.x; o < bytes; o += blockDim.x) {
+        const int s = o / N;
+        e[o] = cb[4 * s * cw + (o - s * N)];
     }
-    const uint32_t word = __ballot_sync(0xffffffffu, bit);
-    if (lane == 0) syn[b * W + w] = word;
+    __syncthreads();
+    for (int k = threadIdx.x; k < cnt * W; k += blockDim.x) syn[b0 * W + k] = words[k];
 }
 
-__device__ __forceinline__ uint32_t xbit(uint32_t c) { return (c == 1u) | (c == 2u); }
-__device__ __forceinline__ uint32_t zbit(uint32_t c) { return (c == 2u) | (c == 3u); }
+// Four codes, one per byte; values above 3 (no Pauli code) count as I.
+__device__ __forceinline__ uint32_t valid_codes(uint32_t v) {
+    const uint32_t bad = v & 0xFCFCFCFCu;
+    if (bad == 0) return v;
+    uint32_t r = 0;
+    for (int l = 0; l < 4; ++l)
+        if (!((bad >> (8 * l)) & 0xFFu)) r |= v & (0xFFu << (8 * l));
+    return r;
+}
 
-// One warp per shot: residual R = E^ E; 1 if R anticommutes with a check,
-// 2 if it commutes with all checks but not with all logical operators.
+// Classification of 32 consecutive shots per CTA: residual R = E^ E; 1 if R
+// anticommutes with a check, 2 if it commutes with all checks but not with all
+// logical operators.  The codes of a product are the XOR of the codes, so the
+// tile's residuals are the XOR of the two arrays, read once in 32-bit words;
+// warp votes turn them into bit planes (bit s of a qubit's word = shot s), and
+// a thread then tests one check for all 32 shots with four loads.
+// Bound: the tile's passes through shared memory; one warp per shot with
+// byte loads per edge took 775 us for 10^6 planar d = 7 shots; this takes
+// 104 us (174 MB of memory traffic).
+// Shared memory: residuals, 32 rows of `stride` bytes | planes uint2[N] | two
+// words.  Rows are contiguous as in memory when N is no multiple of 4, else
+// padded to an odd number of words (lanes read the same qubit of 32 rows).
 __global__ void check_logical_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli, const uint8_t *logicals,
-                                     int nlog, int N, int M, int B, const uint8_t *err, const uint8_t *est,
-                                     uint8_t *fail_out) {
-    const long b = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (b >= B) return;
-    const uint8_t *e = err + b * N, *h = est + b * N;
+                                     int nlog, int N, int M, int B, int stride, const uint8_t *err,
+                                     const uint8_t *est, uint8_t *fail_out) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    uint2 *planes = reinterpret_cast<uint2 *>(smem + ((32 * stride + 7) & ~7));
+    uint32_t *verdict = reinterpret_cast<uint32_t *>(planes + N);  // [0] detected, [1] logical (bit = shot)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const long b0 = 32L * blockIdx.x;
+    const int cnt = B - b0 < 32 ? (int)(B - b0) : 32;
+    const uint8_t *e = err + b0 * N, *h = est + b0 * N;
+    if (threadIdx.x < 2) verdict[threadIdx.x] = 0u;
+    const int bytes = cnt * N;
+    const bool words = ((reinterpret_cast<uintptr_t>(e) | reinterpret_cast<uintptr_t>(h)) & 3u) == 0;
+    const int done = words ? bytes & ~3 : 0;
+    for (int o = 4 * threadIdx.x; o < done; o += 4 * blockDim.x) {
+        const uint32_t r = valid_codes(__ldg(reinterpret_cast<const uint32_t *>(e + o))) ^
+                           valid_codes(__ldg(reinterpret_cast<const uint32_t *>(h + o)));
+        const int at = stride == N ? o : (o / N) * stride + o % N;  // padded rows: N and stride multiples of 4
+        *reinterpret_cast<uint32_t *>(smem + at) = r;
+    }
+    for (int o = done + threadIdx.x; o < bytes; o += blockDim.x) {
+        const int s = o / N;
+        smem[s * stride + (o - s * N)] = (uint8_t)(valid_codes(e[o]) ^ valid_codes(h[o]));
+    }
+    __syncthreads();
+    const uint8_t *row = smem + (lane < cnt ? lane : 0) * stride;
+    for (int j0 = 32 * warp; j0 < N; j0 += 32 * nwarps) {
+        uint2 mine = make_uint2(0u, 0u);
+        const int n = N - j0 < 32 ? N - j0 : 32;
+        for (int l = 0; l < n; ++l) {
+            const uint32_t c = row[j0 + l];
+            const uint32_t p0 = __ballot_sync(0xffffffffu, c & 1u), p1 = __ballot_sync(0xffffffffu, c & 2u);
+            if (lane == l) mine = make_uint2(p0, p1);
+        }
+        if (lane < n) planes[j0 + lane] = mine;
+    }
+    __syncthreads();
     uint32_t det = 0;
-    for (int i = lane; i < M; i += 32) {
-        const uint32_t cp = chk_pauli[i];
+    for (int i = threadIdx.x; i < M; i += blockDim.x) det |= check_word(chk_slot, chk_pauli, i, planes);
+    det = __reduce_or_sync(0xffffffffu, det);
+    if (lane == 0 && det) atomicOr(verdict, det);
+    for (int l = warp; l < nlog; l += nwarps) {
         uint32_t par = 0;
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const uint32_t sl = chk_slot[4 * i + n];
-            if (sl != kNoSlot) {
-                const int j = sl >> 2;
-                const uint32_t rx = xbit(e[j]) ^ xbit(h[j]), rz = zbit(e[j]) ^ zbit(h[j]);
-                const uint32_t p = (cp >> (2 * n)) & 3u;
-                par ^= (rx & zbit(p)) ^ (rz & xbit(p));
-            }
-        }
-        det |= par;
+        for (int j = lane; j < N; j += 32) par ^= anti_word(planes[j], logicals[(size_t)l * N + j]);
+        par = __reduce_xor_sync(0xffffffffu, par);
+        if (lane == 0 && par) atomicOr(verdict + 1, par);
     }
-    const bool detected = __any_sync(0xffffffffu, det) != 0;
-    bool logical = false;
-    if (!detected) {
-        for (int l = 0; l < nlog; ++l) {
-            uint32_t par = 0;
-            for (int j = lane; j < N; j += 32) {
-                const uint32_t rx = xbit(e[j]) ^ xbit(h[j]), rz = zbit(e[j]) ^ zbit(h[j]);
-                const uint32_t p = logicals[(size_t)l * N + j];
-                par ^= (rx & zbit(p)) ^ (rz & xbit(p));
-            }
-            const uint32_t odd = __popc(__ballot_sync(0xffffffffu, par)) & 1u;
-            if (odd) logical = true;
-        }
-    }
-    if (lane == 0) fail_out[b] = detected ? 1 : logical ? 2 : 0;
+    __syncthreads();
+    if (warp == 0 && lane < cnt)
+        fail_out[b0 + lane] = ((verdict[0] >> lane) & 1u) ? 1 : ((verdict[1] >> lane) & 1u) ? 2 : 0;
 }
 
 
@@ -158,9 +295,20 @@ uint64_t threshold(double c) {
 }
 
 int launch_grid(long items, int per_block) {
-    long g = (items + per_block - 1) / per_block;
-    if (g > (1L << 30)) g = 1L << 30;
+    const long g = (items + per_block - 1) / per_block;
     return (int)(g < 1 ? 1 : g);
+}
+
+// Warps of a CTA that works on a tile of 32 shots in `units` equal steps (32
+// threads each): about six steps a warp where there are tiles for every SM
+// (the tile's barriers and per-warp set-up cost less then), one step a warp
+// while the tiles leave SMs idle.
+int tile_warps(const bpq_tanner *t, int B, int units) {
+    const long tiles = (B + 31L) / 32;
+    const int most = units < 1 ? 1 : units > 16 ? 16 : units;
+    if (tiles < 4L * t->num_sms) return most;
+    const int w = (units + 5) / 6;
+    return w < 4 ? (most < 4 ? most : 4) : w > 16 ? 16 : w;
 }
 
 // ---------------------------------------------------------------- no-allocation staging
@@ -463,14 +611,16 @@ int bpq_sample(const bpq_tanner *t, double px, double py, double pz, uint64_t se
     if (B == 0) return BPQ_OK;
     if (!err_dev || !syn_dev) return fail(BPQ_EINVAL, "NULL output");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int nblk = (t->N + 3) / 4;
-    bpq::sample_errors_kernel<<<bpq::launch_grid((long)B * nblk, 256), 256, 0, st>>>(
-        t->N, B, seed, shot0, bpq::threshold(cx), bpq::threshold(cy), bpq::threshold(cz), err_dev);
-    const int W = (t->M + 31) / 32;
-    if (t->M > 0)
-        bpq::syndrome_kernel<<<bpq::launch_grid((long)B * W * 32, 256), 256, 0, st>>>(
-            reinterpret_cast<const uint16_t *>(t->d_table), t->d_table + t->off_chk_pauli, t->N, t->M, W, B, err_dev,
-            syn_dev);
+    const int nblk = (t->N + 3) / 4, W = (t->M + 31) / 32;
+    const size_t smem = 4 * (size_t)32 * (nblk | 1) + 8 * (size_t)t->N + 4 * (size_t)32 * W;
+    if (smem > 48 * 1024) {
+        rc = bpq::cuda_check(cudaFuncSetAttribute(bpq::sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem), "sample attribute");
+        if (rc) return rc;
+    }
+    bpq::sample_kernel<<<bpq::launch_grid(B, 32), 32 * bpq::tile_warps(t, B, nblk), smem, st>>>(
+        reinterpret_cast<const uint16_t *>(t->d_table), t->d_table + t->off_chk_pauli, t->N, t->M, W, B, seed, shot0,
+        bpq::threshold(cx), bpq::threshold(cy), bpq::threshold(cz), err_dev, syn_dev);
     return bpq::cuda_check(cudaGetLastError(), "sample launch");
 }
 
@@ -709,9 +859,17 @@ int bpq_check_logical(const bpq_tanner *t, const uint8_t *err_dev, const uint8_t
     if (B == 0) return BPQ_OK;
     if (!err_dev || !est_dev || !fail_dev) return fail(BPQ_EINVAL, "NULL argument");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    bpq::check_logical_kernel<<<bpq::launch_grid((long)B * 32, 256), 256, 0, st>>>(
+    const int stride = t->N % 4 ? t->N : 4 * ((t->N / 4) | 1);
+    const size_t smem = (((size_t)32 * stride + 7) & ~size_t(7)) + 8 * (size_t)t->N + 8;
+    if (smem > 48 * 1024) {
+        rc = bpq::cuda_check(cudaFuncSetAttribute(bpq::check_logical_kernel,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                             "check_logical attribute");
+        if (rc) return rc;
+    }
+    bpq::check_logical_kernel<<<bpq::launch_grid(B, 32), 32 * bpq::tile_warps(t, B, (t->N + 31) / 32), smem, st>>>(
         reinterpret_cast<const uint16_t *>(t->d_table), t->d_table + t->off_chk_pauli, t->d_logicals,
-        (int)(t->logicals.size() / t->N), t->N, t->M, B, err_dev, est_dev, fail_dev);
+        (int)(t->logicals.size() / t->N), t->N, t->M, B, stride, err_dev, est_dev, fail_dev);
     return bpq::cuda_check(cudaGetLastError(), "check_logical launch");
 }
 
