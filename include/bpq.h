@@ -238,10 +238,12 @@ int bpq_decode_trace(const bpq_tanner *t, const uint32_t *syn_dev, const float *
  * with at most 512 threads) and shot groups per CTA (at most 15, or 32 for
  * one-warp groups).  A shot group decodes one shot at a time, or two with two
  * shots per thread (bpq_set_shots_per_thread; then at most 2 nodes per
- * thread and 28 one-warp groups per CTA).  0 = let the library choose (two
- * nodes per thread, about 256 threads per CTA).  Stored in the
- * handle; bpq_get_launch reports the shape of the plain/Momentum/AdaGrad/
- * EWAInit kernels. */
+ * thread and 28 one-warp groups per CTA).  0 = let the library choose: two
+ * nodes per thread and about 256 threads per CTA; with two shots per thread
+ * one warp per group up to 96 nodes, and 256 threads per group above 512
+ * nodes where shared memory holds two such CTAs per SM (so the choice can
+ * depend on the variant's state).  Stored in the handle; bpq_get_launch
+ * reports the shape for Momentum-BP. */
 int bpq_set_launch(bpq_tanner *t, int threads_per_shot, int shots_per_cta);
 int bpq_get_launch(const bpq_tanner *t, int *threads_per_shot, int *shots_per_cta, int *ctas);
 
@@ -252,10 +254,11 @@ int bpq_get_launch(const bpq_tanner *t, int *threads_per_shot, int *shots_per_ct
  * next shot from the queue as soon as its own shot stops (split table layout
  * only, see bpq_tanner_layout; plain, Momentum, AdaGrad and EWAInit BP; not
  * the trace, serial, batched or AEWA-BP paths); 0 = automatic (2 where it
- * applies and the batch holds at least 128 shots per resident one-shot shot
- * group, e.g. 77824 toric d = 15 shots on a GB300: a pair's iteration does two
- * shots' work, so smaller batches, whose time is set by their slowest shots,
- * finish sooner with one shot per thread).  Per-shot results are the same
+ * applies and the batch holds at least 40 shots per resident one-shot shot
+ * group, e.g. 24320 toric d = 15 shots on a GB300 - 192 for codes of at most
+ * 96 nodes: a pair's iteration does two shots' work, so smaller batches, whose
+ * time is set by their slowest shots, finish sooner with one shot per
+ * thread).  Per-shot results are the same
  * bit for bit either way.  bpq_get_shots_per_thread reports what bpq_decode
  * will use for `variant` on large batches.
  * Errors: EINVAL (value outside 0..2, 2 on a table without the split

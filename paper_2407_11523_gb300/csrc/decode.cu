@@ -23,13 +23,13 @@ DecodeKernelFn pick(int variant, int npt, bool trace, int layout) {
     return nullptr;
 }
 
-DecodeKernelFn pick_pair(int variant, int npt, int layout) {
+DecodeKernelFn pick_pair(int variant, bool one, int layout) {
     const bool full = layout == 2;
     switch (variant) {
-        case BPQ_PLAIN: return full ? pick_plain_pair_full(npt) : pick_plain_pair(npt);
-        case BPQ_MOMENTUM: return full ? pick_momentum_pair_full(npt) : pick_momentum_pair(npt);
-        case BPQ_ADAGRAD: return full ? pick_adagrad_pair_full(npt) : pick_adagrad_pair(npt);
-        case BPQ_EWAINIT: return full ? pick_ewainit_pair_full(npt) : pick_ewainit_pair(npt);
+        case BPQ_PLAIN: return full ? pick_plain_pair_full(one) : pick_plain_pair(one);
+        case BPQ_MOMENTUM: return full ? pick_momentum_pair_full(one) : pick_momentum_pair(one);
+        case BPQ_ADAGRAD: return full ? pick_adagrad_pair_full(one) : pick_adagrad_pair(one);
+        case BPQ_EWAINIT: return full ? pick_ewainit_pair_full(one) : pick_ewainit_pair(one);
     }
     return nullptr;
 }
@@ -50,14 +50,34 @@ bool decode_uses_pairs(const bpq_tanner *t, int variant, bool trace) {
 
 int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     const int nodes = t->N > t->M ? t->N : t->M;
-    int T = t->threads_per_shot;
-    if (T <= 0) T = (((nodes + 1) / 2 + 31) / 32) * 32;  // two nodes per thread
+    const int nstate = state_arrays(variant), n_pad = (t->N + 3) & ~3;
+    const uint32_t slots = (uint32_t)(4 * n_pad + 4);  // float2 slots
+    // per group: two vote words (16 bytes) | float2 slots | float2 state
+    const size_t group_bytes = kPairVoteBytes + 8 * (size_t)slots + 8 * (size_t)(nstate * n_pad);
+    const size_t one_smem = pair_offsets(variant, true, t->M, n_pad).groups + group_bytes;
+    int T = t->threads_per_shot, gpc = t->shots_per_cta;
+    if (T <= 0) {
+        // Automatic.  Two nodes per thread, except that a code of at most 96
+        // nodes takes one warp per group (no barrier, warp votes only: planar
+        // d = 7, 10^6 shots, EWAInit 2.97 ms against 3.29 with two warps, d = 6
+        // 0.94 against 1.07; d = 8, four nodes per lane, 1.61 against 1.49), and
+        // a code of more than 512 nodes takes 256 threads where shared memory
+        // holds two such CTAs (more nodes per thread but more shots per SM:
+        // plain BP on planar d = 25, 30001 shots, 18.9 ms against 23.0, d = 21
+        // 11.9 against 13.7; with one CTA per SM it is slower: EWAInit on
+        // planar d = 25, 5.8 against 5.0).  One group per CTA but for the
+        // one-warp groups (planar d = 11 with 128 threads: 4.41 against 4.56).
+        T = (((nodes + 1) / 2 + 31) / 32) * 32;
+        if (nodes <= 96) T = 32;
+        else if (nodes > 512 && 2 * (one_smem + 1024) <= 228 * 1024) T = 256;
+        if (gpc <= 0) gpc = T == 32 ? 8 : 1;
+    } else if ((nodes + T - 1) / T > 2) {
+        return fail(BPQ_EINVAL, "two shots per thread take at most two nodes per thread");
+    }
     if (T % 32 || T < 32 || T > kMaxThreadsPerShot)
         return fail(BPQ_EINVAL, "threads per shot group must be a multiple of 32 in [32, 1024]");
     const int npt = (nodes + T - 1) / T;
-    if (npt > 2) return fail(BPQ_EINVAL, "two shots per thread take at most two nodes per thread");
     const int max_groups = T == 32 ? kMaxPairGroupsPerCta : 15;
-    int gpc = t->shots_per_cta;
     if (gpc <= 0) gpc = 256 / T > 0 ? 256 / T : 1;  // about 256 threads per CTA
     if (gpc > max_groups) gpc = max_groups;
     while (gpc > 1 && gpc * T > 1024) --gpc;
@@ -65,13 +85,12 @@ int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     s->G = T / 32;
     s->npt = npt;
     s->groups_per_cta = gpc;
-    s->n_pad = (t->N + 3) & ~3;
-    s->slots_floats = (uint32_t)(4 * s->n_pad + 4);  // float2 slots
-    const int nstate = state_arrays(variant);
-    // per group: two vote words (16 bytes) | float2 slots | float2 state
-    s->group_bytes = (uint32_t)(16 + 8 * s->slots_floats + 8 * nstate * s->n_pad);
-    // table | Pi [3][n_pad] | initial messages [4 n_pad] | groups
-    s->smem = kSmemHeader + t->table.size() + (size_t)28 * s->n_pad + (size_t)gpc * s->group_bytes;
+    s->n_pad = n_pad;
+    s->slots_floats = slots;
+    s->group_bytes = (uint32_t)group_bytes;
+    s->one = gpc == 1 && one_smem <= 227 * 1024;
+    s->smem = s->one ? one_smem
+                     : pair_offsets(variant, false, t->M, n_pad).groups + (size_t)gpc * group_bytes;
     if (s->smem > 227 * 1024) return fail(BPQ_EINVAL, "shared memory of the launch shape exceeds 227 KB");
     return BPQ_OK;
 }
@@ -160,9 +179,12 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // automatic choice: a pair's iteration does two shots' work, so a
         // batch's tail (its slowest shots) runs longer; pairing pays only
         // once each resident one-shot group would decode many shots.
-        // Measured on GB300 (EWAInit-BP): toric d = 15 pairs win from 65536
-        // shots, planar d = 25 from 16384, both about 100 shots per resident
-        // one-shot group; planar d = 9 breaks even at 262144 (172 per group)
+        // Measured on GB300, one shot per thread against two (ms): toric
+        // d = 15 EWAInit 20000 shots 1.298 / 1.279, 65536 3.93 / 3.73; planar
+        // d = 9 plain 50000 1.62 / 1.60; planar d = 21 Momentum 5000 2.32 /
+        // 2.28: all at 16 to 33 shots per resident one-shot group.  One-warp
+        // pair groups have the longest tail: planar d = 7 EWAInit 300000 shots
+        // (123 per group) 0.986 / 1.027, 10^6 in favour of pairs.
         LaunchShape one;
         int per_sm = 0;
         DecodeKernelFn f1 = nullptr;
@@ -170,19 +192,20 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one.smem) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
-            (long)a.B < kPairShotsPerGroup * (long)per_sm * t->num_sms * one.groups_per_cta)
+            decode_pair_shape(t, variant, &s) == BPQ_OK &&
+            (long)a.B < pair_shots_per_group(s.T) * (long)per_sm * t->num_sms * one.groups_per_cta)
             pairs = false;
     }
     int rc = pairs ? decode_pair_shape(t, variant, &s) : decode_launch_shape(t, variant, &s);
     if (rc) return rc;
     DecodeKernelFn fn = nullptr;
     if (t->debug_checks) {
-        fn = trace ? nullptr : pick_debug(variant, s.npt, pairs, a.split);
+        fn = trace ? nullptr : pick_debug(variant, s.npt, pairs, s.one, a.split);
         if (!fn)
             return fail(BPQ_EINVAL, "no bounds-checked kernel for this launch (plain, Momentum, AdaGrad or EWAInit BP, "
                                     "at most two nodes per thread, not a trace)");
     } else {
-        fn = pairs ? pick_pair(variant, s.npt, a.split) : pick(variant, s.npt, trace, a.split);
+        fn = pairs ? pick_pair(variant, s.one, a.split) : pick(variant, s.npt, trace, a.split);
     }
     if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant (AEWA-BP has no trace mode)");
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);

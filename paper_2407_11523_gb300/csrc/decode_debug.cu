@@ -13,12 +13,13 @@ namespace bpq {
 namespace {
 
 template <int V>
-DecodeKernelFn pick_debug_v(int npt, bool pairs, int layout) {
+DecodeKernelFn pick_debug_v(int npt, bool pairs, bool one, int layout) {
     if (pairs) {
-        if (layout == 2) return npt == 1 ? dk_debug::decode_pair_kernel<V, 1, true> : dk_debug::decode_pair_kernel<V, 2, true>;
-        if (layout == 1) return npt == 1 ? dk_debug::decode_pair_kernel<V, 1, false> : dk_debug::decode_pair_kernel<V, 2, false>;
+        if (layout == 2) return one ? dk_debug::decode_pair_kernel<V, true, true> : dk_debug::decode_pair_kernel<V, true, false>;
+        if (layout == 1) return one ? dk_debug::decode_pair_kernel<V, false, true> : dk_debug::decode_pair_kernel<V, false, false>;
         return nullptr;
     }
+    if (npt < 1 || npt > 2) return nullptr;
     switch (layout) {
         case 2: return npt == 1 ? dk_debug::decode_kernel<V, 1, false, true, true> : dk_debug::decode_kernel<V, 2, false, true, true>;
         case 1: return npt == 1 ? dk_debug::decode_kernel<V, 1, false, true, false> : dk_debug::decode_kernel<V, 2, false, true, false>;
@@ -28,13 +29,12 @@ DecodeKernelFn pick_debug_v(int npt, bool pairs, int layout) {
 
 }  // namespace
 
-DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int layout) {
-    if (npt < 1 || npt > 2) return nullptr;
+DecodeKernelFn pick_debug(int variant, int npt, bool pairs, bool one, int layout) {
     switch (variant) {
-        case BPQ_PLAIN: return pick_debug_v<BPQ_PLAIN>(npt, pairs, layout);
-        case BPQ_MOMENTUM: return pick_debug_v<BPQ_MOMENTUM>(npt, pairs, layout);
-        case BPQ_ADAGRAD: return pick_debug_v<BPQ_ADAGRAD>(npt, pairs, layout);
-        case BPQ_EWAINIT: return pick_debug_v<BPQ_EWAINIT>(npt, pairs, layout);
+        case BPQ_PLAIN: return pick_debug_v<BPQ_PLAIN>(npt, pairs, one, layout);
+        case BPQ_MOMENTUM: return pick_debug_v<BPQ_MOMENTUM>(npt, pairs, one, layout);
+        case BPQ_ADAGRAD: return pick_debug_v<BPQ_ADAGRAD>(npt, pairs, one, layout);
+        case BPQ_EWAINIT: return pick_debug_v<BPQ_EWAINIT>(npt, pairs, one, layout);
     }
     return nullptr;
 }

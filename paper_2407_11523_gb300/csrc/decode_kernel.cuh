@@ -485,16 +485,25 @@ __device__ __forceinline__ void load_adjacency(const DecodeArgs &a, const uint8_
     }
 }
 
-// Prior LLRs Pi_{v_j,W} = ln(p^I / p^W) of a code into shared memory
-// ([3][n_pad], computed by all threads of the CTA).
+// Prior LLRs Pi_{v_j,W} = ln(p^I / p^W) of qubit j, in bits.
+__device__ __forceinline__ void prior_llr(const DecodeArgs &a, int j, float (&P)[3]) {
+    const float px = a.prior[3 * j], py = a.prior[3 * j + 1], pz = a.prior[3 * j + 2];
+    const float pI = 1.0f - px - py - pz;
+    P[0] = log2f(pI / px);
+    P[1] = log2f(pI / py);
+    P[2] = log2f(pI / pz);
+}
+
+// The prior LLRs of a code into shared memory ([3][n_pad], computed by all
+// threads of the CTA).
 __device__ __forceinline__ void load_prior(const DecodeArgs &a, float *PiS) {
     const int Np = a.n_pad;
     for (int j = threadIdx.x; j < a.N; j += blockDim.x) {
-        const float px = a.prior[3 * j], py = a.prior[3 * j + 1], pz = a.prior[3 * j + 2];
-        const float pI = 1.0f - px - py - pz;
-        PiS[j] = log2f(pI / px);
-        PiS[Np + j] = log2f(pI / py);
-        PiS[2 * Np + j] = log2f(pI / pz);
+        float P[3];
+        prior_llr(a, j, P);
+        PiS[j] = P[0];
+        PiS[Np + j] = P[1];
+        PiS[2 * Np + j] = P[2];
     }
 }
 

@@ -66,6 +66,7 @@ struct LaunchShape {
     int n_pad;
     uint32_t slots_floats, group_bytes;
     size_t smem;
+    bool one = false;  // two shots per thread: the kernel for one shot group per CTA
 };
 
 using DecodeKernelFn = void (*)(const DecodeArgs);
@@ -90,20 +91,21 @@ BatchKernelFn pick_plain_batch(bool generic);
 BatchKernelFn pick_momentum_batch(bool generic);
 BatchKernelFn pick_adagrad_batch(bool generic);
 BatchKernelFn pick_ewainit_batch(bool generic);
-// Two shots per thread (decode_pair.cuh), split tables, npt in {1, 2}; the
-// _full functions for split tables without padding.
-DecodeKernelFn pick_plain_pair(int npt);
-DecodeKernelFn pick_plain_pair_full(int npt);
-DecodeKernelFn pick_momentum_pair(int npt);
-DecodeKernelFn pick_momentum_pair_full(int npt);
-DecodeKernelFn pick_adagrad_pair(int npt);
-DecodeKernelFn pick_adagrad_pair_full(int npt);
-DecodeKernelFn pick_ewainit_pair(int npt);
-DecodeKernelFn pick_ewainit_pair_full(int npt);
+// Two shots per thread (decode_pair.cuh), split tables; one: one shot group
+// per CTA; the _full functions for split tables without padding.
+DecodeKernelFn pick_plain_pair(bool one);
+DecodeKernelFn pick_plain_pair_full(bool one);
+DecodeKernelFn pick_momentum_pair(bool one);
+DecodeKernelFn pick_momentum_pair_full(bool one);
+DecodeKernelFn pick_adagrad_pair(bool one);
+DecodeKernelFn pick_adagrad_pair_full(bool one);
+DecodeKernelFn pick_ewainit_pair(bool one);
+DecodeKernelFn pick_ewainit_pair_full(bool one);
 
 // Bounds-checked kernels (decode_debug.cu; bpq_set_debug_checks): npt in
-// {1, 2}, pairs on split layouts; nullptr where none is compiled.
-DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int layout);
+// {1, 2} with one shot per thread, pairs on split layouts (one: one shot
+// group per CTA); nullptr where none is compiled.
+DecodeKernelFn pick_debug(int variant, int npt, bool pairs, bool one, int layout);
 
 int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 // Whether bpq_decode runs the two-shots-per-thread kernel for this graph and
@@ -112,9 +114,30 @@ int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 bool decode_uses_pairs(const bpq_tanner *t, int variant, bool trace);
 int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 constexpr int kMaxPairGroupsPerCta = 28;  // two shot indices per group in the 256-byte header
-// Automatic choice of two shots per thread: from this many shots per
-// resident one-shot group of the batch.
-constexpr long kPairShotsPerGroup = 128;
+constexpr int kPairMaxNodes = 16;         // nodes per thread: two bits of a 32-bit word each
+
+// Shared memory of the two-shots-per-thread kernels, read by the kernel and
+// by the host's sizing: byte offsets of the CTA's tables and of its first
+// shot group.  idx: four slots per check, 32-bit byte offsets in the kernels
+// for one group per CTA, else 16-bit indices; prior: one float per Pauli and qubit, two
+// equal ones for plain BP.
+__host__ __device__ constexpr int pair_prior_copies(int variant) { return variant == BPQ_PLAIN ? 2 : 1; }
+constexpr uint32_t kPairVoteBytes = 16;
+struct PairOffsets {
+    uint32_t idx, used, prior, init, groups;
+};
+__host__ __device__ inline PairOffsets pair_offsets(int variant, bool one, int M, int n_pad) {
+    PairOffsets o;
+    o.idx = kSmemHeader;
+    o.used = o.idx + (one ? 16u : 8u) * (uint32_t)((M + 1) & ~1);
+    o.prior = o.used + (((uint32_t)n_pad + 15u) & ~15u);
+    o.init = o.prior + 12u * (uint32_t)(pair_prior_copies(variant) * n_pad);
+    o.groups = o.init + 16u * (uint32_t)n_pad;
+    return o;
+}
+// Automatic choice of two shots per thread: from this many shots of the batch
+// per resident one-shot group (T: threads of a pair group).
+constexpr long pair_shots_per_group(int T) { return T == 32 ? 192 : 40; }
 // Shape of a code inside the batched kernel (CTAs of kBatchThreads threads).
 int decode_batch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 
