@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libbpq.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["api.cu", "batch.cu", "server.cu", "train.cu", "decode.cu", "decode_plain.cu", "decode_momentum.cu", "decode_adagrad.cu",
+SOURCES = ["api.cu", "batch.cu", "server.cu", "train.cu", "decode.cu", "decode_small.cu", "decode_plain.cu", "decode_momentum.cu", "decode_adagrad.cu",
            "decode_ewainit.cu", "decode_aewa.cu", "decode_plain_full.cu", "decode_momentum_full.cu",
            "decode_adagrad_full.cu", "decode_ewainit_full.cu", "decode_aewa_full.cu", "decode_plain_pair.cu",
            "decode_momentum_pair.cu", "decode_adagrad_pair.cu", "decode_ewainit_pair.cu", "decode_plain_batch.cu",

@@ -640,8 +640,6 @@ int bpq_decode(const bpq_tanner *t, const uint32_t *syn_dev, const float *prior_
     a.conv = conv_dev;
     a.iters = iters_dev;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = bpq::cuda_check(cudaMemsetAsync(work_dev, 0, 8, st), "workspace reset");
-    if (rc) return rc;
     return bpq::decode_launch(t, a, variant, false, st, nullptr);
 }
 
@@ -714,8 +712,6 @@ int bpq_decode_trace(const bpq_tanner *t, const uint32_t *syn_dev, const float *
     a.tr_Q = Q_dev;
     a.tr_dec = dec_dev;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int rc2 = bpq::cuda_check(cudaMemsetAsync(work_dev, 0, 8, st), "workspace reset");
-    if (rc2) return rc2;
     return bpq::decode_launch(t, a, variant, true, st, nullptr);
 }
 

@@ -2,6 +2,8 @@
 // is in decode_kernel.cuh, instantiated per variant in decode_<variant>.cu).
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "bpq_internal.h"
 #include "decode_launch.h"
 
@@ -95,10 +97,11 @@ int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     return BPQ_OK;
 }
 
-int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
+namespace {
+// Shape of the one-shot-per-thread kernels with T threads per shot and gpc
+// shot groups per CTA (0: about 256 threads per CTA).
+int one_shot_shape(const bpq_tanner *t, int variant, int T, int gpc, LaunchShape *s) {
     const int nodes = t->N > t->M ? t->N : t->M;
-    int T = t->threads_per_shot;
-    if (T <= 0) T = (((nodes + 1) / 2 + 31) / 32) * 32;  // two nodes per thread
     if (T % 32 || T < 32 || T > kMaxThreadsPerShot)
         return fail(BPQ_EINVAL, "threads per shot must be a multiple of 32 in [32, 1024]");
     const int npt = (nodes + T - 1) / T;
@@ -108,7 +111,6 @@ int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     // the 15 named barriers
     const int max_groups = T == 32 ? kMaxGroupsPerCta : 15;
     const int max_threads = npt <= 2 ? 1024 : 512;
-    int gpc = t->shots_per_cta;
     if (gpc <= 0) gpc = 256 / T > 0 ? 256 / T : 1;  // about 256 threads per CTA
     if (gpc > max_groups) gpc = max_groups;
     while (gpc > 1 && gpc * T > max_threads) --gpc;
@@ -124,6 +126,13 @@ int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     s->smem = kSmemHeader + t->table.size() + (size_t)12 * s->n_pad + (size_t)gpc * s->group_bytes;
     if (s->smem > 227 * 1024) return fail(BPQ_EINVAL, "shared memory of the launch shape exceeds 227 KB");
     return BPQ_OK;
+}
+}  // namespace
+
+int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
+    const int nodes = t->N > t->M ? t->N : t->M;
+    const int T = t->threads_per_shot > 0 ? t->threads_per_shot : (((nodes + 1) / 2 + 31) / 32) * 32;
+    return one_shot_shape(t, variant, T, t->shots_per_cta, s);  // automatic: two nodes per thread
 }
 
 namespace {
@@ -172,7 +181,54 @@ int decode_batch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     return BPQ_OK;
 }
 
+namespace {
+
+// Launch of a small batch (decode_small.cu): one CTA per shot, `lanes` lanes
+// per node, every shot resident at once.  Returns false if the batch, the code
+// or the handle's launch preferences call for the queue kernels.
+//
+// Measured (kernel and launch, EWAInit or Momentum, us), against one node per
+// thread in the queue kernel: planar d = 9, 150 shots: 4 lanes 66, queue 92;
+// 300 shots: 4 lanes 107, 2 lanes 80, 1 lane 79, queue 91; 600: 2 lanes 103,
+// 1 lane 92, queue 94; toric d = 15, 150 shots: 2 lanes 102, 1 lane 86, queue
+// 95.  More lanes shorten a shot's chain but add instructions (every lane of a
+// node computes its posterior), so they pay while an SM holds at most about
+// 640 threads of them; one lane per node pays (no queue reset, no table
+// staging) while every shot has a CTA of its own.
+bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t st, int *rc) {
+    if (a.split == 0 || t->debug_checks || t->threads_per_shot || t->shots_per_cta || t->shots_per_thread) return false;
+    const int nodes = t->N > t->M ? t->N : t->M;
+    const long shots_per_sm = ((long)a.B + t->num_sms - 1) / t->num_sms;
+    if (nodes > 1024 || shots_per_sm > 32) return false;
+    int lanes = 4;
+    while (lanes > 1 && lanes * nodes * shots_per_sm > 640) lanes /= 2;
+    const int threads = (lanes * nodes + 31) / 32 * 32;
+    const size_t smem = 16 * (size_t)((t->N + 3) & ~3);
+    SmallKernelFn fn = pick_small(variant, lanes);
+    int per_sm = 0;
+    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess ||
+        shots_per_sm > per_sm)
+        return false;
+    a.n_pad = (t->N + 3) & ~3;
+    const bool unclipped = a.split == 2 && variant != BPQ_ADAGRAD;
+    fn<<<(unsigned)a.B, threads, smem, st>>>(a, variant == BPQ_AEWA ? 11 : 1, unclipped ? INFINITY : a.clip2);
+    *rc = cuda_check(cudaGetLastError(), "decode launch");
+    return true;
+}
+
+// One node per thread instead of the automatic two for batches of fewer than
+// this many shots per resident two-node group: they are bound by their slowest
+// shots, whose iterations are shorter then (kernel and launch, ms, two nodes
+// against one: planar d = 9 Momentum 1000 shots 0.139 / 0.112, 5000 (3.3 per
+// group) 0.209 / 0.183; toric d = 15 1000 (1.6 per group) 0.175 / 0.158, 5000
+// (8.2 per group) 0.407 / 0.447).
+constexpr long kOneNodeShotsPerGroup = 3;
+
+}  // namespace
+
 int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out) {
+    int small_rc = BPQ_OK;
+    if (!trace && launch_small(t, a, variant, st, &small_rc)) return small_rc;
     LaunchShape s;
     bool pairs = decode_uses_pairs(t, variant, trace);
     if (pairs && t->shots_per_thread == 0) {
@@ -210,10 +266,22 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant (AEWA-BP has no trace mode)");
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
-    const int threads = s.T * s.groups_per_cta;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, s.smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
+    const int nodes = t->N > t->M ? t->N : t->M;
+    if (!pairs && !trace && s.npt == 2 && !t->threads_per_shot && !t->shots_per_cta && nodes <= kMaxThreadsPerShot &&
+        (long)a.B < kOneNodeShotsPerGroup * per_sm * t->num_sms * s.groups_per_cta) {
+        rc = one_shot_shape(t, variant, (nodes + 31) / 32 * 32, 0, &s);
+        if (rc) return rc;
+        fn = t->debug_checks ? pick_debug(variant, s.npt, false, false, a.split) : pick(variant, s.npt, false, a.split);
+        if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant");
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+        if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
+        if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
+    }
+    const int threads = s.T * s.groups_per_cta;
     long ctas = (long)per_sm * t->num_sms;
     const long per_cta = (long)s.groups_per_cta * (pairs ? 2 : 1);
     const long need = (a.B + per_cta - 1) / per_cta;
@@ -224,6 +292,8 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     a.slots_floats = s.slots_floats;
     a.group_bytes = s.group_bytes;
     if (ctas_out) *ctas_out = (int)ctas;
+    rc = cuda_check(cudaMemsetAsync(a.work, 0, 8, st), "workspace reset");  // the shot queue, the error word
+    if (rc) return rc;
     fn<<<(unsigned)ctas, threads, s.smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("decode launch: ") + cudaGetErrorString(e));

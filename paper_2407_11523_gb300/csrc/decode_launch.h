@@ -71,6 +71,7 @@ struct LaunchShape {
 
 using DecodeKernelFn = void (*)(const DecodeArgs);
 using BatchKernelFn = void (*)(const BatchArgs);
+using SmallKernelFn = void (*)(const DecodeArgs, int runs, float clip);
 
 // Kernels of one variant, for nodes per thread npt in [1, 4]; split selects the
 // specialisation for tables in the split layout, and the _full functions the
@@ -101,6 +102,12 @@ DecodeKernelFn pick_adagrad_pair(bool one);
 DecodeKernelFn pick_adagrad_pair_full(bool one);
 DecodeKernelFn pick_ewainit_pair(bool one);
 DecodeKernelFn pick_ewainit_pair_full(bool one);
+
+// One CTA per shot, `lanes` (1, 2 or 4) lanes per node (decode_small.cu), split
+// tables, every variant.  runs: 11 for AEWA-BP, else 1; clip: the bound of the
+// check side in bits (infinite where the kernels for tables without padding
+// have none).
+SmallKernelFn pick_small(int variant, int lanes);
 
 // Bounds-checked kernels (decode_debug.cu; bpq_set_debug_checks): npt in
 // {1, 2} with one shot per thread, pairs on split layouts (one: one shot
