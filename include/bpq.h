@@ -301,28 +301,24 @@ int bpq_autotune(bpq_tanner *t, const uint32_t *syn_dev, const float *prior_dev,
  * updates its posterior by the variant's rule and sends new v->c messages
  * (eq. (v_update); eq. (mombp5) for Momentum and AdaGrad); the hard
  * decision and syndrome test follow each full sweep.  The kernel runs the
- * sweep's dependency levels in order, all qubits of a level at once, which
- * gives the serial order's result exactly; one warp decodes one shot.
+ * sweep in steps of mutually independent qubits, each after the earlier
+ * qubits that share a check with it, which gives the serial order's result
+ * exactly; 32, 16 or 8 lanes of a warp decode one shot.
  * variant: plain, Momentum, AdaGrad or EWAInit BP (EINVAL otherwise).
  * Arguments, layouts, ownership, asynchrony and errors as bpq_decode; iters
  * counts sweeps.  EINVAL also when one shot's state does not fit in shared
- * memory (about 10^4 edges for EWAInit-BP).  A warp decodes one shot, or two
- * (bpq_set_serial_shots_per_warp) with the same per-shot results bit for
- * bit. */
+ * memory (about 10^4 edges for EWAInit-BP).  Per-shot results are the same bit
+ * for bit however many shots a warp decodes (bpq_set_serial_shots_per_warp). */
 int bpq_decode_serial(const bpq_tanner *t, const uint32_t *syn_dev, const float *prior_dev, int variant,
                       const bpq_params *params, int max_iter, int B, uint8_t *est_dev, uint8_t *conv_dev,
                       uint8_t *iters_dev, void *work_dev, void *stream);
 
 /* Shots per warp of bpq_decode_serial (an implementation choice; the paper
- * has no GPU design): 1 = each warp decodes one shot; 2 = each warp decodes
- * two, its lanes working on the same qubit of both, whose messages share
- * 64-bit shared-memory slots and packed f32x2 arithmetic (each shot stops on
- * its own and the warp takes the next one for that half); 0 = automatic (2
- * where shared memory still holds 16 two-shot warps per SM and the batch
- * holds at least 128 shots per resident one-shot warp, e.g. 622592 planar
- * d = 7 shots on a GB300; the kernel is latency-bound, so codes whose
- * two-shot warps fill shared memory sooner, such as toric d = 15, keep one
- * shot per warp).  The trace keeps one shot per warp.
+ * has no GPU design): 1 = each warp decodes one shot, two lanes to a qubit; 2 =
+ * each half warp decodes one, a lane to a qubit (each shot stops on its own and
+ * its lanes take the next one); 0 = automatic (1, 2, or four shots of 8 lanes,
+ * by the code's size, the variant's state and the batch: small codes in large
+ * batches take more).  The trace keeps one shot per warp.
  * Errors: EINVAL (a value outside 0..2); bpq_decode_serial returns EINVAL
  * for 2 when two shots of the code do not fit in shared memory. */
 int bpq_set_serial_shots_per_warp(bpq_tanner *t, int shots_per_warp);

@@ -554,8 +554,12 @@ int bpq_tanner_upload(bpq_tanner *t, int device) {
     const size_t o_log = o_ptr + al(sizeof(int32_t) * t->chk_ptr.size());
     const size_t o_tab2 = o_log + al(t->logicals.size() + 1);
     const size_t o_canon2 = o_tab2 + al(t->table_split.size());
-    const size_t o_serial = o_canon2 + al(sizeof(int32_t) * t->var_canon_split.size());
-    const size_t total = o_serial + al(t->serial.size());
+    size_t o_serial[bpq::kSerialTables];
+    size_t total = o_canon2 + al(sizeof(int32_t) * t->var_canon_split.size());
+    for (int k = 0; k < bpq::kSerialTables; ++k) {
+        o_serial[k] = total;
+        total += al(t->serial[k].data.size());
+    }
     void *blob = nullptr;
     rc = bpq::cuda_check(cudaMalloc(&blob, total), "cudaMalloc");
     if (rc) return rc;
@@ -572,8 +576,8 @@ int bpq_tanner_upload(bpq_tanner *t, int device) {
     if (e == cudaSuccess && t->split)
         e = cudaMemcpy(b + o_canon2, t->var_canon_split.data(), sizeof(int32_t) * t->var_canon_split.size(),
                        cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !t->serial.empty())
-        e = cudaMemcpy(b + o_serial, t->serial.data(), t->serial.size(), cudaMemcpyHostToDevice);
+    for (int k = 0; k < bpq::kSerialTables && e == cudaSuccess; ++k)
+        e = cudaMemcpy(b + o_serial[k], t->serial[k].data.data(), t->serial[k].data.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(blob);
         return bpq::cuda_check(e, "cudaMemcpy");
@@ -587,7 +591,7 @@ int bpq_tanner_upload(bpq_tanner *t, int device) {
     t->d_logicals = t->logicals.empty() ? nullptr : b + o_log;
     t->d_table_split = t->split ? b + o_tab2 : nullptr;
     t->d_var_canon_split = t->split ? reinterpret_cast<const int32_t *>(b + o_canon2) : nullptr;
-    t->d_serial = b + o_serial;
+    for (int k = 0; k < bpq::kSerialTables; ++k) t->d_serial[k] = b + o_serial[k];
     return BPQ_OK;
 }
 

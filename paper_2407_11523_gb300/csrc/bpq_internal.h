@@ -32,24 +32,25 @@ inline bool misaligned(const void *p, size_t align) {
     return (reinterpret_cast<uintptr_t>(p) & (align - 1)) != 0;
 }
 
-// One qubit of the serial schedule's sweep (48 bytes, 16-byte aligned); the
-// serial table lists them level by level (see serial.cu).  Message slots
-// index the kernel's per-shot message array: every edge has one slot, laid
-// out so that the lanes of one access fall in distinct shared-memory banks;
-// two extra slots follow the edges' (zero: reads as a certain message with
-// positive sign, the identity of the check rule; trash: takes writes of
-// padding edges).
-struct SerialVar {
-    uint16_t own[4];     // slot of the qubit's edge k (the trash slot for padding)
-    uint16_t oth[4][3];  // slots of the other edges of edge k's check (the zero slot for padding)
-    uint16_t chk[4];     // the check of edge k (0 for padding)
-    uint16_t j;          // the qubit
-    uint8_t pauli;       // H_ij of edge k in bits 2k, 2k+1 (0 for padding)
-    uint8_t last;        // bit k: the qubit is the last of edge k's check in the sweep
-    uint8_t real;        // bit k: edge k exists (not padding)
-    uint8_t pad[3];
+// Step table of the serial schedule (see serial_kernel.cuh): the sweep in
+// steps of at most 16 or 8 qubits.
+//   data: half uint4[2][N] | meta u32[N] | first position of each step
+//   u16[steps + 1] (these are staged in shared memory) | qubit u16[N] | checks
+//   of the four edges u16[N][4] | canonical edge indices u16[N][4], every part
+//   16-byte aligned.
+// half: for edges 0, 1 (then 2, 3) the 16-bit byte offsets of the message slots
+// of the two edges, then of the three other edges of each one's check.  Message
+// slots: `slots` for the edges, then the zero slot (for the missing edges of a
+// check: a certain message with positive sign, the identity of the check rule),
+// the slot of no information (read by padding edges, whose c->v message is then
+// 0) and the trash slot (written by padding edges).
+struct SerialTable {
+    std::vector<uint8_t> data;
+    int steps = 0, slots = 0;
+    uint32_t off_meta = 0, off_steps = 0, off_qubit = 0, off_chk = 0, off_canon = 0;
 };
-static_assert(sizeof(SerialVar) == 48, "SerialVar layout");
+constexpr int kSerialTables = 2;
+constexpr int kSerialWidth[kSerialTables] = {16, 8};
 
 }  // namespace bpq
 
@@ -80,15 +81,8 @@ struct bpq_tanner {
     bool full = false;
     std::vector<uint8_t> table_split;
     std::vector<int32_t> var_canon_split;  // 4 n4, indexed by split slot
-    // Serial schedule (bpq::build_serial_table): SerialVar[N] in level order |
-    // level_ptr u16[levels + 1] | canon u16[N][4] (check-major index of each
-    // qubit's edge k, E for padding; 16-byte aligned, read by the trace
-    // kernels only, so the kernels stage the table up to it), padded to 16
-    // bytes; serial_slots
-    // message slots for the edges, then the zero and the trash slot.
-    std::vector<uint8_t> serial;
-    int serial_levels = 0, serial_slots = 0;
-    uint32_t serial_off_levels = 0, serial_off_canon = 0;
+    // Serial schedule (bpq::build_serial_table), by step width
+    bpq::SerialTable serial[bpq::kSerialTables];
 
     // device
     int device = -1;
@@ -96,7 +90,7 @@ struct bpq_tanner {
     const uint8_t *d_table = nullptr;
     const int32_t *d_var_canon = nullptr;
     const uint8_t *d_table_split = nullptr;
-    const uint8_t *d_serial = nullptr;
+    const uint8_t *d_serial[bpq::kSerialTables] = {};
     const int32_t *d_var_canon_split = nullptr;
     const int32_t *d_chk_ptr = nullptr;
     const uint8_t *d_logicals = nullptr;
@@ -107,7 +101,7 @@ struct bpq_tanner {
     int threads_per_shot = 0, shots_per_cta = 0, shots_per_thread = 0;
     // nodes per thread inside the batched kernel and the servers (0 = automatic)
     int batch_nodes_per_thread = 0;
-    // shots per warp of the serial-schedule kernel (0 = automatic)
+    // shots per warp of the serial-schedule kernels (0 = automatic)
     int serial_shots_per_warp = 0;
     // run the bounds-checked kernels (bpq_set_debug_checks)
     bool debug_checks = false;
@@ -116,6 +110,6 @@ struct bpq_tanner {
 namespace bpq {
 // Fill t->table, offsets and var_canon from the CSR; returns BPQ_OK or an error.
 int build_tables(bpq_tanner *t);
-// Fill t->serial (called by build_tables).
+// Fill t->serial[] (called by build_tables).
 int build_serial_table(bpq_tanner *t);
 }  // namespace bpq

@@ -1,36 +1,95 @@
 // Host side of the serial-schedule decoders (serial_kernel.cuh) and the
-// one-shot-per-warp kernels; the two-shots-per-warp kernels are instantiated
-// in serial_pair.cu.
+// kernels with a whole warp per shot; narrower groups are instantiated in
+// serial16.cu and serial8.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
-#include <new>
-#include <vector>
 
 #include "serial_kernel.cuh"
 
 namespace bpq {
 namespace sk {
 
-SerialKernelFn pick_serial(int variant, bool trace, bool split) {
-#define BPQ_SERIAL_CASE(V)                                                                   \
-    case V:                                                                                  \
-        return trace ? (split ? serial_kernel<V, true, true> : serial_kernel<V, true, false>) \
-                     : (split ? serial_kernel<V, false, true> : serial_kernel<V, false, false>);
-    switch (variant) {
-        BPQ_SERIAL_CASE(BPQ_PLAIN)
-        BPQ_SERIAL_CASE(BPQ_MOMENTUM)
-        BPQ_SERIAL_CASE(BPQ_ADAGRAD)
-        BPQ_SERIAL_CASE(BPQ_EWAINIT)
-    }
-#undef BPQ_SERIAL_CASE
-    return nullptr;
+namespace {
+SerialKernelFn pick_trace(int variant, bool split) { BPQ_SERIAL_SWITCH(true, 32, 2) }
+SerialKernelFn pick_decode(int variant, bool split) { BPQ_SERIAL_SWITCH(false, 32, 2) }
+}  // namespace
+
+SerialKernelFn pick_serial32(int variant, bool trace, bool split) {
+    return trace ? pick_trace(variant, split) : pick_decode(variant, split);
 }
 
 }  // namespace sk
 
 namespace {
+
+// The ways to decode: lanes per shot, and the step table they use (32 lanes
+// take two per qubit, hence the 16-qubit steps).
+enum SerialMode { kSerial32 = 0, kSerial16 = 1, kSerial8 = 2 };
+constexpr int kModeLanes[3] = {32, 16, 8}, kModeTable[3] = {0, 0, 1};
+
+// Shared memory of a launch.
+struct SerialShape {
+    int lanes, warps;        // warps: that fit (0: not even one)
+    size_t fixed, shot_bytes;
+    uint32_t off_state, off_syn, off_qb, off_dec, shot_words;
+    size_t smem(int n) const { return fixed + (size_t)n * (32 / lanes) * shot_bytes; }
+};
+
+SerialShape serial_shape(const bpq_tanner *t, int variant, int mode) {
+    const SerialTable &s = t->serial[kModeTable[mode]];
+    const uint32_t n_pad = (uint32_t)((t->N + 3) & ~3);
+    SerialShape r;
+    r.lanes = kModeLanes[mode];
+    r.fixed = 128 + s.off_qubit + (size_t)(12 + (t->split ? 8 : 12)) * n_pad;
+    // messages (and three constant slots) | state | syndrome words | qubit bytes
+    r.off_state = ((uint32_t)s.slots + 3u + 3u) & ~3u;
+    r.off_syn = r.off_state + (uint32_t)sk::serial_state_arrays(variant) * n_pad;
+    r.off_qb = r.off_syn + (uint32_t)(((t->M + 31) / 32 + 3) & ~3);
+    r.off_dec = r.off_qb + n_pad / 4;
+    r.shot_words = r.off_dec + (sk::serial_state_arrays(variant) ? 0u : n_pad / 4);
+    // the shots of a warp: `lanes` banks apart
+    if (r.lanes < 32) r.shot_words += (uint32_t)(r.lanes - (int)(r.shot_words % 32) + 32) % 32;
+    r.shot_bytes = 4 * (size_t)r.shot_words;
+    const size_t limit = 227 * 1024, warp_bytes = (32 / r.lanes) * r.shot_bytes;
+    r.warps = r.fixed + warp_bytes > limit
+                  ? 0 : (int)std::min<size_t>(sk::serial_max_warps(r.lanes), (limit - r.fixed) / warp_bytes);
+    return r;
+}
+
+// The mode of a batch: the least of an estimate of its time, for ten sweeps a
+// shot and a slowest shot that runs max_iter, from figures measured on GB300: a
+// step costs a warp about 190 issue slots with two lanes per qubit and 290
+// with one (shared by the warp's shots), and 480 or 660 cycles when the warp has
+// its scheduler to itself; a scheduler issues 0.28 slots a cycle per resident
+// warp, 0.85 at most.  So narrow groups are for small codes, whose shots fit
+// shared memory many times, in large batches.  Measured, 32 / 16 / 8 lanes per
+// shot (ms, EWAInit): planar d = 7, 10^6 shots 7.30 / 6.02 / 4.33, 10^5 1.11 /
+// 1.10 / 1.04, 20000 0.51 / 0.58 / 0.65; planar d = 11, 10^5 3.19 / 2.86 / 2.89;
+// toric d = 10, 10^5 1.78 / 1.75 / 1.96; toric d = 15, 10^6 24.0 / 25.1 / 45.5;
+// planar d = 25, 20000 5.8 / 7.1 / 14.5.  (A warp per shot on the dependency
+// levels, one lane per qubit, took 10.2, 1.68, 0.76, 4.77, 2.64, 30.1, 6.57.)
+int serial_mode(const bpq_tanner *t, int variant, int max_iter, int B) {
+    if (t->serial_shots_per_warp) return t->serial_shots_per_warp == 1 ? kSerial32 : kSerial16;
+    int best = kSerial32;
+    double least = 0;
+    for (int mode = kSerial32; mode <= kSerial8; ++mode) {
+        const SerialShape s = serial_shape(t, variant, mode);
+        if (s.warps < 1) continue;
+        const double steps = t->serial[kModeTable[mode]].steps, per_warp = 32 / s.lanes;
+        const double busy = std::min<double>(s.warps, std::ceil(B / (per_warp * t->num_sms)));
+        const double slots = steps * (mode == kSerial32 ? 190 : 290 / per_warp);
+        const double cycles = 10.0 * B * slots / (std::min(0.85, 0.07 * busy) * 4 * t->num_sms) +
+                              max_iter * steps * (mode == kSerial32 ? 480 : 660);
+        if (mode == kSerial32 || cycles < least) {
+            best = mode;
+            least = cycles;
+        }
+    }
+    return best;
+}
 
 // Validate, fill the arguments from the parallel decoder's (parameters in
 // the kernel's units) and launch.
@@ -46,13 +105,22 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     if (rc) return rc;
     if (B == 0) return BPQ_OK;
     if (!trace && (!est || !conv || !iters)) return fail(BPQ_EINVAL, "NULL output");
+    const int mode = trace ? kSerial32 : serial_mode(t, variant, max_iter, B);
+    const SerialTable &s = t->serial[kModeTable[mode]];
+    const SerialShape shape = serial_shape(t, variant, mode);
+    if (shape.warps < 1)
+        return fail(BPQ_EINVAL, mode == kSerial32 ? "code too large for the serial kernel's shared memory"
+                                           : "two shots per warp do not fit in shared memory for this code");
     SerialArgs a;
     std::memset(&a, 0, sizeof a);
-    a.table = t->d_serial;
-    a.table_bytes = t->serial_off_canon;
-    a.off_levels = t->serial_off_levels;
-    a.off_canon = t->serial_off_canon;
-    a.nlevels = t->serial_levels;
+    a.table = t->d_serial[kModeTable[mode]];
+    a.table_bytes = s.off_qubit;
+    a.off_meta = s.off_meta;
+    a.off_steps = s.off_steps;
+    a.off_qubit = s.off_qubit;
+    a.off_chk = s.off_chk;
+    a.off_canon = s.off_canon;
+    a.nsteps = s.steps;
     a.syn = syn;
     a.prior = prior;
     a.est = est;
@@ -70,18 +138,12 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     a.B = B;
     a.max_iter = max_iter;
     a.n_pad = (t->N + 3) & ~3;
-    a.zero_slot = (uint32_t)t->serial_slots;
-    a.msg_floats = (a.zero_slot + 2u + 3u) & ~3u;
-    // one shot per warp: messages | state | syndrome words | qubit bytes;
-    // two: the same with float2 slots, two syndromes and two bytes per qubit
-    const uint32_t state_floats = (uint32_t)(sk::serial_state_arrays(variant) * a.n_pad);
-    const uint32_t W4 = (uint32_t)((a.W + 3) & ~3);
-    auto layout = [&](uint32_t k) {
-        a.off_syn = 4u * k * (a.msg_floats + state_floats);
-        a.syn_stride = W4;
-        a.off_qb = a.off_syn + 4u * k * W4;
-        a.warp_bytes = (a.off_qb + k * (uint32_t)a.n_pad + 15u) & ~15u;
-    };
+    a.zero_slot = (uint32_t)s.slots;
+    a.shot_words = shape.shot_words;
+    a.off_state = shape.off_state;
+    a.off_syn = shape.off_syn;
+    a.off_qb = shape.off_qb;
+    a.off_dec = shape.off_dec;
     a.alpha = d.alpha;
     a.gamma = d.gamma;
     a.eps = d.eps;
@@ -91,33 +153,13 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     a.phi_clip = d.phi_clip;
     a.ada_from1 = d.ada_from1;
 
-    const size_t fixed = 128 + a.table_bytes + (size_t)12 * a.n_pad;
-    const size_t limit = 227 * 1024;
-    layout(1);
-    if (fixed + a.warp_bytes > limit) return fail(BPQ_EINVAL, "code too large for the serial kernel's shared memory");
-    const long warps1 = (long)std::min<size_t>(32, (limit - fixed) / a.warp_bytes);
-    // two shots per warp (not for traces): on request, or automatically where
-    // shared memory still holds kSerialPairWarps two-shot warps per SM and the
-    // batch gives every resident one-shot warp kSerialPairShots shots.  The
-    // kernel is latency-bound: with fewer warps the two-shot kernel's shorter
-    // instruction stream per shot does not make up for the lost warps (toric
-    // d = 15 on GB300: 7 two-shot warps, 2.26e7 against 2.53e7 shots/s at
-    // 1e5 shots, 3.2e7 against 3.3e7 at 1e6), and small batches, whose time
-    // is set by their slowest shots, finish sooner with one shot per warp.
-    bool pairs = false;
-    if (!trace) {
-        layout(2);
-        const bool fits = fixed + a.warp_bytes <= limit;
-        const int k = t->serial_shots_per_warp;
-        if (k == 2 && !fits) return fail(BPQ_EINVAL, "two shots per warp do not fit in shared memory for this code");
-        const bool full_occupancy = fits && (limit - fixed) / a.warp_bytes >= (size_t)sk::kSerialPairWarps;
-        pairs = fits && (k == 2 || (k == 0 && full_occupancy && (long)B >= kSerialPairShots * warps1 * t->num_sms));
-        if (!pairs) layout(1);
-    }
-    int warps = (int)std::min<size_t>(pairs ? sk::kSerialPairWarps : 32, (limit - fixed) / a.warp_bytes);
-    const size_t smem = fixed + (size_t)warps * a.warp_bytes;
-    sk::SerialKernelFn fn = pairs ? sk::pick_serial_pair(variant, t->full ? 2 : t->split ? 1 : 0)
-                                  : sk::pick_serial(variant, trace, t->split);
+    // small batches: spread over the SMs instead of filling the first ones
+    const long per_warp = 32 / shape.lanes, wave = per_warp * t->num_sms;
+    const int warps = (int)std::min<long>(shape.warps, (B + wave - 1) / wave);
+    const size_t smem = shape.smem(warps);
+    sk::SerialKernelFn fn = mode == kSerial32   ? sk::pick_serial32(variant, trace, t->split)
+                            : mode == kSerial16 ? sk::pick_serial16(variant, t->split)
+                                                : sk::pick_serial8(variant, t->split);
     if (!fn) return fail(BPQ_EINVAL, "no serial kernel for this variant");
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
@@ -125,7 +167,7 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "serial kernel does not fit on an SM");
     long ctas = (long)per_sm * t->num_sms;
-    const long per_cta = (long)warps * (pairs ? 2 : 1);
+    const long per_cta = warps * per_warp;
     const long need = (B + per_cta - 1) / per_cta;
     if (ctas > need) ctas = need;
     rc = cuda_check(cudaMemsetAsync(work, 0, 8, st), "workspace reset");

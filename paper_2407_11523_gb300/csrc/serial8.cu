@@ -1,0 +1,9 @@
+// Serial-schedule kernels with 8 lanes per shot (serial_kernel.cuh), in a
+// translation unit of their own so that they compile in parallel with the others.
+#include "serial_kernel.cuh"
+
+namespace bpq {
+namespace sk {
+SerialKernelFn pick_serial8(int variant, bool split) { BPQ_SERIAL_SWITCH(false, 8, 1) }
+}  // namespace sk
+}  // namespace bpq

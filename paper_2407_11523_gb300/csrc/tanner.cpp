@@ -16,6 +16,8 @@
 #include <array>
 #include <cstring>
 #include <new>
+#include <queue>
+#include <vector>
 
 #include "bpq_internal.h"
 
@@ -155,168 +157,169 @@ int build_tables(bpq_tanner *t) {
 }
 
 namespace {
-// Message slots of the serial kernels' edges: slot = bank + 32 * row, with
-// bank chosen greedily so that the edges one warp instruction touches (the
-// k-th edge, or its check's r-th other edge, of the qubits of one 32-lane
-// step of a level) fall in distinct banks where possible: distinct slots
-// mod 32 across the warp (32-bit accesses of the one-shot kernel) and
-// distinct slots mod 16 within each half-warp (the 64-bit slot accesses of
-// the two-shot kernel are served half a warp at a time).  Edges are
-// coloured in sweep order; each bank holds at most ceil(E / 32) + 1 edges.
-std::vector<int> colour_serial_slots(const std::vector<std::array<int, 4>> &at, const std::vector<int> &edge_chk,
-                                     const std::vector<int32_t> &chk_ptr, const std::vector<int> &order,
-                                     const std::vector<int> &lp, int E, int *nslots) {
-    const int nlev = (int)lp.size() - 1;
-    struct Use {
-        int edge, lane;
-    };
-    std::vector<std::vector<Use>> groups;
-    for (int l = 0; l < nlev; ++l)
-        for (int s0 = lp[l]; s0 < lp[l + 1]; s0 += 32) {
-            const int s1 = std::min(lp[l + 1], s0 + 32);
-            for (int k = 0; k < 4; ++k)
-                for (int r = 0; r < 4; ++r) {
-                    std::vector<Use> g;
-                    for (int v = s0; v < s1; ++v) {
-                        const int e = at[order[v]][k];
-                        if (e < 0) continue;
-                        const int i = edge_chk[e];
-                        if (r == 3) {
-                            g.push_back({e, v - s0});
-                            continue;
-                        }
-                        int f = 0;
-                        for (int x = chk_ptr[i]; x < chk_ptr[i + 1]; ++x)
-                            if (x != e && f++ == r) g.push_back({x, v - s0});
-                    }
-                    if (!g.empty()) groups.push_back(std::move(g));
-                }
+
+// The sweep in steps of at most `lanes` qubits, each after every earlier qubit
+// that shares a check with it: list scheduling, among the qubits whose
+// predecessors are done those with the longest chain of successors first (then
+// the lower index).  order: the qubits step by step; first: the first position
+// of each step, and N.
+void schedule_sweep(const std::vector<std::vector<int>> &later, int lanes, std::vector<int> &order,
+                    std::vector<int> &first) {
+    const int N = (int)later.size();
+    std::vector<int> waits(N, 0), chain(N, 1);
+    for (int j = N - 1; j >= 0; --j)
+        for (int k : later[j]) {
+            ++waits[k];
+            chain[j] = std::max(chain[j], chain[k] + 1);
         }
-    struct Member {
-        int group, lane;
+    auto before = [&](int x, int y) { return chain[x] != chain[y] ? chain[x] < chain[y] : x > y; };
+    std::priority_queue<int, std::vector<int>, decltype(before)> ready(before);
+    for (int j = 0; j < N; ++j)
+        if (!waits[j]) ready.push(j);
+    order.clear();
+    first.assign(1, 0);
+    while (!ready.empty()) {
+        const size_t begin = order.size();
+        while ((int)(order.size() - begin) < lanes && !ready.empty()) {
+            order.push_back(ready.top());
+            ready.pop();
+        }
+        for (size_t v = begin; v < order.size(); ++v)
+            for (int k : later[order[v]])
+                if (--waits[k] == 0) ready.push(k);
+        first.push_back((int)order.size());
+    }
+}
+
+// Message slots of the edges: slot = bank + 32 * row, with bank chosen
+// greedily so that the edges one access touches (the k-th edge, or its check's
+// r-th other edge, of the qubits of one step) fall in distinct banks modulo
+// `width` where possible (the shots of a warp are that many banks apart), and,
+// with 16 qubits a step, those of edges k and k + 2 together in distinct banks
+// (two lanes per qubit).  Edges are taken in sweep order; each bank holds at most
+// ceil(E / 32) + 1 edges.  touch[16 j + 4 k + r]: the edge that qubit j's access
+// (k, r) touches, r = 3 its own, -1 for none.
+std::vector<int> colour_serial_slots(const std::vector<int> &touch, const std::vector<int> &order,
+                                     const std::vector<int> &first, int width, int E, int *nslots) {
+    struct Use {
+        int step, access;
     };
-    std::vector<std::vector<Member>> edge_groups(E);  // the groups of an edge, with its lane in each
-    for (int gi = 0; gi < (int)groups.size(); ++gi)
-        for (const Use &u : groups[gi]) edge_groups[u.edge].push_back({gi, u.lane});
+    std::vector<int> ptr(E + 1, 0), at;  // the uses of each edge, flat
+    for (size_t x = 0; x < touch.size(); ++x)
+        if (touch[x] >= 0) ++ptr[touch[x] + 1];
+    for (int e = 0; e < E; ++e) ptr[e + 1] += ptr[e];
+    std::vector<Use> uses(ptr[E]);
+    at.assign(ptr.begin(), ptr.end() - 1);
+    const int steps = (int)first.size() - 1;
+    for (int s = 0; s < steps; ++s)
+        for (int v = first[s]; v < first[s + 1]; ++v)
+            for (int x = 0; x < 16; ++x) {
+                const int e = touch[16 * (size_t)order[v] + x];
+                if (e >= 0) uses[at[e]++] = {s, x};
+            }
+    // edges already in a bank: of one access, modulo the width; of the accesses
+    // (k, r) and (k + 2, r), modulo 32
+    std::vector<uint8_t> one((size_t)16 * steps * width, 0), two((size_t)8 * steps * 32, 0);
     const int cap = (E + 31) / 32 + 1;
-    std::vector<int> bank(E, -1), fill(32, 0), slot(E);
+    std::vector<int> fill(32, 0), slot(E, 0);
     for (int v = 0; v < (int)order.size(); ++v)
-        for (int e : at[order[v]]) {
+        for (int k = 0; k < 4; ++k) {
+            const int e = touch[16 * (size_t)order[v] + 4 * k + 3];
             if (e < 0) continue;
             int cost[32] = {0};
-            for (const Member &eg : edge_groups[e])
-                for (const Use &u : groups[eg.group]) {
-                    const int b = bank[u.edge];
-                    if (b < 0) continue;
-                    ++cost[b];
-                    if ((u.lane < 16) == (eg.lane < 16)) {
-                        ++cost[b & 15];
-                        ++cost[(b & 15) + 16];
-                    }
-                }
+            for (int u = ptr[e]; u < ptr[e + 1]; ++u) {
+                const uint8_t *r1 = &one[((size_t)16 * uses[u].step + uses[u].access) * width];
+                const uint8_t *r2 = &two[((size_t)8 * uses[u].step + (uses[u].access & 7)) * 32];
+                for (int b = 0; b < 32; ++b) cost[b] += 2 * r1[b % width] + (width == 16 ? r2[b] : 0);
+            }
             int best = -1;
             for (int b = 0; b < 32; ++b)
                 if (fill[b] < cap && (best < 0 || cost[b] < cost[best] || (cost[b] == cost[best] && fill[b] < fill[best])))
                     best = b;
-            bank[e] = best;
+            for (int u = ptr[e]; u < ptr[e + 1]; ++u) {
+                ++one[((size_t)16 * uses[u].step + uses[u].access) * width + best % width];
+                ++two[((size_t)8 * uses[u].step + (uses[u].access & 7)) * 32 + best];
+            }
             slot[e] = best + 32 * fill[best]++;
         }
-    int top = 0;
-    for (int b = 0; b < 32; ++b) top = std::max(top, fill[b]);
-    *nslots = 32 * top;
+    // the last slot in use, not the last full row
+    *nslots = E ? *std::max_element(slot.begin(), slot.end()) + 1 : 0;
     return slot;
 }
 }  // namespace
 
 int build_serial_table(bpq_tanner *t) {
     const int N = t->N, M = t->M, E = t->E;
-    // level(j) = 1 + the largest level among the earlier qubits sharing a check with j
-    std::vector<std::vector<int>> var_edges(N);
-    std::vector<int> edge_chk(E);
+    std::vector<std::vector<int>> var_edges(N), later(N);
+    std::vector<int> edge_chk(E), chk_lastq(M, -1);
     for (int i = 0; i < M; ++i)
         for (int e = t->chk_ptr[i]; e < t->chk_ptr[i + 1]; ++e) {
             var_edges[t->chk_var[e]].push_back(e);
             edge_chk[e] = i;
+            chk_lastq[i] = std::max(chk_lastq[i], t->chk_var[e]);
+            for (int f = e + 1; f < t->chk_ptr[i + 1]; ++f) later[t->chk_var[e]].push_back(t->chk_var[f]);
         }
-    std::vector<int> level(N), chk_last(M, -1), chk_lastq(M, -1);
-    int nlevels = 0;
-    for (int j = 0; j < N; ++j) {
-        int l = 0;
-        for (int e : var_edges[j]) l = std::max(l, chk_last[edge_chk[e]] + 1);
-        level[j] = l;
-        for (int e : var_edges[j]) {
-            chk_last[edge_chk[e]] = l;
-            chk_lastq[edge_chk[e]] = j;  // qubits in index order: the last one stays
-        }
-        nlevels = std::max(nlevels, l + 1);
-    }
-    std::vector<int> order(N);
-    for (int j = 0; j < N; ++j) order[j] = j;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return level[x] < level[y]; });
-    std::vector<int> lp(nlevels + 1);
-    for (int l = 0, v = 0; l <= nlevels; ++l) {
-        while (v < N && level[order[v]] < l) ++v;
-        lp[l] = v;
-    }
     // edge at each of a qubit's four positions (-1: padding): in increasing
     // check order, or (split layout) the X edges at 0, 1 and the Z edges at
-    // 2, 3
-    std::vector<std::array<int, 4>> at(N);
+    // 2, 3; and the other edges of each one's check
+    std::vector<int> touch((size_t)16 * N, -1);
     for (int j = 0; j < N; ++j) {
-        at[j] = {-1, -1, -1, -1};
         int nx = 0, nz = 0;
         for (int q = 0; q < (int)var_edges[j].size(); ++q) {
-            const int e = var_edges[j][q];
-            at[j][!t->split ? q : t->chk_pauli[e] == 1 ? nx++ : 2 + nz++] = e;
+            const int e = var_edges[j][q], i = edge_chk[e];
+            const int k = !t->split ? q : t->chk_pauli[e] == 1 ? nx++ : 2 + nz++;
+            int *x = &touch[16 * (size_t)j + 4 * k], r = 0;
+            x[3] = e;
+            for (int f = t->chk_ptr[i]; f < t->chk_ptr[i + 1]; ++f)
+                if (f != e) x[r++] = f;
         }
     }
-    int nslots = 0;
-    const std::vector<int> slot = colour_serial_slots(at, edge_chk, t->chk_ptr, order, lp, E, &nslots);
-    if (nslots + 2 > 0xFFFF || M >= 0xFFFF || E >= 0xFFFF || N > 0xFFFF)
-        return fail(BPQ_EINVAL, "code too large for the serial table");
-    const uint16_t kZero = (uint16_t)nslots, kTrash = (uint16_t)(nslots + 1);
-
-    const size_t vars_bytes = sizeof(SerialVar) * (size_t)N;
-    const size_t off_levels = vars_bytes;
-    const size_t off_canon = (off_levels + 2 * (size_t)(nlevels + 1) + 15) & ~size_t(15);
-    const size_t bytes = (off_canon + 8 * (size_t)N + 15) & ~size_t(15);
-    t->serial.assign(bytes, 0);
-    SerialVar *vars = reinterpret_cast<SerialVar *>(t->serial.data());
-    uint16_t *lpt = reinterpret_cast<uint16_t *>(t->serial.data() + off_levels);
-    uint16_t *canon = reinterpret_cast<uint16_t *>(t->serial.data() + off_canon);
-    for (int v = 0; v < N; ++v) {
-        const int j = order[v];
-        SerialVar &sv = vars[v];
-        sv.j = (uint16_t)j;
-        sv.pauli = 0;
-        sv.last = 0;
-        sv.real = 0;
-        for (int k = 0; k < 4; ++k) {
-            sv.own[k] = kTrash;
-            sv.chk[k] = 0;
-            canon[4 * v + k] = (uint16_t)E;
-            for (int f = 0; f < 3; ++f) sv.oth[k][f] = kZero;
+    auto al = [](size_t x) { return (x + 15) & ~size_t(15); };
+    for (int w = 0; w < kSerialTables; ++w) {
+        SerialTable &s = t->serial[w];
+        std::vector<int> order, first;
+        schedule_sweep(later, kSerialWidth[w], order, first);
+        s.steps = (int)first.size() - 1;
+        const std::vector<int> slot = colour_serial_slots(touch, order, first, kSerialWidth[w], E, &s.slots);
+        if (4 * (s.slots + 3) > 0x10000 || M >= 0xFFFF || E >= 0xFFFF || N > 0xFFFF)
+            return fail(BPQ_EINVAL, "code too large for the serial table");
+        const uint16_t zero = (uint16_t)(4 * s.slots), none = (uint16_t)(4 * (s.slots + 1)),
+                       trash = (uint16_t)(4 * (s.slots + 2));
+        s.off_meta = (uint32_t)(32 * (size_t)N);
+        s.off_steps = (uint32_t)al(s.off_meta + 4 * (size_t)N);
+        s.off_qubit = (uint32_t)al(s.off_steps + 2 * first.size());
+        s.off_chk = (uint32_t)al(s.off_qubit + 2 * (size_t)N);
+        s.off_canon = (uint32_t)al(s.off_chk + 8 * (size_t)N);
+        s.data.assign(al(s.off_canon + 8 * (size_t)N), 0);
+        uint8_t *d = s.data.data();
+        for (int v = 0; v < N; ++v) {
+            const int j = order[v];
+            uint16_t rec[16], chk[4] = {0, 0, 0, 0}, canon[4];
+            uint32_t meta = 0;
+            for (int k = 0; k < 4; ++k) {
+                const int *x = &touch[16 * (size_t)j + 4 * k], e = x[3];
+                uint16_t *half = rec + 8 * (k / 2);
+                half[k % 2] = e < 0 ? trash : (uint16_t)(4 * slot[e]);
+                for (int r = 0; r < 3; ++r) half[2 + 3 * (k % 2) + r] = e < 0 ? none : x[r] < 0 ? zero : (uint16_t)(4 * slot[x[r]]);
+                canon[k] = (uint16_t)(e < 0 ? E : e);
+                if (e < 0) continue;
+                chk[k] = (uint16_t)edge_chk[e];
+                meta |= (uint32_t)t->chk_pauli[e] << (2 * k) | 1u << (12 + k);
+                if (chk_lastq[edge_chk[e]] == j) meta |= 1u << (8 + k);
+            }
+            const uint16_t q = (uint16_t)j;
+            std::memcpy(d + 16 * (size_t)v, rec, 16);
+            std::memcpy(d + 16 * ((size_t)N + v), rec + 8, 16);
+            std::memcpy(d + s.off_meta + 4 * (size_t)v, &meta, 4);
+            std::memcpy(d + s.off_qubit + 2 * (size_t)v, &q, 2);
+            std::memcpy(d + s.off_chk + 8 * (size_t)v, chk, 8);
+            std::memcpy(d + s.off_canon + 8 * (size_t)v, canon, 8);
         }
-        for (int k = 0; k < 4; ++k) {
-            const int e = at[j][k];
-            if (e < 0) continue;
-            const int i = edge_chk[e];
-            sv.real |= (uint8_t)(1u << k);
-            sv.own[k] = (uint16_t)slot[e];
-            sv.chk[k] = (uint16_t)i;
-            canon[4 * v + k] = (uint16_t)e;
-            sv.pauli |= (uint8_t)(t->chk_pauli[e] << (2 * k));
-            if (chk_lastq[i] == j) sv.last |= (uint8_t)(1u << k);
-            int f = 0;
-            for (int x = t->chk_ptr[i]; x < t->chk_ptr[i + 1]; ++x)
-                if (x != e) sv.oth[k][f++] = (uint16_t)slot[x];
+        for (size_t l = 0; l < first.size(); ++l) {
+            const uint16_t f = (uint16_t)first[l];
+            std::memcpy(d + s.off_steps + 2 * l, &f, 2);
         }
     }
-    for (int l = 0; l <= nlevels; ++l) lpt[l] = (uint16_t)lp[l];
-    t->serial_levels = nlevels;
-    t->serial_slots = nslots;
-    t->serial_off_levels = (uint32_t)off_levels;
-    t->serial_off_canon = (uint32_t)off_canon;
     return BPQ_OK;
 }
 
