@@ -114,15 +114,20 @@ struct Adj {
     uint32_t vp;      // qubit Paulis, 2 bits per slot 4 x + k (0: unused)
     int ce;           // canonical index of the check's first edge
     float sigma;      // (-1)^{s_i}
+    float ws[4];      // w_e (-1)^{s_i} of the owned check's edges
+    uint32_t logp;    // Pauli of logical operator l on the qubit in bits 2l, 2l + 1 (coset loss)
 };
 
 __device__ __forceinline__ Adj load_adj(const TrainArgs &a, int x, int shot) {
     Adj d;
-    d.vp = 0;
+    d.vp = d.logp = 0;
     d.ce = 0;
     d.sigma = 1.f;
 #pragma unroll
-    for (int n = 0; n < 4; ++n) d.sl[n] = kNoSlot;
+    for (int n = 0; n < 4; ++n) {
+        d.sl[n] = kNoSlot;
+        d.ws[n] = 0.f;
+    }
     if (x < a.M) {
         const uint2 s = reinterpret_cast<const uint2 *>(a.table)[x];
         d.sl[0] = s.x & 0xFFFFu;
@@ -131,8 +136,14 @@ __device__ __forceinline__ Adj load_adj(const TrainArgs &a, int x, int shot) {
         d.sl[3] = s.y >> 16;
         d.ce = a.chk_ptr[x];
         if ((a.syn[(size_t)shot * a.W + (x >> 5)] >> (x & 31)) & 1u) d.sigma = -1.f;
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+            if (d.sl[n] != kNoSlot) d.ws[n] = a.w[d.ce + n] * d.sigma;
     }
-    if (x < a.N) d.vp = a.table[a.off_var_pauli + x];
+    if (x < a.N) {
+        d.vp = a.table[a.off_var_pauli + x];
+        for (int l = 0; l < a.n_log; ++l) d.logp |= (a.logicals[(size_t)l * a.N + x] & 3u) << (2 * l);
+    }
     return d;
 }
 
@@ -149,8 +160,10 @@ __device__ __forceinline__ void prior_llr(const TrainArgs &a, int x, float (&P)[
 
 // a [+] b = (1 + a)(1 + b) - 1.
 __device__ __forceinline__ float boxsum(float a, float b) { return __fmaf_rn(a, b, __fadd_rn(a, b)); }
+// Divisions by denominators below 2^126 (which all are here): __fdividef is
+// within 2 ulp and a fifth of the instructions of the rounded one.
 // h(y) = y (y + 2) / (y + 1).
-__device__ __forceinline__ float hfun(float y) { return __fmul_rn(y, __fadd_rn(1.f, __fdiv_rn(1.f, __fadd_rn(y, 1.f)))); }
+__device__ __forceinline__ float hfun(float y) { return __fmul_rn(y, __fadd_rn(1.f, __fdividef(1.f, __fadd_rn(y, 1.f)))); }
 
 // Check node of the owned check from m_v->c in v: q_f of each edge, E_n, the
 // signs (bit n: m_n < 0), r_n = 2 atanh prod_{f != n} tanh(m_f / 2), and the
@@ -168,7 +181,7 @@ __device__ __forceinline__ void check_node(const TrainArgs &a, const Adj &d, con
         c.q[n] = 0.f;
         if (d.sl[n] != kNoSlot) {
             const float m = v[d.sl[n]];
-            c.q[n] = fminf(__fdiv_rn(2.0f, expm1f(fabsf(m))), 1e12f);
+            c.q[n] = fminf(__fdividef(2.0f, expm1f(fabsf(m))), 1e12f);
             c.neg |= (m < 0.f ? 1u : 0u) << n;
         }
     }
@@ -180,11 +193,11 @@ __device__ __forceinline__ void check_node(const TrainArgs &a, const Adj &d, con
     const uint32_t odd = __popc(c.neg) & 1u;
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-        const float mag = log1pf(__fdiv_rn(2.0f, c.E[n]));
+        const float mag = log1pf(__fdividef(2.0f, c.E[n]));
         c.r[n] = ((c.neg >> n) & 1u) != odd ? -mag : mag;
         c.out[n] = 0.f;
         if (d.sl[n] != kNoSlot)
-            c.out[n] = fminf(fmaxf(__fmul_rn(__fmul_rn(a.w[d.ce + n], d.sigma), c.r[n]), -a.clip), a.clip);
+            c.out[n] = fminf(fmaxf(__fmul_rn(d.ws[n], c.r[n]), -a.clip), a.clip);
     }
 }
 
@@ -285,7 +298,7 @@ __device__ __forceinline__ float2 parity_combine(float2 x, float2 y) {
 __device__ __forceinline__ void marginals(const float (&Q)[3], float (&pi)[4]) {
     const float c0 = fminf(0.f, fminf(Q[0], fminf(Q[1], Q[2])));
     const float e[4] = {expf(c0), expf(c0 - Q[0]), expf(c0 - Q[1]), expf(c0 - Q[2])};
-    const float z = 1.f / (e[0] + e[1] + e[2] + e[3]);
+    const float z = __fdividef(1.f, e[0] + e[1] + e[2] + e[3]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) pi[k] = e[k] * z;
 }
@@ -301,9 +314,9 @@ __device__ __forceinline__ float2 comm_anti(const float (&pi)[4], uint32_t P) {
 
 // What the logical operators need from one warp: the parity distribution over
 // its qubits and, for the gradient, sum ln |c - a| and the number of negative
-// c - a.  A chunk of operators is gathered per barrier: as many as `cap` float4
-// hold for the CTA's warps.
-constexpr int kLogCap = 32;  // float4 of shared memory
+// c - a.  A chunk of operators is gathered per barrier: as many as 32 float4 hold
+// for the CTA's warps.
+__host__ __device__ inline int logical_chunk(int n_log, int warps) { return n_log * warps <= 32 ? n_log : 32 / warps; }
 
 template <bool GRAD>
 __device__ __forceinline__ float4 logical_partial(float2 ca, bool has) {
@@ -340,18 +353,16 @@ __device__ __forceinline__ float4 logical_total(const float4 *part, int i, int n
     return t;
 }
 
-// Pauli of logical operator l on qubit x.
-__device__ __forceinline__ uint32_t logical_pauli(const TrainArgs &a, int l, int x) {
-    return x < a.N ? a.logicals[(size_t)l * a.N + x] : 0u;
-}
+// Pauli of logical operator l on the thread's qubit.
+__device__ __forceinline__ uint32_t logical_pauli(const Adj &d, int l) { return (d.logp >> (2 * l)) & 3u; }
 
 // Parities <E, L> of the true error with the logical operators (bit l), the
 // same on every thread.
-__device__ __forceinline__ uint32_t true_logical_parities(const TrainArgs &a, int x, int shot) {
+__device__ __forceinline__ uint32_t true_logical_parities(const TrainArgs &a, const Adj &d, int x, int shot) {
     uint32_t tau = 0;
     const uint32_t e = x < a.N ? a.err[(size_t)shot * a.N + x] : 0u;
     for (int l = 0; l < a.n_log; ++l)
-        tau |= (uint32_t)(__syncthreads_count((int)anti(e, logical_pauli(a, l, x))) & 1) << l;
+        tau |= (uint32_t)(__syncthreads_count((int)anti(e, logical_pauli(d, l))) & 1) << l;
     return tau;
 }
 
@@ -367,11 +378,11 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
     const int Np = a.n_pad;
     float *msg = sm;                                                   // [4 Np]
     float2 *ub = reinterpret_cast<float2 *>(sm + 4 * Np);              // [4 Np] edge parity distributions (coset)
-    float4 *part = reinterpret_cast<float4 *>(sm + 12 * Np);           // [kLogCap] (coset)
+    float4 *part = reinterpret_cast<float4 *>(sm + 12 * Np);           // [chunk][warps] (coset)
     __shared__ float red[32];
     const int x = threadIdx.x, shot = blockIdx.x, warp = x >> 5, warps = blockDim.x >> 5;
     const Adj d = load_adj(a, x, shot);
-    const uint32_t tau = COSET ? true_logical_parities(a, x, shot) : 0u;
+    const uint32_t tau = COSET ? true_logical_parities(a, d, x, shot) : 0u;
     const bool qubit = x < a.N, check = x < a.M;
     float Pi0[3] = {0.f, 0.f, 0.f}, Q[3] = {0.f, 0.f, 0.f}, g[3] = {0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
     if (qubit) {
@@ -381,7 +392,7 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
         initial_messages(a, d.vp, Pi0, v);
         put4(msg + 4 * x, v);
     }
-    const int chunk = min(a.n_log, kLogCap / warps);
+    const int chunk = logical_chunk(a.n_log, warps);
     float loss = 0.f, loss_log = 0.f;
     // the coset loss's check terms of the iteration whose ub is complete
     auto check_terms = [&]() {
@@ -443,7 +454,7 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
             for (int l0 = 0; l0 < a.n_log; l0 += chunk) {
                 const int n = min(chunk, a.n_log - l0);
                 for (int i = 0; i < n; ++i) {
-                    const uint32_t P = logical_pauli(a, l0 + i, x);
+                    const uint32_t P = logical_pauli(d, l0 + i);
                     const float4 r = logical_partial<false>(comm_anti(pi, P), P != 0u);
                     if ((x & 31) == 0) part[warp * n + i] = r;
                 }
@@ -481,10 +492,11 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
 }
 
 // Shared memory of the backward kernel, in floats.
-__host__ __device__ inline size_t backward_floats(int Np, int K, bool momentum) {
+inline size_t backward_floats(int Np, int K, bool momentum, int n_log, int warps) {
     // m_v->c history | m_c->v | its adjoint | adjoint of m_v->c | edge
     // parities' second half | Q (and g) history | logical partials | warp sums
-    return (size_t)4 * Np * (K + 1 + 4) + (size_t)3 * Np * (K + 1) * (momentum ? 2 : 1) + 4 * kLogCap + 96;
+    return (size_t)4 * Np * (K + 1 + 4) + (size_t)3 * Np * (K + 1) * (momentum ? 2 : 1) +
+           (size_t)(4 * logical_chunk(n_log, warps) + 3) * warps;
 }
 
 // Backward: one CTA per shot; segments of K iterations recomputed from the
@@ -502,8 +514,11 @@ __host__ __device__ inline size_t backward_floats(int Np, int K, bool momentum) 
 // the product over the other qubits, and d u_j / d Q_W = 2 pi_W (c_j -
 // [W commutes with the operator's Pauli on j]), i.e. 2 pi_W c_j where W
 // anticommutes and -2 pi_W a_j where it commutes.
-template <int MODEL, bool COSET>
-__global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs a) {
+// SMALL: CTAs of at most 320 threads take up to 96 registers a thread (20 warps
+// per SM): planar d = 9, whose shared memory holds five CTAs of five warps, runs
+// 1731 us with five and 72 registers, 1639 us with four and 80.
+template <int MODEL, bool COSET, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 320 : 1024, SMALL ? 2 : 1) train_backward_kernel(const TrainArgs a) {
     extern __shared__ __align__(16) float sm[];
     const int Np = a.n_pad, K = a.K, S4 = 4 * Np;
     float *vh = sm;                               // [K+1][S4]  m_v->c^(t0 .. t0+K)
@@ -516,10 +531,10 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
     float *Qh = vbar + S4;                        // [K+1][3Np]  Q^(t0 .. t0+K)
     float *gh = Qh + (size_t)(K + 1) * 3 * Np;    // [K+1][3Np]  g^(t0 .. t0+K) (Momentum only)
     float4 *part = reinterpret_cast<float4 *>(gh + (MODEL == kMomentum ? (size_t)(K + 1) * 3 * Np : 0));
-    float *red = reinterpret_cast<float *>(part + kLogCap);  // [3 warps]
+    float *red = reinterpret_cast<float *>(part + logical_chunk(a.n_log, blockDim.x >> 5) * (blockDim.x >> 5));  // [3 warps]
     const int x = threadIdx.x, shot = blockIdx.x, warp = x >> 5, warps = blockDim.x >> 5;
     const Adj d = load_adj(a, x, shot);
-    const uint32_t tau = COSET ? true_logical_parities(a, x, shot) : 0u;
+    const uint32_t tau = COSET ? true_logical_parities(a, d, x, shot) : 0u;
     const bool qubit = x < a.N, check = x < a.M;
     float Pi0[3] = {0.f, 0.f, 0.f};
     if (qubit) prior_llr(a, x, Pi0);
@@ -529,7 +544,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
     float gbar[3] = {0.f, 0.f, 0.f};  // adjoint of g^(t) (Momentum)
     float wbar[4] = {0.f, 0.f, 0.f, 0.f};
     float *row = a.rows + (size_t)shot * a.width;
-    const int chunk = COSET ? min(a.n_log, kLogCap / warps) : 1;
+    const int chunk = logical_chunk(a.n_log, warps);
     const float scale_c = 1.f / ((float)a.B * (float)a.T * (float)a.M);
     const float scale_l = 1.f / ((float)a.B * (float)a.T * (float)a.n_log);
     CheckNode c;
@@ -543,10 +558,10 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
             for (int n = 0; n < 4; ++n) {
                 G[n] = 0.f;
                 if (d.sl[n] == kNoSlot) continue;
-                const float ws = a.w[d.ce + n] * d.sigma, cb = cbar[d.sl[n]];
-                if (fabsf(ws * c.r[n]) <= a.clip) {
+                const float cb = cbar[d.sl[n]];
+                if (fabsf(d.ws[n] * c.r[n]) <= a.clip) {
                     wbar[n] += cb * d.sigma * c.r[n];
-                    const float h = cb * ws / hfun(c.E[n]);
+                    const float h = __fdividef(cb * d.ws[n], hfun(c.E[n]));
                     G[n] = c.r[n] < 0.f ? -h : h;
                 }
             }
@@ -652,7 +667,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
                 for (int l0 = 0; l0 < a.n_log; l0 += chunk) {
                     const int n = min(chunk, a.n_log - l0);
                     for (int i = 0; i < n; ++i) {
-                        const uint32_t P = logical_pauli(a, l0 + i, x);
+                        const uint32_t P = logical_pauli(d, l0 + i);
                         const float4 r = logical_partial<true>(comm_anti(pi, P), P != 0u);
                         if ((x & 31) == 0) part[warp * n + i] = r;
                     }
@@ -666,7 +681,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
                             eo = parity_combine(eo, in[m]);
                         }
                         const float P = d.sigma < 0.f ? eo.y : eo.x;
-                        const float g0 = P > kMinProb ? -d.sigma / P * scale_c : 0.f;
+                        const float g0 = P > kMinProb ? -d.sigma * __fdividef(scale_c, P) : 0.f;
                         float u[4];
 #pragma unroll
                         for (int m = 0; m < 4; ++m) u[m] = in[m].x - in[m].y;
@@ -678,7 +693,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
                     }
                     // the operators' gradient (the CTA's totals of this chunk)
                     for (int i = 0; i < n; ++i) {
-                        const uint32_t P = logical_pauli(a, l0 + i, x);
+                        const uint32_t P = logical_pauli(d, l0 + i);
                         if (!P) continue;
                         const float4 tot = logical_total<true>(part, i, n, warps);
                         const bool odd = (tau >> (l0 + i)) & 1u;
@@ -688,7 +703,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
                         const float u = ca.x - ca.y, lg = logf(fmaxf(fabsf(u), 1e-30f));
                         const int others = (int)tot.w - (u < 0.f ? 1 : 0);
                         const float U = expf(tot.z - lg);  // product over the others
-                        const float gl = (((others & 1) != 0) == odd ? -U : U) / Pm * scale_l;
+                        const float gl = (((others & 1) != 0) == odd ? -U : U) * __fdividef(scale_l, Pm);
 #pragma unroll
                         for (int w = 0; w < 3; ++w) Qbar[w] += gl * pi[w + 1] * (anti(w + 1, P) ? ca.x : -ca.y);
                     }
@@ -743,7 +758,7 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
                     if (Lsum[h] == 0.f) continue;
                     const int i = h == 0 ? 1 : 0, j = h == 2 ? 1 : 2;
                     const float uh = expf(-fabsf(Q[h])), ud = expf(-fabsf(Q[i] - Q[j]));
-                    const float sh = (Q[h] < 0.f ? 1.f : uh) / (1.f + uh), sd = 1.f / (1.f + ud);
+                    const float sh = __fdividef(Q[h] < 0.f ? 1.f : uh, 1.f + uh), sd = __fdividef(1.f, 1.f + ud);
                     Qtot[h] -= Lsum[h] * sh;
                     const bool first = Q[i] < Q[j];  // the larger share: of the smaller Q
                     Qtot[i] += Lsum[h] * (first ? sd : ud * sd);
@@ -802,6 +817,15 @@ __global__ void __launch_bounds__(1024, 1) train_backward_kernel(const TrainArgs
     if (check)
         for (int n = 0; n < 4; ++n)
             if (d.sl[n] != kNoSlot) row[2 * a.T + d.ce + n] = wbar[n];
+}
+
+template <int MODEL, bool COSET>
+void (*pick_size(int threads))(const TrainArgs) {
+    return threads <= 320 ? train_backward_kernel<MODEL, COSET, true> : train_backward_kernel<MODEL, COSET, false>;
+}
+void (*pick_backward(bool momentum, bool coset, int threads))(const TrainArgs) {
+    if (momentum) return coset ? pick_size<kMomentum, true>(threads) : pick_size<kMomentum, false>(threads);
+    return coset ? pick_size<kEWAInit, true>(threads) : pick_size<kEWAInit, false>(threads);
 }
 
 // Sums over the shots: out_k = scale * sum_b rows[b][k], the columns k of the
@@ -937,14 +961,16 @@ int bpq_train_forward(const bpq_tanner *t, int model, const uint32_t *syn_dev, c
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool mom = model == BPQ_TRAIN_MOMENTUM;
     const bool coset = a.loss_kind == BPQ_TRAIN_LOSS_COSET;
-    const size_t smem = sizeof(float) * ((coset ? 12 : 4) * (size_t)a.n_pad + (coset ? 4 * bpq::tr::kLogCap : 0));
+    const int threads = bpq::tr::threads_for(t), warps = threads / 32;
+    const size_t smem = sizeof(float) * ((coset ? 12 : 4) * (size_t)a.n_pad +
+                                         4 * (size_t)bpq::tr::logical_chunk(a.n_log, warps) * warps);
     if (smem > 227 * 1024) return fail(BPQ_EINVAL, "code too large for the training kernels' shared memory");
     using namespace bpq::tr;
     void (*fn)(const TrainArgs) = mom ? (coset ? train_forward_kernel<kMomentum, true> : train_forward_kernel<kMomentum, false>)
                                       : (coset ? train_forward_kernel<kEWAInit, true> : train_forward_kernel<kEWAInit, false>);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("train forward attribute: ") + cudaGetErrorString(e));
-    fn<<<B, bpq::tr::threads_for(t), smem, st>>>(a);
+    fn<<<B, threads, smem, st>>>(a);
     // per-shot sums: over qubits (posterior loss) or already normalised (coset loss)
     bpq::tr::launch_reduce(a.loss_shot, B, 1, {{loss_dev}, {1}},
                            coset ? 1.f / (float)B : 1.f / ((float)B * (float)t->N), st);
@@ -964,15 +990,13 @@ int bpq_train_backward(const bpq_tanner *t, int model, const uint32_t *syn_dev, 
     if (!grad_alpha_dev || !grad_beta_dev || !grad_w_dev || (mom && !grad_gamma_dev))
         return fail(BPQ_EINVAL, "NULL gradient output");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t smem = sizeof(float) * bpq::tr::backward_floats(a.n_pad, a.K, mom);
+    const int threads = bpq::tr::threads_for(t);
+    const size_t smem = sizeof(float) * bpq::tr::backward_floats(a.n_pad, a.K, mom, a.n_log, threads / 32);
     if (smem > 227 * 1024) return fail(BPQ_EINVAL, "checkpoint interval too long for shared memory");
-    using namespace bpq::tr;
-    const bool coset = a.loss_kind == kCoset;
-    void (*fn)(const TrainArgs) = mom ? (coset ? train_backward_kernel<kMomentum, true> : train_backward_kernel<kMomentum, false>)
-                                      : (coset ? train_backward_kernel<kEWAInit, true> : train_backward_kernel<kEWAInit, false>);
+    void (*fn)(const bpq::tr::TrainArgs) = bpq::tr::pick_backward(mom, a.loss_kind == BPQ_TRAIN_LOSS_COSET, threads);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("train backward attribute: ") + cudaGetErrorString(e));
-    fn<<<B, bpq::tr::threads_for(t), smem, st>>>(a);
+    fn<<<B, threads, smem, st>>>(a);
     // per-shot rows hold [alpha | beta | w | gamma]
     bpq::tr::launch_reduce(a.rows, B, a.width,
                            {{grad_alpha_dev, grad_beta_dev, grad_w_dev, mom ? grad_gamma_dev : nullptr},
