@@ -254,8 +254,8 @@ int bpq_get_launch(const bpq_tanner *t, int *threads_per_shot, int *shots_per_ct
  * next shot from the queue as soon as its own shot stops (split table layout
  * only, see bpq_tanner_layout; plain, Momentum, AdaGrad and EWAInit BP; not
  * the trace, serial, batched or AEWA-BP paths); 0 = automatic (2 where it
- * applies and the batch holds at least 40 shots per resident one-shot shot
- * group, e.g. 24320 toric d = 15 shots on a GB300 - 192 for codes of at most
+ * applies and the batch holds at least 80 shots per resident one-shot shot
+ * group, e.g. 48640 toric d = 15 shots on a GB300 - 256 for codes of at most
  * 96 nodes: a pair's iteration does two shots' work, so smaller batches, whose
  * time is set by their slowest shots, finish sooner with one shot per
  * thread).  Per-shot results are the same
@@ -387,7 +387,10 @@ void bpq_batch_free(bpq_batch *b);
  * its 1024 threads (at most 15 multi-warp or 32 one-warp groups) and in
  * 227 KB of shared memory.  0 = automatic: the choice that keeps the most
  * node slots of a CTA busy (groups x max(N, M) / (nodes_per_thread x 1024)),
- * two nodes per thread on a tie.  Independent of bpq_set_launch.
+ * two nodes per thread on a tie.  In the batched kernel the threads that the
+ * groups leave over form one more, smaller group (not counted in the reported
+ * shape) where they are at least half a group's, shared memory has room for it
+ * and the plan holds many shots.  Independent of bpq_set_launch.
  * Errors: EINVAL (a value outside 0..2, or a shape that does not fit).
  * bpq_get_batch_launch reports the shape for `variant` (any output pointer
  * may be NULL). */

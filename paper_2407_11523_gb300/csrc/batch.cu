@@ -52,6 +52,19 @@ void batch_start_items(const std::vector<double> &weight, int ctas, int *start) 
 }
 
 namespace {
+// The batched kernel's threads that an item's shot groups leave over form one
+// more, smaller group (its shots take longer: more nodes per thread) where they
+// are at least half a group's and shared memory has room (planar d = 25: 416 of
+// 1024 threads, idle otherwise), and an item's initial messages take a table of
+// their own where shared memory has room for that: both once the batch holds
+// this many CTA loads of shots per SM, since a smaller batch ends with its
+// slowest shots and does not repay the table.  Without and with both, ten codes
+// in turn (us): plain, p = 0.03, 1146 shots (2 loads) 258 / 269, 4000 (6) 631 /
+// 630, 10000 (16) 1437 / 1327, 30000 (47) 4028 / 3709; EWAInit, p = 0.06, 4000
+// shots 479 / 510, 10000 1007 / 988, 30000 2765 / 2581; 262144 shots 24.7 / 21.2
+// ms.
+constexpr long kManyLoads = 8;
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
 }  // namespace bpq
@@ -94,6 +107,7 @@ int bpq_batch_plan(const bpq_batch_item *items, int n_items, int variant, const 
 
     std::vector<bpq::DecodeArgs> desc(n_items);
     std::vector<double> weight(n_items);
+    std::vector<bpq::LaunchShape> shape(n_items);
     size_t smem = 0;
     int npt_max = 1;
     bool generic = false;  // some item uses the generic table layout
@@ -114,13 +128,27 @@ int bpq_batch_plan(const bpq_batch_item *items, int n_items, int variant, const 
         a.n_pad = s.n_pad;
         a.slots_floats = s.slots_floats;
         a.group_bytes = s.group_bytes;
-        a.npt = s.npt;
         a.groups_per_cta = s.groups_per_cta;
+        shape[g] = s;
         npt_max = std::max(npt_max, s.npt);
         generic = generic || a.split == 0;
-        smem = std::max(smem, s.smem);
         weight[g] = (double)items[g].B * t->E;
         useful_ctas += (items[g].B + s.groups_per_cta - 1) / s.groups_per_cta;
+    }
+    const bool many = useful_ctas >= bpq::kManyLoads * items[0].tanner->num_sms;
+    for (int g = 0; g < n_items; ++g) {
+        bpq::DecodeArgs &a = desc[g];
+        bpq::LaunchShape &s = shape[g];
+        const int left = bpq::kBatchThreads - s.groups_per_cta * s.T;
+        if (many && s.groups_per_cta < 15 && 2 * left >= s.T && s.smem + s.group_bytes <= 227 * 1024) {
+            a.rest_warps = left / 32;
+            s.smem += s.group_bytes;
+        }
+        if (many && s.smem + 16 * (size_t)s.n_pad <= 227 * 1024) {
+            a.init_bytes = 16u * (uint32_t)s.n_pad;
+            s.smem += a.init_bytes;
+        }
+        smem = std::max(smem, s.smem);
     }
     if (smem > 227 * 1024) return fail(BPQ_EINVAL, "a code of the batch needs more than 227 KB of shared memory");
 

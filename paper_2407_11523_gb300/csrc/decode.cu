@@ -2,6 +2,7 @@
 // is in decode_kernel.cuh, instantiated per variant in decode_<variant>.cu).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "bpq_internal.h"
@@ -125,6 +126,17 @@ int one_shot_shape(const bpq_tanner *t, int variant, int T, int gpc, LaunchShape
     s->group_bytes = (uint32_t)(4 * s->slots_floats + 4 * nstate * s->n_pad);
     s->smem = kSmemHeader + t->table.size() + (size_t)12 * s->n_pad + (size_t)gpc * s->group_bytes;
     if (s->smem > 227 * 1024) return fail(BPQ_EINVAL, "shared memory of the launch shape exceeds 227 KB");
+    // the initial messages, unless they cost a resident CTA (48 registers a
+    // thread: 1280 threads per SM).  Without and with them: AdaGrad on xzzx
+    // d = 7, 5.7 iterations a shot, 200000 shots, 1.30 and 1.24 ms; AEWA on planar
+    // d = 11, 11.3 iterations, 10^5 shots, 11.3 and 11.2
+    const size_t init = 16 * (size_t)s->n_pad, by_threads = std::max(1, 1280 / (T * gpc));
+    auto resident = [&](size_t smem) { return std::min<size_t>(by_threads, 228 * 1024 / (smem + 1024)); };
+    s->init_bytes = 0;
+    if (s->smem + init <= 227 * 1024 && resident(s->smem + init) == resident(s->smem)) {
+        s->init_bytes = (uint32_t)init;
+        s->smem += init;
+    }
     return BPQ_OK;
 }
 }  // namespace
@@ -235,12 +247,16 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // automatic choice: a pair's iteration does two shots' work, so a
         // batch's tail (its slowest shots) runs longer; pairing pays only
         // once each resident one-shot group would decode many shots.
-        // Measured on GB300, one shot per thread against two (ms): toric
-        // d = 15 EWAInit 20000 shots 1.298 / 1.279, 65536 3.93 / 3.73; planar
-        // d = 9 plain 50000 1.62 / 1.60; planar d = 21 Momentum 5000 2.32 /
-        // 2.28: all at 16 to 33 shots per resident one-shot group.  One-warp
-        // pair groups have the longest tail: planar d = 7 EWAInit 300000 shots
-        // (123 per group) 0.986 / 1.027, 10^6 in favour of pairs.
+        // Measured on GB300, one shot per thread against two (ms; shots per
+        // resident one-shot group): toric d = 15 EWAInit, p = 0.06, 20000 (33)
+        // 0.877 / 0.923, p = 0.08, 40000 (66) 2.41 / 2.36; planar d = 13
+        // EWAInit 50000 (55) 1.40 / 1.44, 100000 (110) 2.71 / 2.73; planar
+        // d = 9 EWAInit 100000 (66) 0.914 / 0.952, plain 120000 (79) 2.79 /
+        // 2.73; planar d = 11 plain 100000 (82) 4.22 / 4.12; planar d = 25
+        // plain 10000 (66) 6.00 / 5.97.  The crossing lies between 60 and 110.
+        // One-warp pair groups have the longest tail: planar d = 7 EWAInit
+        // 300000 (123) 0.957 / 1.011, 600000 (247) 1.843 / 1.844, 10^6 (411)
+        // 3.04 / 2.93; AdaGrad on xzzx d = 7 200000 (82) 1.08 / 1.30.
         LaunchShape one;
         int per_sm = 0;
         DecodeKernelFn f1 = nullptr;
@@ -274,6 +290,8 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         (long)a.B < kOneNodeShotsPerGroup * per_sm * t->num_sms * s.groups_per_cta) {
         rc = one_shot_shape(t, variant, (nodes + 31) / 32 * 32, 0, &s);
         if (rc) return rc;
+        s.smem -= s.init_bytes;  // too few shots per group to repay the table
+        s.init_bytes = 0;
         fn = t->debug_checks ? pick_debug(variant, s.npt, false, false, a.split) : pick(variant, s.npt, false, a.split);
         if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant");
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
@@ -291,6 +309,7 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     a.n_pad = s.n_pad;
     a.slots_floats = s.slots_floats;
     a.group_bytes = s.group_bytes;
+    a.init_bytes = pairs ? 0 : s.init_bytes;
     if (ctas_out) *ctas_out = (int)ctas;
     rc = cuda_check(cudaMemsetAsync(a.work, 0, 8, st), "workspace reset");  // the shot queue, the error word
     if (rc) return rc;

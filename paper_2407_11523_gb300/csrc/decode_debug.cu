@@ -12,6 +12,15 @@ namespace bpq {
 
 namespace {
 
+template <int V, int NPT>
+DecodeKernelFn pick_debug_one(int layout) {
+    switch (layout) {
+        case 2: return dk_debug::decode_kernel<V, NPT, false, true, true>;
+        case 1: return dk_debug::decode_kernel<V, NPT, false, true, false>;
+        default: return dk_debug::decode_kernel<V, NPT, false, false, false>;
+    }
+}
+
 template <int V>
 DecodeKernelFn pick_debug_v(int npt, bool pairs, bool one, int layout) {
     if (pairs) {
@@ -19,12 +28,7 @@ DecodeKernelFn pick_debug_v(int npt, bool pairs, bool one, int layout) {
         if (layout == 1) return one ? dk_debug::decode_pair_kernel<V, false, true> : dk_debug::decode_pair_kernel<V, false, false>;
         return nullptr;
     }
-    if (npt < 1 || npt > 2) return nullptr;
-    switch (layout) {
-        case 2: return npt == 1 ? dk_debug::decode_kernel<V, 1, false, true, true> : dk_debug::decode_kernel<V, 2, false, true, true>;
-        case 1: return npt == 1 ? dk_debug::decode_kernel<V, 1, false, true, false> : dk_debug::decode_kernel<V, 2, false, true, false>;
-        default: return npt == 1 ? dk_debug::decode_kernel<V, 1, false, false, false> : dk_debug::decode_kernel<V, 2, false, false, false>;
-    }
+    return npt == 1 ? pick_debug_one<V, 1>(layout) : npt == 2 ? pick_debug_one<V, 2>(layout) : nullptr;
 }
 
 }  // namespace

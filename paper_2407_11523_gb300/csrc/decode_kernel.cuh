@@ -1,16 +1,27 @@
 // Flooding-schedule GF(4) belief propagation on sm_103a: one group of G warps
-// decodes one shot at a time; each thread owns NPT checks and NPT qubits
-// (node j belongs to thread j mod 32G).  The shot's edge messages live in
-// shared memory, one float per edge, updated in place: the check pass turns
-// variable-to-check messages into check-to-variable messages and the variable
-// pass turns them back.  Groups synchronise on their own named barrier, so
-// every shot stops as soon as its hard decision satisfies the syndrome, and
-// the group then takes the next shot from a global work queue (a persistent
-// kernel, grid = SMs x resident CTAs).  The Tanner-graph adjacency is staged
-// once per CTA into shared memory by a bulk TMA copy; the per-qubit prior
-// LLRs sit in shared memory (shared by the CTA's groups) and the per-qubit
-// variant state in the group's shared memory, so that registers hold only
-// adjacency and temporaries.
+// decodes one shot at a time; thread tg of the group's T = 32G threads owns the
+// checks and qubits tg, tg + T, ... (at most kMaxLoopNodes of each).  The shot's
+// edge messages live in shared memory, one float per edge, updated in place: the
+// check pass turns variable-to-check messages into check-to-variable messages
+// and the variable pass turns them back.  Groups synchronise on their own named
+// barrier, so every shot stops as soon as its hard decision satisfies the
+// syndrome, and the group then takes the next shot from a global work queue (a
+// persistent kernel, grid = SMs x resident CTAs).  The Tanner-graph adjacency is
+// staged once per CTA into shared memory by a bulk TMA copy; a thread with one
+// or two nodes keeps its own in registers, one with more reads it on every
+// pass.  The per-qubit prior LLRs and, where they fit, the initial messages
+// (which do not depend on the shot: a shot starts with a copy) sit in shared
+// memory, shared by the CTA's groups, and the per-qubit variant state in the
+// group's shared memory, so that registers hold only temporaries.  The owned
+// checks' syndrome bits sit in one word that rotates so that the current one is
+// at the sign and at the parity position, and the decisions take two bits per
+// qubit of another; for split tables they are the two anticommutation bits, so
+// that no Pauli code is built and taken apart again.  Together: AdaGrad on xzzx
+// d = 7, 200000 shots, 1.31 -> 1.24 ms; AEWA on planar d = 11, 10^5 shots,
+// 11.38 -> 11.2.
+//
+// What bounds it: instruction issue, with the special-function unit close
+// behind and the shots' uneven iteration counts at the end of a batch.
 //
 // Arithmetic (Sec. II-B1 and Sec. III of the paper, fp32):
 //  * check-to-variable, eq. (h_update): 2 atanh(prod_k tanh(m_k/2)) with
@@ -48,8 +59,8 @@
 // Bounds-checked build: with BPQ_DEBUG defined (decode_debug_*.cu compile
 // these headers a second time, into namespace dk_debug), every CTA checks its
 // launch's shared-memory layout against the dynamic shared memory it got,
-// every thread checks the slot indices and table offsets of the nodes it
-// loads, and every output write checks its index.  A failed check sets the
+// the staged table's slot indices are checked where they are prepared, and every
+// output write checks its index.  A failed check sets the
 // device error word (work[1] = 5) and substitutes a safe index (the zero slot,
 // or no write); a CTA whose layout does not fit returns before its first
 // barrier.  Nothing traps.
@@ -444,44 +455,40 @@ __device__ __forceinline__ float adagrad_q(const ShotParams &sp, float qp, float
     return __fmaf_rn(-__fmul_rn(sp.alpha, gp), rcp(__fadd_rn(sqrt_approx(G), sp.eps)), qp);
 }
 
-// Per-thread adjacency of the owned checks and qubits of one code:
-// cs: the four message slots of each owned check (padding -> zero slot);
-// info: check Paulis (bits 0-7) | qubit Paulis (bits 8-15); pp: qubit
-// Paulis one per byte.
+// Owned nodes of a thread at most: two bits of a 32-bit word each.
+constexpr int kMaxLoopNodes = 16;
+
+// The staged table's slots of missing edges become the zero slot (all threads
+// of the CTA; a barrier before and after).
+__device__ __forceinline__ void prepare_table(const DecodeArgs &a, uint8_t *tab) {
+    const uint16_t zero = (uint16_t)(4 * a.n_pad);
+    uint16_t *slot = reinterpret_cast<uint16_t *>(tab);
+    for (int k = threadIdx.x; k < 4 * a.M; k += blockDim.x)
+        if (BPQ_IN_BOUNDS(2 * k + 1, a.table_bytes, a.work + 1)) {
+            // a slot index is an edge slot (< 4 n_pad) or no slot
+            if (slot[k] == kNoSlot || !BPQ_IN_BOUNDS(slot[k], zero + 1u, a.work + 1)) slot[k] = zero;
+        }
+}
+
+// Adjacency of a thread's first NPT checks and qubits in registers (from the
+// prepared table).  NPT = 0: none are kept, the passes read the prepared
+// table; one or two nodes in registers are faster where they cover the code (the
+// read stands before every message load: AdaGrad on xzzx d = 7, two nodes per
+// thread, 200000 shots, 1.39 ms from the table against 1.24; AEWA on planar
+// d = 11, 10^5 shots, 12.7 against 11.2).
 template <int NPT>
-struct ThreadAdj {
-    uint32_t cs_lo[NPT], cs_hi[NPT], info[NPT], pp[NPT];
+struct Owned {
+    uint2 chk[NPT ? NPT : 1];  // slots of the check's edges, 16 bits each
+    uint32_t vp[NPT ? NPT : 1];  // Pauli codes of the qubit's edges, two bits each
 };
 
 template <int NPT>
-__device__ __forceinline__ void load_adjacency(const DecodeArgs &a, const uint8_t *tab, int T, int tg, int npt,
-                                               ThreadAdj<NPT> &adj) {
-    const uint32_t kZero = 4u * (uint32_t)a.n_pad;
+__device__ __forceinline__ void load_owned(const DecodeArgs &a, const uint8_t *tab, int T, int tg, Owned<NPT> &o) {
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
-        adj.cs_lo[k] = adj.cs_hi[k] = kZero | (kZero << 16);
-        adj.info[k] = 0u;
-        adj.pp[k] = 0u;
-        const int i = k * T + tg;
-        if (k < npt && i < a.M && BPQ_IN_BOUNDS(8 * i + 7, a.table_bytes, a.work + 1) &&
-            BPQ_IN_BOUNDS(a.off_chk_pauli + i, a.table_bytes, a.work + 1)) {
-            const uint2 s = *reinterpret_cast<const uint2 *>(tab + 8 * i);
-            uint32_t s0 = s.x & 0xFFFFu, s1 = s.x >> 16, s2 = s.y & 0xFFFFu, s3 = s.y >> 16;
-#ifdef BPQ_DEBUG
-            // a slot index is an edge slot (< 4 n_pad) or no slot
-            uint32_t *sv[4] = {&s0, &s1, &s2, &s3};
-            for (int n = 0; n < 4; ++n)
-                if (*sv[n] != kNoSlot && !BPQ_IN_BOUNDS(*sv[n], kZero, a.work + 1)) *sv[n] = kNoSlot;
-#endif
-            adj.cs_lo[k] = (s0 == kNoSlot ? kZero : s0) | ((s1 == kNoSlot ? kZero : s1) << 16);
-            adj.cs_hi[k] = (s2 == kNoSlot ? kZero : s2) | ((s3 == kNoSlot ? kZero : s3) << 16);
-            adj.info[k] = tab[a.off_chk_pauli + i];
-        }
-        if (k < npt && i < a.N && BPQ_IN_BOUNDS(a.off_var_pauli + i, a.table_bytes, a.work + 1)) {
-            const uint32_t vp = tab[a.off_var_pauli + i];
-            adj.info[k] |= vp << 8;
-            adj.pp[k] = (vp & 3u) | (((vp >> 2) & 3u) << 8) | (((vp >> 4) & 3u) << 16) | (((vp >> 6) & 3u) << 24);
-        }
+        const int x = k * T + tg;
+        o.chk[k] = x < a.M ? reinterpret_cast<const uint2 *>(tab)[x] : make_uint2(0u, 0u);
+        o.vp[k] = x < a.N ? tab[a.off_var_pauli + x] : 0u;
     }
 }
 
@@ -507,146 +514,169 @@ __device__ __forceinline__ void load_prior(const DecodeArgs &a, float *PiS) {
     }
 }
 
-// Shared-memory regions of shot group `group` of a code laid out from `base`
-// (base = the staged table): table | Pi [3][Np] | groups.
+// Shared-memory regions of shot group `group` of a code laid out from `base`:
+// table | Pi [3][Np] | initial messages (a.init_bytes: 4 Np floats, or none) |
+// groups.
 struct GroupMem {
-    float *PiS, *slots, *state;
+    const uint8_t *tab;
+    float *PiS, *init, *slots, *state;  // init: nullptr if the table holds none
 };
 
 __device__ __forceinline__ GroupMem group_mem(const DecodeArgs &a, uint8_t *base, int group) {
     GroupMem m;
+    m.tab = base;
     m.PiS = reinterpret_cast<float *>(base + a.table_bytes);
-    uint8_t *g = base + a.table_bytes + (size_t)12 * a.n_pad + (size_t)group * a.group_bytes;
+    uint8_t *g = base + a.table_bytes + (size_t)12 * a.n_pad;
+    m.init = a.init_bytes ? reinterpret_cast<float *>(g) : nullptr;
+    g += a.init_bytes + (size_t)group * a.group_bytes;
     m.slots = reinterpret_cast<float *>(g);
     m.state = m.slots + a.slots_floats;
     return m;
 }
 
-// Decode one shot with a group of G warps (thread tg of 32G): eq. (init),
+// The initial messages of eq. (init), lambda(Pi^(0)) on every edge (unused
+// positions 0), into the CTA's table, if it holds one.  Needs the prior and the
+// staged table.
+template <int VARIANT, bool SPLIT, bool FULL>
+__device__ __forceinline__ void load_init(const DecodeArgs &a, const GroupMem &m) {
+    if (!m.init) return;
+    const ShotParams sp = shot_params<PhiForm<VARIANT>::value>(a, a.alpha);
+    const float z4[4] = {0.f, 0.f, 0.f, 0.f};
+    const int Np = a.n_pad;
+    for (int j = threadIdx.x; j < a.N; j += blockDim.x)
+        emit_v2c<false, SPLIT, PhiForm<VARIANT>::value, true, FULL>(a, sp, m.init, j, 0, 0, m.tab[a.off_var_pauli + j],
+                                                                    m.PiS[j], m.PiS[Np + j], m.PiS[2 * Np + j], z4, 0u);
+}
+
+// Pauli code of a decision kept by decode_shot: the code itself, or (split
+// layout) bit 0: anticommutes with X, bit 1: with Z.
+template <bool SPLIT>
+__device__ __forceinline__ uint32_t decision_code(uint32_t d) {
+    return SPLIT ? ((d & 1u) << 1) | ((d ^ (d >> 1)) & 1u) : d;
+}
+
+// Decode one shot with a group of G warps (thread tg of T = 32G): eq. (init),
 // then iterations of the check pass and the variable pass until the hard
 // decision satisfies the syndrome or max_iter is reached; writes the shot's
-// outputs.  npt <= NPT is the number of nodes each thread owns.  FULL
-// (split layout only): every check has four edges and every qubit two X and
-// two Z edges, so no edge is padding.  STAGED: a.syn, a.est, a.conv and
-// a.iters may point into shared memory (the serving kernel stages each
-// request's syndrome and outputs there), so the syndrome words are read with
-// a generic load instead of the read-only global path.
+// outputs.  FULL (split layout only): every check has four edges and every
+// qubit two X and two Z edges, so no edge is padding.  STAGED: a.syn, a.est,
+// a.conv and a.iters may point into shared memory (the serving kernel stages
+// each request's syndrome and outputs there), so the syndrome words are read
+// with a generic load instead of the read-only global path.
 template <int VARIANT, int NPT, bool TRACE, bool SPLIT, bool FULL, bool STAGED = false>
-__device__ __forceinline__ int decode_shot(const DecodeArgs &a, const ThreadAdj<NPT> &adj, const GroupMem &m,
-                                           int npt, int T, int tg, int G, int bar_id, int shot, float alpha) {
-    const ShotParams sp = shot_params<PhiForm<VARIANT>::value>(a, alpha);
+__device__ __forceinline__ int decode_shot(const DecodeArgs &a, const Owned<NPT> &own, const GroupMem &m, int T, int tg,
+                                           int G, int bar_id, int shot, float alpha) {
+    constexpr bool PHI = PhiForm<VARIANT>::value;
+    const ShotParams sp = shot_params<PHI>(a, alpha);
     const int N = sp.N, M = sp.M, Np = sp.Np;
-    const uint32_t kZero = 4u * (uint32_t)Np, kTrash = kZero + 1u;
+    const uint32_t kZero = 4u * (uint32_t)Np;
     float *slots = m.slots, *state = m.state;
     const float *PiS = m.PiS;
+    const uint2 *chk = reinterpret_cast<const uint2 *>(m.tab);  // four 16-bit slots per check
+    const uint8_t *vps = m.tab + a.off_var_pauli;
+    const int nk = NPT ? NPT : ((M > N ? M : N) + T - 1) / T;  // owned nodes of thread 0
 
-    // syndrome bits of the owned checks (bit k <-> check k*T + tg)
-    uint32_t sbits = 0;
-#pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-        const int i = k * T + tg;
-        if (k < npt && i < M) {
-            const uint32_t *src = a.syn + (size_t)shot * a.W + (i >> 5);
-            const uint32_t w = STAGED ? *reinterpret_cast<const volatile uint32_t *>(src) : __ldg(src);
-            sbits |= ((w >> (i & 31)) & 1u) << k;
+    // syndrome bits of the owned checks: that of the k-th is at bits 31 (sign)
+    // and 0 (parity) of the word rotated left by 2k
+    uint32_t syn = 0;
+    {
+        const uint32_t *src = a.syn + (size_t)shot * a.W;
+        for (int i = tg, k = 0; i < M; i += T, k += 2) {
+            const uint32_t w = STAGED ? *reinterpret_cast<const volatile uint32_t *>(src + (i >> 5)) : __ldg(src + (i >> 5));
+            if ((w >> (i & 31)) & 1u) syn |= __funnelshift_r(0x80000001u, 0x80000001u, k);
         }
     }
 
     // eq. (init): lambda(Pi^(0)), i.e. the variable pass with Q = Pi^(0)
     // and no incoming messages; Q^(0) = Pi^(0), g^(0) = G^(0) = 0; EWAInit
     // starts from Pi^(1) = Pi^(0) and keeps alpha Pi^(0)
-    uint32_t dk[NPT];
+    for (int j = tg; j < N; j += T) {
+        if (StateArrays<VARIANT>::n >= 3) {
 #pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-        dk[k] = 0;
-        const int j = k * T + tg;
-        if (k < npt && j < N) {
-            const float PX = PiS[j], PY = PiS[Np + j], PZ = PiS[2 * Np + j];
-            if (StateArrays<VARIANT>::n >= 3) {
-                state[j] = PX;
-                state[Np + j] = PY;
-                state[2 * Np + j] = PZ;
+            for (int w = 0; w < 3; ++w) {
+                const float pw = PiS[w * Np + j];
+                state[w * Np + j] = pw;
+                state[(3 + w) * Np + j] = VARIANT == BPQ_EWAINIT ? alpha * pw : 0.f;
             }
-            if (VARIANT == BPQ_EWAINIT) {
-                state[3 * Np + j] = alpha * PX;
-                state[4 * Np + j] = alpha * PY;
-                state[5 * Np + j] = alpha * PZ;
-            } else if (StateArrays<VARIANT>::n == 6) {
-                state[3 * Np + j] = 0.f;
-                state[4 * Np + j] = 0.f;
-                state[5 * Np + j] = 0.f;
+        }
+        if (!TRACE && m.init) {
+            if (SPLIT) {
+#pragma unroll
+                for (int n = 0; n < 4; ++n) slots[n * Np + j] = m.init[n * Np + j];
+            } else {
+                reinterpret_cast<float4 *>(slots)[j] = reinterpret_cast<const float4 *>(m.init)[j];
             }
+        } else {
             const float z4[4] = {0.f, 0.f, 0.f, 0.f};
-            emit_v2c<TRACE, SPLIT, PhiForm<VARIANT>::value, true, FULL>(a, sp, slots, j, 0, shot, adj.info[k] >> 8,
-                                                                        PX, PY, PZ, z4, 0u);
+            emit_v2c<TRACE, SPLIT, PHI, true, FULL>(a, sp, slots, j, 0, shot, vps[j], PiS[j], PiS[Np + j],
+                                                    PiS[2 * Np + j], z4, 0u);
         }
     }
     group_sync(G, bar_id);
 
     int conv = 0, iters = 0;
+    // decisions of the owned qubits, two bits each, the last owned qubit lowest:
+    // whether they anticommute with X and with Z (split layout), or the code
+    uint32_t dec = 0;
     for (int t = 1;; ++t) {
         const bool do_check = t > 1 && (!TRACE || t > sp.max_iter);
         const bool do_msgs = t <= sp.max_iter;
-        uint32_t mismatch = 0;
+        uint32_t mismatch = 0, sw = syn;  // bit 0 of mismatch: a check fails the syndrome test
 
         // ---- check pass: syndrome test of the previous decision, then eq. (h_update) ----
-#pragma unroll
-        for (int k = 0; k < NPT; ++k) {
+#pragma unroll (NPT ? NPT : 1)
+        for (int k = 0; k < nk; ++k) {
             const int i = k * T + tg;
-            if (k < npt && i < M) {
-                const uint32_t sl[4] = {adj.cs_lo[k] & 0xFFFFu, adj.cs_lo[k] >> 16, adj.cs_hi[k] & 0xFFFFu,
-                                        adj.cs_hi[k] >> 16};
-                const uint32_t sb = (sbits >> k) & 1u;
-                uint32_t u[4];
+            if (i >= M) break;
+            const uint2 s4 = NPT ? own.chk[k] : chk[i];
+            const uint32_t sl[4] = {s4.x & 0xFFFFu, s4.x >> 16, s4.y & 0xFFFFu, s4.y >> 16};
+            uint32_t u[4];
 #pragma unroll
-                for (int n = 0; n < 4; ++n) u[n] = __float_as_uint(slots[sl[n]]);
-                // bit 31: the product of the incoming signs; bit 0: the parity
-                // of the previous decision on this check's edges
-                const uint32_t ux = u[0] ^ u[1] ^ u[2] ^ u[3];
-                if (do_check) mismatch |= (ux ^ sb) & 1u;
-                if (do_msgs) {
-                    float mag[4];
+            for (int n = 0; n < 4; ++n) u[n] = __float_as_uint(slots[sl[n]]);
+            // bit 31: (-1)^{s_i} times the product of the incoming signs; bit 0:
+            // the parity of the previous decision on this check's edges plus s_i
+            const uint32_t ux = u[0] ^ u[1] ^ u[2] ^ u[3] ^ sw;
+            sw = __funnelshift_l(sw, sw, 2);
+            mismatch |= ux;
+            if (do_msgs) {
+                float mag[4], ext[4];
 #pragma unroll
-                    for (int n = 0; n < 4; ++n) mag[n] = __uint_as_float(u[n] & 0x7FFFFFFEu);
-                    // (-1)^{s_i} times the product of the incoming signs
-                    const uint32_t sgn = (ux ^ (sb << 31)) & 0x80000000u;
-                    float ext[4];
-                    if (PhiForm<VARIANT>::value) {
-                        // extrinsic sums of phi(|m|) over the other three edges
-                        const float e01 = mag[0] + mag[1], e23 = mag[2] + mag[3];
-                        ext[0] = mag[1] + e23;
-                        ext[1] = mag[0] + e23;
-                        ext[2] = e01 + mag[3];
-                        ext[3] = e01 + mag[2];
-                    } else {
-                        // extrinsic D of each edge: the (+) of the other three deltas,
-                        // two (+) per packed f32x2 instruction pair (each lane equals
-                        // the scalar oplus; a (+) b and b (+) a round alike)
-                        const float2 d = oplus2(make_float2(mag[0], mag[2]), make_float2(mag[1], mag[3]));
-                        const float2 e01 = oplus2(make_float2(mag[1], mag[0]), make_float2(d.y, d.y));
-                        const float2 e23 = oplus2(make_float2(mag[3], mag[2]), make_float2(d.x, d.x));
-                        ext[0] = e01.x;
-                        ext[1] = e01.y;
-                        ext[2] = e23.x;
-                        ext[3] = e23.y;
-                    }
+                for (int n = 0; n < 4; ++n) mag[n] = __uint_as_float(u[n] & 0x7FFFFFFEu);
+                if (PHI) {
+                    // extrinsic sums of phi(|m|) over the other three edges
+                    const float e01 = mag[0] + mag[1], e23 = mag[2] + mag[3];
+                    ext[0] = mag[1] + e23;
+                    ext[1] = mag[0] + e23;
+                    ext[2] = e01 + mag[3];
+                    ext[3] = e01 + mag[2];
+                } else {
+                    // extrinsic D of each edge: the (+) of the other three deltas,
+                    // two (+) per packed f32x2 instruction pair (each lane equals
+                    // the scalar oplus; a (+) b and b (+) a round alike)
+                    const float2 d = oplus2(make_float2(mag[0], mag[2]), make_float2(mag[1], mag[3]));
+                    const float2 e01 = oplus2(make_float2(mag[1], mag[0]), make_float2(d.y, d.y));
+                    const float2 e23 = oplus2(make_float2(mag[3], mag[2]), make_float2(d.x, d.x));
+                    ext[0] = e01.x;
+                    ext[1] = e01.y;
+                    ext[2] = e23.x;
+                    ext[3] = e23.y;
+                }
 #pragma unroll
-                    for (int n = 0; n < 4; ++n) {
-                        // every incoming delta is at least delta_clip, so without
-                        // padding (FULL) the delta-form magnitude is at most
-                        // msg_clip already (up to rounding); padded edges read
-                        // delta = 0 and need the clip
-                        const float w0 = PhiForm<VARIANT>::value ? phi_check(ext[n]) : c2v_magnitude(ext[n]);
-                        const float wv = FULL && !PhiForm<VARIANT>::value ? w0 : fminf(w0, sp.clip2);
-                        const float mm = __uint_as_float(__float_as_uint(wv) ^ ((sgn ^ u[n]) & 0x80000000u));
-                        slots[FULL ? sl[n] : sl[n] == kZero ? kTrash : sl[n]] = mm;
-                        if (TRACE && a.tr_c2v && sl[n] != kZero)
-                            a.tr_c2v[((size_t)shot * sp.max_iter + (t - 1)) * a.E + a.chk_ptr[i] + n] = kLn2 * mm;
-                    }
+                for (int n = 0; n < 4; ++n) {
+                    // every incoming delta is at least delta_clip, so without
+                    // padding (FULL) the delta-form magnitude is at most
+                    // msg_clip already (up to rounding); padded edges read
+                    // delta = 0 and need the clip
+                    const float w0 = PHI ? phi_check(ext[n]) : c2v_magnitude(ext[n]);
+                    const float wv = FULL && !PHI ? w0 : fminf(w0, sp.clip2);
+                    const float mm = __uint_as_float(__float_as_uint(wv) ^ ((ux ^ u[n]) & 0x80000000u));
+                    if (FULL || sl[n] != kZero) slots[sl[n]] = mm;
+                    if (TRACE && a.tr_c2v && sl[n] != kZero)
+                        a.tr_c2v[((size_t)shot * sp.max_iter + (t - 1)) * a.E + a.chk_ptr[i] + n] = kLn2 * mm;
                 }
             }
         }
-        const int any = group_any(G, bar_id, (int)mismatch);
+        const int any = group_any(G, bar_id, (int)(do_check ? mismatch & 1u : 0u));
         if (do_check && !any) {
             conv = 1;
             iters = t - 1;
@@ -659,99 +689,106 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const ThreadAdj<
         }
 
         // ---- variable pass: posterior of the variant, decision, eq. (v_update)/(mombp5) ----
-#pragma unroll
-        for (int k = 0; k < NPT; ++k) {
+        dec = 0;
+#pragma unroll (NPT ? NPT : 1)
+        for (int k = 0; k < nk; ++k) {
             const int j = k * T + tg;
-            if (k < npt && j < N) {
-                const uint32_t vp = adj.info[k] >> 8;
-                float win[4], S[3];
-                if (SPLIT) {
-                    // positions 0, 1: X-type edges (anticommute with Z and Y);
-                    // 2, 3: Z-type edges (with X and Y); unused slots hold 0
+            if (j >= N) break;
+            const uint32_t vp = FULL ? 0xFFu : NPT ? own.vp[k] : vps[j];
+            float win[4], S[3];
+            if (SPLIT) {
+                // positions 0, 1: X-type edges (anticommute with Z and Y);
+                // 2, 3: Z-type edges (with X and Y); unused slots hold 0
 #pragma unroll
-                    for (int n = 0; n < 4; ++n) win[n] = slots[n * Np + j];
-                    const float2 s20 = __fadd2_rn(make_float2(win[0], win[2]), make_float2(win[1], win[3]));
-                    S[2] = s20.x;
-                    S[0] = s20.y;
-                    S[1] = S[0] + S[2];
-                } else {
-                    const float4 w4 = *reinterpret_cast<const float4 *>(slots + 4 * j);
-                    win[0] = w4.x;
-                    win[1] = w4.y;
-                    win[2] = w4.z;
-                    win[3] = w4.w;
-                    anticommuting_sums(vp, win, S[0], S[1], S[2]);
-                }
-                const float Pi[3] = {PiS[j], PiS[Np + j], PiS[2 * Np + j]};
-                float Q[3];
-                if (VARIANT == BPQ_EWAINIT) {
-                    // eq. (EWAInit): the state holds Pi^(t) (Pi^(0) at t = 1), so
-                    // Q^(t) = Pi^(t) + S and Pi^(t+1) = alpha Pi^(0) + (1-alpha) Q^(t);
-                    // Paulis X and Y share one f32x2 pair
-                    const float oma = 1.f - alpha;
-                    const float2 q01 = __fadd2_rn(make_float2(state[j], state[Np + j]), make_float2(S[0], S[1]));
-                    const float2 n01 = __ffma2_rn(make_float2(oma, oma), q01,
-                                                  make_float2(state[3 * Np + j], state[4 * Np + j]));
-                    Q[0] = q01.x;
-                    Q[1] = q01.y;
-                    Q[2] = state[2 * Np + j] + S[2];
-                    state[j] = n01.x;
-                    state[Np + j] = n01.y;
-                    state[2 * Np + j] = fmaf(oma, Q[2], state[5 * Np + j]);
-                } else {
-#pragma unroll
-                    for (int w = 0; w < 3; ++w) {
-                        if (VARIANT == BPQ_PLAIN) {
-                            Q[w] = Pi[w] + S[w];  // eq. (p_update)
-                        } else if (VARIANT == BPQ_MOMENTUM) {
-                            // eqs. (mombp1), (mombp2) with the gradient of (mombp3)
-                            const float qp = state[w * Np + j];
-                            const float g = momentum_g(sp, qp, Pi[w], S[w], state[(3 + w) * Np + j]);
-                            Q[w] = momentum_q(sp, qp, g);
-                            state[w * Np + j] = Q[w];
-                            state[(3 + w) * Np + j] = g;
-                        } else {
-                            // eq. (boost) from t = 2; G accumulates g'^2
-                            const float qp = state[w * Np + j];
-                            const float gp = adagrad_gp(qp, Pi[w], S[w]);
-                            const float Gs = adagrad_G(state[(3 + w) * Np + j], gp, t >= 2 || sp.ada_from1);
-                            Q[w] = t == 1 ? Pi[w] + S[w] : adagrad_q(sp, qp, gp, Gs);
-                            state[w * Np + j] = Q[w];
-                            state[(3 + w) * Np + j] = Gs;
-                        }
-                    }
-                }
-                // hard decision: I if all Q_W > 0, else the first minimum of X, Y, Z
-                // (the minimum is shared with emit_v2c's c0)
-                const float mq = fminf(Q[0], fminf(Q[1], Q[2]));
-                const uint32_t d = mq > 0.f ? 0u : Q[0] == mq ? 1u : Q[1] == mq ? 2u : 3u;
-                dk[k] = d;
-                // per-edge <E^_j, H_ij> for the next syndrome test (carried in the
-                // messages' least significant bits)
-                const uint32_t ab = SPLIT ? anti_bits_split(d) : anti_bytes(d, adj.pp[k]);
-                if (TRACE) {
-                    const size_t o = (size_t)shot * sp.max_iter + (t - 1);
-                    if (a.tr_Q) {
-                        a.tr_Q[(o * N + j) * 3 + 0] = kLn2 * Q[0];
-                        a.tr_Q[(o * N + j) * 3 + 1] = kLn2 * Q[1];
-                        a.tr_Q[(o * N + j) * 3 + 2] = kLn2 * Q[2];
-                    }
-                    if (a.tr_dec) a.tr_dec[o * N + j] = (uint8_t)d;
-                }
-                emit_v2c<TRACE, SPLIT, PhiForm<VARIANT>::value, false, FULL>(a, sp, slots, j, t, shot, vp, Q[0], Q[1],
-                                                                             Q[2], win, ab);
+                for (int n = 0; n < 4; ++n) win[n] = slots[n * Np + j];
+                const float2 s20 = __fadd2_rn(make_float2(win[0], win[2]), make_float2(win[1], win[3]));
+                S[2] = s20.x;
+                S[0] = s20.y;
+                S[1] = S[0] + S[2];
+            } else {
+                const float4 w4 = *reinterpret_cast<const float4 *>(slots + 4 * j);
+                win[0] = w4.x;
+                win[1] = w4.y;
+                win[2] = w4.z;
+                win[3] = w4.w;
+                anticommuting_sums(vp, win, S[0], S[1], S[2]);
             }
+            float Q[3];
+            if (VARIANT == BPQ_EWAINIT) {
+                // eq. (EWAInit): the state holds Pi^(t) (Pi^(0) at t = 1), so
+                // Q^(t) = Pi^(t) + S and Pi^(t+1) = alpha Pi^(0) + (1-alpha) Q^(t);
+                // Paulis X and Y share one f32x2 pair
+                const float oma = 1.f - alpha;
+                const float2 q01 = __fadd2_rn(make_float2(state[j], state[Np + j]), make_float2(S[0], S[1]));
+                const float2 n01 = __ffma2_rn(make_float2(oma, oma), q01,
+                                              make_float2(state[3 * Np + j], state[4 * Np + j]));
+                Q[0] = q01.x;
+                Q[1] = q01.y;
+                Q[2] = state[2 * Np + j] + S[2];
+                state[j] = n01.x;
+                state[Np + j] = n01.y;
+                state[2 * Np + j] = fmaf(oma, Q[2], state[5 * Np + j]);
+            } else {
+#pragma unroll
+                for (int w = 0; w < 3; ++w) {
+                    const float Pi = PiS[w * Np + j];
+                    if (VARIANT == BPQ_PLAIN) {
+                        Q[w] = Pi + S[w];  // eq. (p_update)
+                    } else if (VARIANT == BPQ_MOMENTUM) {
+                        // eqs. (mombp1), (mombp2) with the gradient of (mombp3)
+                        const float qp = state[w * Np + j];
+                        const float g = momentum_g(sp, qp, Pi, S[w], state[(3 + w) * Np + j]);
+                        Q[w] = momentum_q(sp, qp, g);
+                        state[w * Np + j] = Q[w];
+                        state[(3 + w) * Np + j] = g;
+                    } else {
+                        // eq. (boost) from t = 2; G accumulates g'^2
+                        const float qp = state[w * Np + j];
+                        const float gp = adagrad_gp(qp, Pi, S[w]);
+                        const float Gs = adagrad_G(state[(3 + w) * Np + j], gp, t >= 2 || sp.ada_from1);
+                        Q[w] = t == 1 ? Pi + S[w] : adagrad_q(sp, qp, gp, Gs);
+                        state[w * Np + j] = Q[w];
+                        state[(3 + w) * Np + j] = Gs;
+                    }
+                }
+            }
+            // hard decision: I if all Q_W > 0, else the first minimum of X, Y, Z
+            // (the minimum is shared with emit_v2c's c0); its per-edge
+            // <E^_j, H_ij> goes into the messages' least significant bits for the
+            // next syndrome test
+            const float mq = fminf(Q[0], fminf(Q[1], Q[2]));
+            uint32_t ab;
+            if (SPLIT) {
+                // anticommutes with X: Y or Z; with Z: X or Y
+                const bool some = !(mq > 0.f);
+                ab = (uint32_t)(some && Q[0] != mq) + 2u * (uint32_t)(some && (Q[0] == mq || Q[1] == mq));
+                dec = 4u * dec + ab;
+            } else {
+                const uint32_t d = mq > 0.f ? 0u : Q[0] == mq ? 1u : Q[1] == mq ? 2u : 3u;
+                dec = 4u * dec + d;
+                ab = anti_bytes(d, (vp & 3u) | ((vp & 0xCu) << 6) | ((vp & 0x30u) << 12) | ((vp & 0xC0u) << 18));
+            }
+            if (TRACE) {
+                const size_t o = (size_t)shot * sp.max_iter + (t - 1);
+                if (a.tr_Q) {
+                    a.tr_Q[(o * N + j) * 3 + 0] = kLn2 * Q[0];
+                    a.tr_Q[(o * N + j) * 3 + 1] = kLn2 * Q[1];
+                    a.tr_Q[(o * N + j) * 3 + 2] = kLn2 * Q[2];
+                }
+                if (a.tr_dec) a.tr_dec[o * N + j] = (uint8_t)decision_code<SPLIT>(dec & 3u);
+            }
+            emit_v2c<TRACE, SPLIT, PHI, false, FULL>(a, sp, slots, j, t, shot, vp, Q[0], Q[1], Q[2], win, ab);
         }
         group_sync(G, bar_id);
     }
 
     // ---- outputs ----
     if (!TRACE || a.est) {
-#pragma unroll
-        for (int k = 0; k < NPT; ++k) {
-            const int j = k * T + tg;
-            if (k < npt && j < N && BPQ_IN_BOUNDS((size_t)shot * N + j, (size_t)a.B * N, a.work + 1))
-                a.est[(size_t)shot * N + j] = (uint8_t)dk[k];
+        int sh = 2 * ((N - tg + T - 1) / T);
+        for (int j = tg; j < N; j += T) {
+            sh -= 2;
+            if (BPQ_IN_BOUNDS((size_t)shot * N + j, (size_t)a.B * N, a.work + 1))
+                a.est[(size_t)shot * N + j] = (uint8_t)decision_code<SPLIT>((dec >> sh) & 3u);
         }
     }
     if (tg == 0 && (!TRACE || a.conv) && BPQ_IN_BOUNDS(shot, a.B, a.work + 1)) {
@@ -764,7 +801,7 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const ThreadAdj<
 // One code per launch: a persistent grid; every shot group takes shots from
 // the global queue until the batch is exhausted.
 template <int VARIANT, int NPT, bool TRACE, bool SPLIT, bool FULL = false>
-__global__ void __launch_bounds__(NPT <= 2 ? 1024 : 512, 1) decode_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(1024, 1) decode_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem);
     int *grp_shot = reinterpret_cast<int *>(smem + 16);
@@ -781,11 +818,13 @@ __global__ void __launch_bounds__(NPT <= 2 ? 1024 : 512, 1) decode_kernel(const 
     // the launch's layout fits the dynamic shared memory (uniform across the
     // CTA, so an early return happens before any barrier)
     {
-        const size_t need = kSmemHeader + (size_t)a.table_bytes + (size_t)12 * a.n_pad +
+        const size_t need = kSmemHeader + (size_t)a.table_bytes + (size_t)12 * a.n_pad + a.init_bytes +
                             (size_t)(blockDim.x / T) * a.group_bytes;
         const bool ok = need <= dynamic_smem_bytes() && a.n_pad >= a.N && a.slots_floats >= 4u * a.n_pad + 2u &&
                         a.group_bytes >= 4u * (a.slots_floats + (uint32_t)StateArrays<VARIANT>::n * a.n_pad) &&
-                        (a.off_var_pauli + (uint32_t)a.N <= a.table_bytes);
+                        (a.off_var_pauli + (uint32_t)a.N <= a.table_bytes) &&
+                        (a.init_bytes == 0 || a.init_bytes >= 16u * (uint32_t)a.n_pad) &&
+                        (a.M > a.N ? a.M : a.N) <= kMaxLoopNodes * T;
         if (!ok) {
             if (tid == 0) atomicExch(a.work + 1, kBoundsError);
             return;
@@ -812,8 +851,11 @@ __global__ void __launch_bounds__(NPT <= 2 ? 1024 : 512, 1) decode_kernel(const 
         return;
     }
 
-    ThreadAdj<NPT> adj;
-    load_adjacency<NPT>(a, tab, T, tg, NPT, adj);
+    if (!FULL) prepare_table(a, tab);
+    load_init<VARIANT == BPQ_AEWA ? BPQ_EWAINIT : VARIANT, SPLIT, FULL>(a, m);
+    if (!FULL || a.init_bytes) __syncthreads();
+    Owned<NPT> own;
+    load_owned<NPT>(a, tab, T, tg, own);
 
     for (;;) {
         if (tg == 0) grp_shot[group] = (int)atomicAdd(a.work, 1u);
@@ -825,48 +867,56 @@ __global__ void __launch_bounds__(NPT <= 2 ? 1024 : 512, 1) decode_kernel(const 
             // a run converges (the outputs are those of the last run); alpha_k =
             // (10 - k) / 10 by IEEE division, the float nearest to it
             for (int k = 0; k <= 10; ++k)
-                if (decode_shot<BPQ_EWAINIT, NPT, TRACE, SPLIT, FULL>(a, adj, m, NPT, T, tg, G, bar_id, shot,
+                if (decode_shot<BPQ_EWAINIT, NPT, TRACE, SPLIT, FULL>(a, own, m, T, tg, G, bar_id, shot,
                                                                     (float)(10 - k) / 10.0f))
                     break;
         } else {
-            decode_shot<VARIANT, NPT, TRACE, SPLIT, FULL>(a, adj, m, NPT, T, tg, G, bar_id, shot, a.alpha);
+            decode_shot<VARIANT, NPT, TRACE, SPLIT, FULL>(a, own, m, T, tg, G, bar_id, shot, a.alpha);
         }
     }
 }
 
 // The shots of the current item taken by one shot group of the batched
 // kernel: the group takes the item's shots one by one from the item's
-// counter until none are left.  NPT, SPLIT and FULL are the item's nodes
-// per thread and table layout, so each item runs the decode_shot
-// specialisation that the one-code kernel runs for it.
+// counter until none are left.  SPLIT and FULL are the item's table layout, so
+// each item runs the decode_shot specialisation that the one-code kernel runs
+// for it.
 template <int VARIANT, int NPT, bool SPLIT, bool FULL>
-__device__ __forceinline__ void batch_item_shots(const DecodeArgs &a, const ThreadAdj<2> &adj2, const GroupMem &m,
-                                                 uint32_t *next, int *slot, int T, int tg, int G, int bar_id) {
-    ThreadAdj<NPT> adj;
-#pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-        adj.cs_lo[k] = adj2.cs_lo[k];
-        adj.cs_hi[k] = adj2.cs_hi[k];
-        adj.info[k] = adj2.info[k];
-        adj.pp[k] = adj2.pp[k];
-    }
+__device__ __forceinline__ void batch_item_shots(const DecodeArgs &a, const GroupMem &m, uint32_t *next, int *slot,
+                                                 int T, int tg, int G, int bar_id) {
+    Owned<NPT> own;
+    load_owned<NPT>(a, m.tab, T, tg, own);
     for (;;) {
         if (tg == 0) *slot = (int)atomicAdd(next, 1u);
         group_sync(G, bar_id);
         const int shot = *slot;
         if (shot >= a.B) break;
-        decode_shot<VARIANT, NPT, false, SPLIT, FULL>(a, adj, m, NPT, T, tg, G, bar_id, shot, a.alpha);
+        decode_shot<VARIANT, NPT, false, SPLIT, FULL>(a, own, m, T, tg, G, bar_id, shot, a.alpha);
     }
+}
+
+// The same for the item's table layout.
+template <int VARIANT, int NPT, bool GENERIC>
+__device__ __forceinline__ void batch_group_shots(const DecodeArgs &a, const GroupMem &m, uint32_t *next, int *slot,
+                                                  int T, int tg, int G, int bar_id) {
+    if (a.split == 2)
+        batch_item_shots<VARIANT, NPT, true, true>(a, m, next, slot, T, tg, G, bar_id);
+    else if (a.split == 1 || !GENERIC)
+        batch_item_shots<VARIANT, NPT, true, false>(a, m, next, slot, T, tg, G, bar_id);
+    else if (GENERIC)
+        batch_item_shots<VARIANT, NPT, false, false>(a, m, next, slot, T, tg, G, bar_id);
 }
 
 // Many codes in one launch.  A CTA of kBatchThreads works on one item (a
 // code's batch) at a time: it splits into that code's shot groups (T_g
-// threads each, one or two nodes per thread), which take the item's shots
-// until none are left; only then does the CTA synchronise, pick the next
-// item with shots left (scanning from its starting item) and re-stage that
-// code's adjacency (bulk TMA) and prior.  Every shot is decoded by the
-// decode_shot specialisation of decode_kernel for its code (nodes per
-// thread and layout), so results equal those of decode_kernel bit for bit.
+// threads each, one or two nodes per thread) and, where enough threads and
+// shared memory are left over, one smaller group with more nodes per thread
+// (rest_warps: planar d = 25, one group of 608 threads and one of 416); they take
+// the item's shots until none are left; only then does the CTA synchronise,
+// pick the next item with shots left (scanning from its starting item) and
+// re-stage that code's adjacency (bulk TMA) and prior.  Every shot is decoded by
+// the decode_shot specialisation of decode_kernel for its code's layout, so
+// results equal those of decode_kernel bit for bit.
 // GENERIC: items may use the generic table layout; without it every item
 // has the split layout, and the kernel holds only the split paths.
 template <int VARIANT, bool GENERIC>
@@ -887,7 +937,6 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_batch_kernel(const Ba
     int cur = -1;
     int from = b.start[blockIdx.x < (unsigned)kMaxBatchCtas ? blockIdx.x : 0];
     uint32_t phase = 0;
-    ThreadAdj<2> adj;
     for (;;) {
         if (tid == 0) {
             int pick = -1;
@@ -925,41 +974,29 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_batch_kernel(const Ba
                 mbar_wait_bounded(mbar, phase ^ 1u, 1u << 22);
                 return;
             }
-            const int T = desc->G * 32;
-            const int group = tid / T;
-            if (group < desc->groups_per_cta && tid - group * T == 0) {
-                const GroupMem m = group_mem(*desc, tab, group);
-                m.slots[4 * desc->n_pad] = 0.f;
+            if (desc->split != 2) prepare_table(*desc, tab);
+            {
+                const GroupMem m0 = group_mem(*desc, tab, 0);
+                if (tid < desc->groups_per_cta + (desc->rest_warps ? 1 : 0))
+                    group_mem(*desc, tab, tid).slots[4 * desc->n_pad] = 0.f;
+                if (desc->split)
+                    load_init<VARIANT, true, false>(*desc, m0);
+                else if (GENERIC)
+                    load_init<VARIANT, false, false>(*desc, m0);
             }
-            load_adjacency<2>(*desc, tab, T, tid - group * T, desc->npt, adj);
             __syncthreads();
             cur = g;
         }
         const DecodeArgs &a = *desc;
-        const int G = a.G, T = G * 32;
-        const int group = tid / T, tg = tid - group * T;
+        const int T = a.G * 32, group = tid / T;
         if (group < a.groups_per_cta) {
-            const GroupMem m = group_mem(a, tab, group);
-            const int bar_id = 1 + group;
-            uint32_t *next = b.work + 2 + g;
-            int *slot = grp_shot + group;
-            const bool one = a.npt == 1;
-            if (a.split == 2) {
-                if (one)
-                    batch_item_shots<VARIANT, 1, true, true>(a, adj, m, next, slot, T, tg, G, bar_id);
-                else
-                    batch_item_shots<VARIANT, 2, true, true>(a, adj, m, next, slot, T, tg, G, bar_id);
-            } else if (a.split == 1 || !GENERIC) {
-                if (one)
-                    batch_item_shots<VARIANT, 1, true, false>(a, adj, m, next, slot, T, tg, G, bar_id);
-                else
-                    batch_item_shots<VARIANT, 2, true, false>(a, adj, m, next, slot, T, tg, G, bar_id);
-            } else if (GENERIC) {
-                if (one)
-                    batch_item_shots<VARIANT, 1, false, false>(a, adj, m, next, slot, T, tg, G, bar_id);
-                else
-                    batch_item_shots<VARIANT, 2, false, false>(a, adj, m, next, slot, T, tg, G, bar_id);
-            }
+            batch_group_shots<VARIANT, 2, GENERIC>(a, group_mem(a, tab, group), b.work + 2 + g, grp_shot + group, T,
+                                                   tid - group * T, a.G, 1 + group);
+        } else if (a.rest_warps) {
+            const int rest = a.groups_per_cta, tg = tid - rest * T;
+            if (tg < 32 * a.rest_warps)
+                batch_group_shots<VARIANT, 0, GENERIC>(a, group_mem(a, tab, rest), b.work + 2 + g, grp_shot + rest,
+                                                       32 * a.rest_warps, tg, a.rest_warps, 1 + rest);
         }
         __syncthreads();
     }
@@ -967,40 +1004,27 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_batch_kernel(const Ba
 
 }  // namespace dk
 
-// AEWA-BP: single-code, non-trace kernels only.
+// Instantiate the kernels of one variant and return the one for npt nodes per
+// thread (above two, and traces: read from the table), trace and split layout.
+#define BPQ_DEFINE_PICK(NAME, V)                                                         \
+    DecodeKernelFn NAME(int npt, bool trace, bool split) {                               \
+        if (trace) return split ? dk::decode_kernel<V, 0, true, true> : dk::decode_kernel<V, 0, true, false>; \
+        switch (npt) {                                                                   \
+            case 1: return split ? dk::decode_kernel<V, 1, false, true> : dk::decode_kernel<V, 1, false, false>; \
+            case 2: return split ? dk::decode_kernel<V, 2, false, true> : dk::decode_kernel<V, 2, false, false>; \
+            default: return split ? dk::decode_kernel<V, 0, false, true> : dk::decode_kernel<V, 0, false, false>; \
+        }                                                                                \
+    }
+
+// AEWA-BP: non-trace kernels only.
 #define BPQ_DEFINE_PICK_AEWA(NAME)                                                       \
     DecodeKernelFn NAME(int npt, bool trace, bool split) {                               \
         if (trace) return nullptr;                                                       \
         switch (npt) {                                                                   \
-            case 1: return split ? dk::decode_kernel<BPQ_AEWA, 1, false, true>             \
-                               : dk::decode_kernel<BPQ_AEWA, 1, false, false>;           \
-            case 2: return split ? dk::decode_kernel<BPQ_AEWA, 2, false, true>             \
-                               : dk::decode_kernel<BPQ_AEWA, 2, false, false>;           \
-            case 3: return split ? dk::decode_kernel<BPQ_AEWA, 3, false, true>             \
-                               : dk::decode_kernel<BPQ_AEWA, 3, false, false>;           \
-            case 4: return split ? dk::decode_kernel<BPQ_AEWA, 4, false, true>             \
-                               : dk::decode_kernel<BPQ_AEWA, 4, false, false>;           \
+            case 1: return split ? dk::decode_kernel<BPQ_AEWA, 1, false, true> : dk::decode_kernel<BPQ_AEWA, 1, false, false>; \
+            case 2: return split ? dk::decode_kernel<BPQ_AEWA, 2, false, true> : dk::decode_kernel<BPQ_AEWA, 2, false, false>; \
+            default: return split ? dk::decode_kernel<BPQ_AEWA, 0, false, true> : dk::decode_kernel<BPQ_AEWA, 0, false, false>; \
         }                                                                                \
-        return nullptr;                                                                  \
-    }
-
-// Instantiate the kernels of one variant and return the one for (NPT,
-// trace, split layout).
-#define BPQ_PICK_NPT(V, NPT, TR)                                                         \
-    (split ? dk::decode_kernel<V, NPT, TR, true> : dk::decode_kernel<V, NPT, TR, false>)
-#define BPQ_DEFINE_PICK(NAME, V)                                                         \
-    DecodeKernelFn NAME(int npt, bool trace, bool split) {                               \
-        switch (npt * 2 + (trace ? 1 : 0)) {                                             \
-            case 2: return BPQ_PICK_NPT(V, 1, false);                                    \
-            case 3: return BPQ_PICK_NPT(V, 1, true);                                     \
-            case 4: return BPQ_PICK_NPT(V, 2, false);                                    \
-            case 5: return BPQ_PICK_NPT(V, 2, true);                                     \
-            case 6: return BPQ_PICK_NPT(V, 3, false);                                    \
-            case 7: return BPQ_PICK_NPT(V, 3, true);                                     \
-            case 8: return BPQ_PICK_NPT(V, 4, false);                                    \
-            case 9: return BPQ_PICK_NPT(V, 4, true);                                     \
-        }                                                                                \
-        return nullptr;                                                                  \
     }
 
 // The batched kernel of one variant (instantiated in a translation unit of
@@ -1018,10 +1042,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_batch_kernel(const Ba
         switch (npt) {                                                                   \
             case 1: return dk::decode_kernel<V, 1, false, true, true>;                   \
             case 2: return dk::decode_kernel<V, 2, false, true, true>;                   \
-            case 3: return dk::decode_kernel<V, 3, false, true, true>;                   \
-            case 4: return dk::decode_kernel<V, 4, false, true, true>;                   \
+            default: return dk::decode_kernel<V, 0, false, true, true>;                  \
         }                                                                                \
-        return nullptr;                                                                  \
     }
 
 }  // namespace bpq

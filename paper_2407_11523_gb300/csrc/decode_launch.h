@@ -39,8 +39,10 @@ struct DecodeArgs {
     int ada_from1;
     int split;                 // 0: generic layout; 1: split layout (bpq_tanner::split);
                                // 2: split layout with every slot used (bpq_tanner::full)
+    uint32_t init_bytes;       // shared memory of the initial messages: 16 n_pad, or 0 (computed per shot)
     // used by the batched kernel only
-    int npt, groups_per_cta;
+    int groups_per_cta;
+    int rest_warps;            // warps of the extra group of the threads left over (0: none)
 };
 
 constexpr uint32_t kDescBytes = (sizeof(DecodeArgs) + 15) & ~15u;  // descriptor copy in shared memory
@@ -66,6 +68,7 @@ struct LaunchShape {
     int n_pad;
     uint32_t slots_floats, group_bytes;
     size_t smem;
+    uint32_t init_bytes = 0;  // DecodeArgs::init_bytes
     bool one = false;  // two shots per thread: the kernel for one shot group per CTA
 };
 
@@ -73,9 +76,9 @@ using DecodeKernelFn = void (*)(const DecodeArgs);
 using BatchKernelFn = void (*)(const BatchArgs);
 using SmallKernelFn = void (*)(const DecodeArgs, int runs, float clip);
 
-// Kernels of one variant, for nodes per thread npt in [1, 4]; split selects the
-// specialisation for tables in the split layout, and the _full functions the
-// non-trace kernels for split tables without padding.
+// Kernels of one variant for npt nodes per thread; split selects the specialisation for tables in the
+// split layout, and the _full functions the non-trace kernels for split tables
+// without padding.
 DecodeKernelFn pick_plain(int npt, bool trace, bool split);
 DecodeKernelFn pick_plain_full(int npt);
 DecodeKernelFn pick_momentum(int npt, bool trace, bool split);
@@ -143,8 +146,9 @@ __host__ __device__ inline PairOffsets pair_offsets(int variant, bool one, int M
     return o;
 }
 // Automatic choice of two shots per thread: from this many shots of the batch
-// per resident one-shot group (T: threads of a pair group).
-constexpr long pair_shots_per_group(int T) { return T == 32 ? 192 : 40; }
+// per resident one-shot group (T: threads of a pair group); measured in
+// decode_launch.
+constexpr long pair_shots_per_group(int T) { return T == 32 ? 256 : 80; }
 // Shape of a code inside the batched kernel (CTAs of kBatchThreads threads).
 int decode_batch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 

@@ -75,7 +75,7 @@ __device__ __forceinline__ void st_release_sys(uint32_t *p, uint32_t v) {
     asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <int VARIANT, int NPT>
+template <int VARIANT>
 __global__ void __launch_bounds__(kBatchThreads, 1) decode_serve_kernel(const ServeArgs s) {
     extern __shared__ __align__(16) uint8_t smem[];
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem);
@@ -100,13 +100,13 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_serve_kernel(const Se
     __shared__ uint4 grp_dst[kMaxGroupsPerCta];
     if (tid == 0) cl_lock = cl_base = cl_cnt = 0;
     int cur = -1;
+    Owned<2> own = {};
     // the CTA's home code: every scan for a code with requests starts there,
     // so that the CTAs spread over the codes with requests instead of all
     // taking the first one published and then moving through the codes in
     // the same order
     const int from = (int)(blockIdx.x % (unsigned)s.ncodes);
     uint32_t phase = 0, idle = 0;
-    ThreadAdj<NPT> adj;
     for (;;) {
         // ---- pick a code with published, unclaimed requests: warp 0 reads
         // the codes' counts in parallel (one code per lane, from `from` on) ----
@@ -182,14 +182,13 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_serve_kernel(const Se
                 mbar_wait_bounded(mbar, phase ^ 1u, 1u << 22);
                 return;
             }
-            const int T = desc->G * 32;
-            const int group = tid / T;
-            if (group < desc->groups_per_cta && tid - group * T == 0) {
-                const GroupMem m = group_mem(*desc, tab, group);
-                m.slots[4 * desc->n_pad] = 0.f;
-            }
-            load_adjacency<NPT>(*desc, tab, T, tid - group * T, desc->npt, adj);
+            if (desc->split != 2) prepare_table(*desc, tab);
+            if (tid < desc->groups_per_cta) group_mem(*desc, tab, tid).slots[4 * desc->n_pad] = 0.f;
             __syncthreads();
+            {
+                const int T = desc->G * 32;
+                load_owned<2>(*desc, tab, T, tid % T, own);
+            }
             cur = g;
         }
         const DecodeArgs &a = *desc;
@@ -294,11 +293,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) decode_serve_kernel(const Se
                 // the next request even while this one decodes
                 if (tg == 0 && s.out->est) st_release_sys(s.consumed + (size_t)g * cap + slot, (uint32_t)k + 1u);
                 if (a.split)
-                    decode_shot<VARIANT, NPT, false, true, false, true>(a, adj, m, a.npt, T, tg, G, bar_id, group,
-                                                                         a.alpha);
+                    decode_shot<VARIANT, 2, false, true, false, true>(a, own, m, T, tg, G, bar_id, group, a.alpha);
                 else
-                    decode_shot<VARIANT, NPT, false, false, false, true>(a, adj, m, a.npt, T, tg, G, bar_id, group,
-                                                                          a.alpha);
+                    decode_shot<VARIANT, 2, false, false, false, true>(a, own, m, T, tg, G, bar_id, group, a.alpha);
                 group_sync(G, bar_id);
                 // warp 0 alone writes to host memory: the estimate (decode_shot
                 // wrote it at est + group * N) in 16-byte stores, to the request's

@@ -7,10 +7,10 @@ namespace bpq {
 
 ServeKernelFn pick_serve_kernel(int variant) {
     switch (variant) {
-        case BPQ_PLAIN: return dk::decode_serve_kernel<BPQ_PLAIN, 2>;
-        case BPQ_MOMENTUM: return dk::decode_serve_kernel<BPQ_MOMENTUM, 2>;
-        case BPQ_ADAGRAD: return dk::decode_serve_kernel<BPQ_ADAGRAD, 2>;
-        case BPQ_EWAINIT: return dk::decode_serve_kernel<BPQ_EWAINIT, 2>;
+        case BPQ_PLAIN: return dk::decode_serve_kernel<BPQ_PLAIN>;
+        case BPQ_MOMENTUM: return dk::decode_serve_kernel<BPQ_MOMENTUM>;
+        case BPQ_ADAGRAD: return dk::decode_serve_kernel<BPQ_ADAGRAD>;
+        case BPQ_EWAINIT: return dk::decode_serve_kernel<BPQ_EWAINIT>;
     }
     return nullptr;
 }

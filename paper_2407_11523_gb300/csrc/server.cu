@@ -430,7 +430,6 @@ int bpq_server_create(const bpq_tanner *const *codes, const float *const *priors
     s->max_iter = max_iter;
     s->max_batch = max_batch;
     int rc = BPQ_OK;
-    int npt_max = 1;
     bool generic = false;  // some code uses the generic table layout
     for (int c = 0; c < n_codes && !rc; ++c) {
         const bpq_tanner *t = codes[c];
@@ -454,9 +453,7 @@ int bpq_server_create(const bpq_tanner *const *codes, const float *const *priors
         a.n_pad = sh.n_pad;
         a.slots_floats = sh.slots_floats;
         a.group_bytes = sh.group_bytes;
-        a.npt = sh.npt;
         a.groups_per_cta = gpc;
-        npt_max = std::max(npt_max, sh.npt);
         generic = generic || a.split == 0;
         s->smem = std::max(s->smem, sh.smem);
         s->codes.push_back(t);
@@ -695,7 +692,6 @@ int bpq_server_create_slots(const bpq_tanner *const *codes, const float *const *
         a.n_pad = sh.n_pad;
         a.slots_floats = sh.slots_floats;
         a.group_bytes = sh.group_bytes;
-        a.npt = sh.npt;
         a.groups_per_cta = sh.groups_per_cta;
         a.B = slots_per_code;
         s->smem = std::max(s->smem, sh.smem);
