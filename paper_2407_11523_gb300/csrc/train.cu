@@ -366,7 +366,11 @@ __device__ __forceinline__ uint32_t true_logical_parities(const TrainArgs &a, co
     return tau;
 }
 
-__device__ __forceinline__ float neg_log(float P) { return -logf(fmaxf(P, kMinProb)); }
+// -log P of one side of a parity distribution; the likely side's from the other,
+// so that a small loss keeps its relative accuracy.
+__device__ __forceinline__ float neg_log(float P, float other) {
+    return P > other ? -log1pf(-other) : -logf(fmaxf(P, kMinProb));
+}
 
 // Forward: one CTA per shot.  Per iteration two barriers: the check threads
 // (which also take the coset loss's check terms of the previous iteration), the
@@ -401,12 +405,12 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
 #pragma unroll
         for (int n = 0; n < 4; ++n)
             if (d.sl[n] != kNoSlot) eo = parity_combine(eo, ub[d.sl[n]]);
-        loss += neg_log(d.sigma < 0.f ? eo.y : eo.x);
+        loss += d.sigma < 0.f ? neg_log(eo.y, eo.x) : neg_log(eo.x, eo.y);
     };
     auto logical_terms = [&](int l0, int n) {
         if (x < n) {
             const float4 t = logical_total<false>(part, x, n, warps);
-            loss_log += neg_log(((tau >> (l0 + x)) & 1u) ? t.y : t.x);
+            loss_log += ((tau >> (l0 + x)) & 1u) ? neg_log(t.y, t.x) : neg_log(t.x, t.y);
         }
     };
     __syncthreads();
@@ -472,13 +476,24 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
         logical_terms(a.n_log - ((a.n_log - 1) % chunk + 1), (a.n_log - 1) % chunk + 1);
         loss = (loss / (float)a.M + loss_log / (float)a.n_log) / (float)a.T;
     } else if (qubit) {
-        // cross-entropy of the final posterior against the true error
+        // cross-entropy of the final posterior against the true error; the
+        // largest term enters through log1p, so that a small loss keeps its
+        // relative accuracy
         const float z[4] = {0.f, -Q[0], -Q[1], -Q[2]};
-        const float zm = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
-        float se = 0.f;
-        for (int k = 0; k < 4; ++k) se += expf(z[k] - zm);
+        int top = 0;
+        float zm = z[0];
+#pragma unroll
+        for (int k = 1; k < 4; ++k)
+            if (z[k] > zm) {
+                zm = z[k];
+                top = k;
+            }
+        float rest = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k != top) rest += expf(z[k] - zm);
         const int e = a.err[(size_t)shot * a.N + x];
-        loss = zm + logf(se) - z[e];
+        loss = (e == 0 ? zm : zm + Q[e == 1 ? 0 : e == 2 ? 1 : 2]) + log1pf(rest);
     }
     if (qubit && a.Q_out)
         for (int w = 0; w < 3; ++w) a.Q_out[((size_t)shot * a.N + x) * 3 + w] = Q[w];
