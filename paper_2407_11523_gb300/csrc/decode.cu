@@ -26,13 +26,13 @@ DecodeKernelFn pick(int variant, int npt, bool trace, int layout) {
     return nullptr;
 }
 
-DecodeKernelFn pick_pair(int variant, bool one, int layout) {
+DecodeKernelFn pick_pair(int variant, int mode, int layout) {
     const bool full = layout == 2;
     switch (variant) {
-        case BPQ_PLAIN: return full ? pick_plain_pair_full(one) : pick_plain_pair(one);
-        case BPQ_MOMENTUM: return full ? pick_momentum_pair_full(one) : pick_momentum_pair(one);
-        case BPQ_ADAGRAD: return full ? pick_adagrad_pair_full(one) : pick_adagrad_pair(one);
-        case BPQ_EWAINIT: return full ? pick_ewainit_pair_full(one) : pick_ewainit_pair(one);
+        case BPQ_PLAIN: return full ? pick_plain_pair_full(mode) : pick_plain_pair(mode);
+        case BPQ_MOMENTUM: return full ? pick_momentum_pair_full(mode) : pick_momentum_pair(mode);
+        case BPQ_ADAGRAD: return full ? pick_adagrad_pair_full(mode) : pick_adagrad_pair(mode);
+        case BPQ_EWAINIT: return full ? pick_ewainit_pair_full(mode) : pick_ewainit_pair(mode);
     }
     return nullptr;
 }
@@ -91,9 +91,13 @@ int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     s->n_pad = n_pad;
     s->slots_floats = slots;
     s->group_bytes = (uint32_t)group_bytes;
-    s->one = gpc == 1 && one_smem <= 227 * 1024;
-    s->smem = s->one ? one_smem
-                     : pair_offsets(variant, false, t->M, n_pad).groups + (size_t)gpc * group_bytes;
+    // one-warp groups too take the table of byte offsets, and have their size
+    // at compile time (planar d = 5, 10^6 shots, plain 4.68 -> 4.34 ms; d = 7,
+    // 500000 shots, Momentum 5.82 -> 5.53, EWAInit 1.82 -> 1.75)
+    const size_t wide = one_smem + (size_t)(gpc - 1) * group_bytes;
+    s->pair_mode = wide > 227 * 1024 ? kPairGroups : gpc == 1 ? kPairOne : T == 32 ? kPairWarps : kPairGroups;
+    s->smem = s->pair_mode != kPairGroups
+                  ? wide : pair_offsets(variant, false, t->M, n_pad).groups + (size_t)gpc * group_bytes;
     if (s->smem > 227 * 1024) return fail(BPQ_EINVAL, "shared memory of the launch shape exceeds 227 KB");
     return BPQ_OK;
 }
@@ -248,15 +252,19 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // batch's tail (its slowest shots) runs longer; pairing pays only
         // once each resident one-shot group would decode many shots.
         // Measured on GB300, one shot per thread against two (ms; shots per
-        // resident one-shot group): toric d = 15 EWAInit, p = 0.06, 20000 (33)
-        // 0.877 / 0.923, p = 0.08, 40000 (66) 2.41 / 2.36; planar d = 13
-        // EWAInit 50000 (55) 1.40 / 1.44, 100000 (110) 2.71 / 2.73; planar
-        // d = 9 EWAInit 100000 (66) 0.914 / 0.952, plain 120000 (79) 2.79 /
-        // 2.73; planar d = 11 plain 100000 (82) 4.22 / 4.12; planar d = 25
-        // plain 10000 (66) 6.00 / 5.97.  The crossing lies between 60 and 110.
-        // One-warp pair groups have the longest tail: planar d = 7 EWAInit
-        // 300000 (123) 0.957 / 1.011, 600000 (247) 1.843 / 1.844, 10^6 (411)
-        // 3.04 / 2.93; AdaGrad on xzzx d = 7 200000 (82) 1.08 / 1.30.
+        // resident one-shot group).  Plain and Momentum BP, whose shots mostly
+        // run long, cross early: planar d = 9 plain 60000 (39) 1.43 / 1.45, 120000
+        // (79) 2.79 / 2.73; planar d = 11 plain 100000 (82) 4.22 / 4.12; planar
+        // d = 25 plain 10000 (66) 6.00 / 5.97; one-warp pair groups: planar d = 7
+        // Momentum 500000 (205) 6.39 / 5.53, d = 5 10^6 (205) 5.14 / 5.02.  EWAInit
+        // and AdaGrad converge in few iterations, so that the slowest shots weigh
+        // more: planar d = 11 EWAInit 100000 (82) 1.50 / 1.56, d = 13 100000 (110)
+        // 2.71 / 2.73, d = 9 200000 (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38;
+        // planar d = 7 300000 (123) 0.957 / 1.011, 500000 (205) 1.85 / 1.75; large
+        // codes again earlier: toric d = 15, p = 0.08, 40000 (66) 2.41 / 2.36,
+        // p = 0.06, 20000 (33) 0.877 / 0.923.  A code whose one-shot group is one
+        // warp too gains nothing for them: planar d = 5 EWAInit 10^6 (205) 1.48 /
+        // 1.60, AdaGrad 5.74 / 5.84.
         LaunchShape one;
         int per_sm = 0;
         DecodeKernelFn f1 = nullptr;
@@ -265,19 +273,19 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
             decode_pair_shape(t, variant, &s) == BPQ_OK &&
-            (long)a.B < pair_shots_per_group(s.T) * (long)per_sm * t->num_sms * one.groups_per_cta)
+            (long)a.B < pair_shots_per_group(variant, s.T, one.T) * (long)per_sm * t->num_sms * one.groups_per_cta)
             pairs = false;
     }
     int rc = pairs ? decode_pair_shape(t, variant, &s) : decode_launch_shape(t, variant, &s);
     if (rc) return rc;
     DecodeKernelFn fn = nullptr;
     if (t->debug_checks) {
-        fn = trace ? nullptr : pick_debug(variant, s.npt, pairs, s.one, a.split);
+        fn = trace ? nullptr : pick_debug(variant, s.npt, pairs, s.pair_mode, a.split);
         if (!fn)
             return fail(BPQ_EINVAL, "no bounds-checked kernel for this launch (plain, Momentum, AdaGrad or EWAInit BP, "
                                     "at most two nodes per thread, not a trace)");
     } else {
-        fn = pairs ? pick_pair(variant, s.one, a.split) : pick(variant, s.npt, trace, a.split);
+        fn = pairs ? pick_pair(variant, s.pair_mode, a.split) : pick(variant, s.npt, trace, a.split);
     }
     if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant (AEWA-BP has no trace mode)");
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
@@ -292,7 +300,7 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         if (rc) return rc;
         s.smem -= s.init_bytes;  // too few shots per group to repay the table
         s.init_bytes = 0;
-        fn = t->debug_checks ? pick_debug(variant, s.npt, false, false, a.split) : pick(variant, s.npt, false, a.split);
+        fn = t->debug_checks ? pick_debug(variant, s.npt, false, 0, a.split) : pick(variant, s.npt, false, a.split);
         if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant");
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
         if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));

@@ -21,24 +21,27 @@ DecodeKernelFn pick_debug_one(int layout) {
     }
 }
 
+template <int V, bool FULL>
+DecodeKernelFn pick_debug_pair(int mode) {
+    return mode == kPairOne     ? dk_debug::decode_pair_kernel<V, FULL, kPairOne>
+           : mode == kPairWarps ? dk_debug::decode_pair_kernel<V, FULL, kPairWarps>
+                                : dk_debug::decode_pair_kernel<V, FULL, kPairGroups>;
+}
+
 template <int V>
-DecodeKernelFn pick_debug_v(int npt, bool pairs, bool one, int layout) {
-    if (pairs) {
-        if (layout == 2) return one ? dk_debug::decode_pair_kernel<V, true, true> : dk_debug::decode_pair_kernel<V, true, false>;
-        if (layout == 1) return one ? dk_debug::decode_pair_kernel<V, false, true> : dk_debug::decode_pair_kernel<V, false, false>;
-        return nullptr;
-    }
+DecodeKernelFn pick_debug_v(int npt, bool pairs, int mode, int layout) {
+    if (pairs) return layout == 2 ? pick_debug_pair<V, true>(mode) : layout == 1 ? pick_debug_pair<V, false>(mode) : nullptr;
     return npt == 1 ? pick_debug_one<V, 1>(layout) : npt == 2 ? pick_debug_one<V, 2>(layout) : nullptr;
 }
 
 }  // namespace
 
-DecodeKernelFn pick_debug(int variant, int npt, bool pairs, bool one, int layout) {
+DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int mode, int layout) {
     switch (variant) {
-        case BPQ_PLAIN: return pick_debug_v<BPQ_PLAIN>(npt, pairs, one, layout);
-        case BPQ_MOMENTUM: return pick_debug_v<BPQ_MOMENTUM>(npt, pairs, one, layout);
-        case BPQ_ADAGRAD: return pick_debug_v<BPQ_ADAGRAD>(npt, pairs, one, layout);
-        case BPQ_EWAINIT: return pick_debug_v<BPQ_EWAINIT>(npt, pairs, one, layout);
+        case BPQ_PLAIN: return pick_debug_v<BPQ_PLAIN>(npt, pairs, mode, layout);
+        case BPQ_MOMENTUM: return pick_debug_v<BPQ_MOMENTUM>(npt, pairs, mode, layout);
+        case BPQ_ADAGRAD: return pick_debug_v<BPQ_ADAGRAD>(npt, pairs, mode, layout);
+        case BPQ_EWAINIT: return pick_debug_v<BPQ_EWAINIT>(npt, pairs, mode, layout);
     }
     return nullptr;
 }

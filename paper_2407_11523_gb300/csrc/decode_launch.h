@@ -69,7 +69,7 @@ struct LaunchShape {
     uint32_t slots_floats, group_bytes;
     size_t smem;
     uint32_t init_bytes = 0;  // DecodeArgs::init_bytes
-    bool one = false;  // two shots per thread: the kernel for one shot group per CTA
+    int pair_mode = 0;  // two shots per thread: PairMode
 };
 
 using DecodeKernelFn = void (*)(const DecodeArgs);
@@ -97,14 +97,14 @@ BatchKernelFn pick_adagrad_batch(bool generic);
 BatchKernelFn pick_ewainit_batch(bool generic);
 // Two shots per thread (decode_pair.cuh), split tables; one: one shot group
 // per CTA; the _full functions for split tables without padding.
-DecodeKernelFn pick_plain_pair(bool one);
-DecodeKernelFn pick_plain_pair_full(bool one);
-DecodeKernelFn pick_momentum_pair(bool one);
-DecodeKernelFn pick_momentum_pair_full(bool one);
-DecodeKernelFn pick_adagrad_pair(bool one);
-DecodeKernelFn pick_adagrad_pair_full(bool one);
-DecodeKernelFn pick_ewainit_pair(bool one);
-DecodeKernelFn pick_ewainit_pair_full(bool one);
+DecodeKernelFn pick_plain_pair(int mode);
+DecodeKernelFn pick_plain_pair_full(int mode);
+DecodeKernelFn pick_momentum_pair(int mode);
+DecodeKernelFn pick_momentum_pair_full(int mode);
+DecodeKernelFn pick_adagrad_pair(int mode);
+DecodeKernelFn pick_adagrad_pair_full(int mode);
+DecodeKernelFn pick_ewainit_pair(int mode);
+DecodeKernelFn pick_ewainit_pair_full(int mode);
 
 // One CTA per shot, `lanes` (1, 2 or 4) lanes per node (decode_small.cu), split
 // tables, every variant.  runs: 11 for AEWA-BP, else 1; clip: the bound of the
@@ -113,9 +113,9 @@ DecodeKernelFn pick_ewainit_pair_full(bool one);
 SmallKernelFn pick_small(int variant, int lanes);
 
 // Bounds-checked kernels (decode_debug.cu; bpq_set_debug_checks): npt in
-// {1, 2} with one shot per thread, pairs on split layouts (one: one shot
-// group per CTA); nullptr where none is compiled.
-DecodeKernelFn pick_debug(int variant, int npt, bool pairs, bool one, int layout);
+// {1, 2} with one shot per thread, pairs on split layouts (mode: PairMode);
+// nullptr where none is compiled.
+DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int mode, int layout);
 
 int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 // Whether bpq_decode runs the two-shots-per-thread kernel for this graph and
@@ -136,19 +136,25 @@ constexpr uint32_t kPairVoteBytes = 16;
 struct PairOffsets {
     uint32_t idx, used, prior, init, groups;
 };
-__host__ __device__ inline PairOffsets pair_offsets(int variant, bool one, int M, int n_pad) {
+// Ways to run two shots per thread: shot groups of any size (16-bit slot
+// table), one group per CTA, one-warp groups.
+enum PairMode { kPairGroups = 0, kPairOne = 1, kPairWarps = 2 };
+__host__ __device__ inline PairOffsets pair_offsets(int variant, bool wide, int M, int n_pad) {
     PairOffsets o;
     o.idx = kSmemHeader;
-    o.used = o.idx + (one ? 16u : 8u) * (uint32_t)((M + 1) & ~1);
+    o.used = o.idx + (wide ? 16u : 8u) * (uint32_t)((M + 1) & ~1);
     o.prior = o.used + (((uint32_t)n_pad + 15u) & ~15u);
     o.init = o.prior + 12u * (uint32_t)(pair_prior_copies(variant) * n_pad);
     o.groups = o.init + 16u * (uint32_t)n_pad;
     return o;
 }
 // Automatic choice of two shots per thread: from this many shots of the batch
-// per resident one-shot group (T: threads of a pair group); measured in
-// decode_launch.
-constexpr long pair_shots_per_group(int T) { return T == 32 ? 256 : 80; }
+// per resident one-shot group (T: threads of a pair group, one_T: of a one-shot
+// group); measured in decode_launch.
+constexpr long pair_shots_per_group(int variant, int T, int one_T) {
+    if (variant == BPQ_PLAIN || variant == BPQ_MOMENTUM) return T == 32 ? 128 : 64;
+    return T > 160 ? 64 : one_T > 32 ? 200 : 2000;
+}
 // Shape of a code inside the batched kernel (CTAs of kBatchThreads threads).
 int decode_batch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 

@@ -23,12 +23,13 @@
 // 8, measured) of the 405 that pass; HBM traffic is negligible.  So the kernel
 // spends shared memory to save instructions and registers:
 //  * the slot addresses of a check are read from a per-CTA table of byte
-//    offsets (one 128-bit load, no unpacking; ONE, one shot group per CTA) in
+//    offsets (one 128-bit load, no unpacking; one shot group per CTA, or
+//    one-warp groups) in
 //    place of packed indices in registers.  That also frees the registers that
 //    tied a thread to two nodes: a thread loops over any number of nodes, so
 //    large codes can take small groups, more of which fit an SM.
-//    With several groups per CTA (ONE = false) the table holds 16-bit slot
-//    indices, which fits larger codes and adds the group's base per edge.
+//    With several larger groups per CTA (kPairGroups) the table holds 16-bit
+//    slot indices, half the size, for codes that the other would not fit.
 //  * a syndrome bit enters as one word whose bits 31 (sign) and 0 (parity)
 //    are both the bit; a register per lane is rotated from check to check.
 //  * the decision is kept as its two anticommutation bits, which the messages
@@ -99,15 +100,15 @@ struct PairMem {
     float2 *state;
 };
 
-template <int VARIANT, bool ONE>
+template <int VARIANT, int MODE>
 __device__ __forceinline__ PairMem pair_mem(const DecodeArgs &a, uint8_t *smem, int group) {
     PairMem m;
-    const PairOffsets o = pair_offsets(VARIANT, ONE, a.M, a.n_pad);
+    const PairOffsets o = pair_offsets(VARIANT, MODE != kPairGroups, a.M, a.n_pad);
     m.idx = smem + o.idx;
     m.used = smem + o.used;
     m.PiS = reinterpret_cast<const float *>(smem + o.prior);
     m.init = reinterpret_cast<const float *>(smem + o.init);
-    uint8_t *g = smem + o.groups + (ONE ? 0u : (uint32_t)group * a.group_bytes);
+    uint8_t *g = smem + o.groups + (MODE == kPairOne ? 0u : (uint32_t)group * a.group_bytes);
     m.votes = reinterpret_cast<uint32_t *>(g);
     m.slots = g + kPairVoteBytes;
     m.state = reinterpret_cast<float2 *>(m.slots) + a.slots_floats;
@@ -115,18 +116,20 @@ __device__ __forceinline__ PairMem pair_mem(const DecodeArgs &a, uint8_t *smem, 
 }
 
 // Byte offsets (from the group's slots) of the four message slots of check i.
-template <bool ONE>
+template <int MODE>
 __device__ __forceinline__ uint4 pair_slots(const uint8_t *idx, int i) {
-    if (ONE) return reinterpret_cast<const uint4 *>(idx)[i];
+    if (MODE != kPairGroups) return reinterpret_cast<const uint4 *>(idx)[i];
     const uint2 s = reinterpret_cast<const uint2 *>(idx)[i];
     return make_uint4((s.x & 0xFFFFu) * 8u, (s.x >> 16) * 8u, (s.y & 0xFFFFu) * 8u, (s.y >> 16) * 8u);
 }
 
-// Barrier of the group: of the CTA when it holds one group.
-template <bool ONE>
+// Barrier of the group: of the CTA when it holds one group, of the warp.
+template <int MODE>
 __device__ __forceinline__ void pair_sync(int G, int bar_id) {
-    if (ONE)
+    if (MODE == kPairOne)
         __syncthreads();
+    else if (MODE == kPairWarps)
+        __syncwarp();
     else
         group_sync(G, bar_id);
 }
@@ -136,16 +139,16 @@ __device__ __forceinline__ void pair_sync(int G, int bar_id) {
 // warp-wide votes into the shared word votes_smem[parity] before the
 // barrier; the word of the other parity, read in the previous iteration, is
 // cleared before the next barrier so that the next iteration finds it zero.
-template <bool ONE>
+template <int MODE>
 __device__ __forceinline__ uint32_t group_any2(int G, int bar_id, uint32_t votes, uint32_t *votes_smem, int tg,
                                                uint32_t parity) {
     const uint32_t w = __reduce_or_sync(0xffffffffu, votes);
-    if (!ONE && G == 1) {
+    if (MODE == kPairWarps || (MODE == kPairGroups && G == 1)) {
         __syncwarp();
         return w;
     }
     if ((tg & 31) == 0 && w) atomicOr(votes_smem + parity, w);
-    pair_sync<ONE>(G, bar_id);
+    pair_sync<MODE>(G, bar_id);
     const uint32_t any = *reinterpret_cast<volatile uint32_t *>(votes_smem + parity);
     if (tg == 0) votes_smem[parity ^ 1u] = 0u;
     return any;
@@ -188,7 +191,7 @@ __device__ __forceinline__ void emit_v2c_pair(float vclip, float2 *slots, int Np
 // Decode shots two at a time with a group of G warps (thread tg of 32G)
 // until the queue is empty.  Each thread owns the nodes tg, tg + T, ... (at
 // most kPairMaxNodes).
-template <int VARIANT, bool FULL, bool ONE>
+template <int VARIANT, bool FULL, int MODE>
 __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem &m, int T, int tg, int G, int bar_id,
                                              int *grp_shot) {
     constexpr bool PHI = PhiForm<VARIANT>::value;
@@ -207,7 +210,7 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
         grp_shot[1] = (int)atomicAdd(a.work, 1u);
         m.votes[0] = m.votes[1] = 0u;
     }
-    pair_sync<ONE>(G, bar_id);
+    pair_sync<MODE>(G, bar_id);
     int shot[2] = {grp_shot[0], grp_shot[1]};
     int t[2] = {1, 1};
     // syndrome bits of the owned checks: that of the k-th is at bits 31 and 0
@@ -253,7 +256,7 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
     load_syndrome(0);
     load_syndrome(1);
     restart(3u);
-    pair_sync<ONE>(G, bar_id);
+    pair_sync<MODE>(G, bar_id);
 
     for (;;) {
         uint32_t mis0 = 0, mis1 = 0;  // bit 0: a check of the lane fails the syndrome test
@@ -261,7 +264,7 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
         // ---- check pass: syndrome tests of the lanes' previous decisions, then eq. (h_update) ----
 #pragma unroll 1
         for (int i = tg; i < M; i += T) {
-            const uint4 o4 = pair_slots<ONE>(m.idx, i);
+            const uint4 o4 = pair_slots<MODE>(m.idx, i);
             const uint32_t off[4] = {o4.x, o4.y, o4.z, o4.w};
             uint2 u[4];
 #pragma unroll
@@ -311,7 +314,7 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
         }
         // a lane's first check pass has no previous decision to test
         const uint32_t mismatch = (t[0] > 1 ? mis0 & 1u : 0u) | (t[1] > 1 ? (mis1 & 1u) << 1 : 0u);
-        const uint32_t any = group_any2<ONE>(G, bar_id, mismatch, m.votes, tg, parity);
+        const uint32_t any = group_any2<MODE>(G, bar_id, mismatch, m.votes, tg, parity);
         parity ^= 1u;
         uint32_t fin = 0;
 #pragma unroll
@@ -404,7 +407,7 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
             emit_v2c_pair<PHI, FULL>(sp.vclip, sj, Np, used, Q[0], Q[1], Q[2], mq, win, ax, az);
         }
         if (fin) restart(fin);  // finished lanes start their next shot from eq. (init)
-        pair_sync<ONE>(G, bar_id);
+        pair_sync<MODE>(G, bar_id);
         if (fin) {
 #pragma unroll
             for (int l = 0; l < 2; ++l)
@@ -422,19 +425,19 @@ __device__ __forceinline__ void decode_pairs(const DecodeArgs &a, const PairMem 
 
 // One code per launch, two shots per thread: a persistent grid whose shot
 // groups take shots from the global queue until the batch is exhausted.
-template <int VARIANT, bool FULL, bool ONE>
+template <int VARIANT, bool FULL, int MODE>
 __global__ void __launch_bounds__(1024, 1) decode_pair_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     int *grp_shot = reinterpret_cast<int *>(smem + 16);
 
     const int tid = threadIdx.x;
-    const int T = ONE ? (int)blockDim.x : a.G * 32;
-    const int G = ONE ? T / 32 : a.G;
-    const int group = ONE ? 0 : tid / T;
-    const int tg = ONE ? tid : tid - group * T;
+    const int T = MODE == kPairOne ? (int)blockDim.x : MODE == kPairWarps ? 32 : a.G * 32;
+    const int G = MODE == kPairGroups ? a.G : T / 32;
+    const int group = MODE == kPairOne ? 0 : tid / T;
+    const int tg = MODE == kPairOne ? tid : tid - group * T;
     const int bar_id = 1 + group;
-    const PairMem m = pair_mem<VARIANT, ONE>(a, smem, group);
-    const PairOffsets o = pair_offsets(VARIANT, ONE, a.M, a.n_pad);
+    const PairMem m = pair_mem<VARIANT, MODE>(a, smem, group);
+    const PairOffsets o = pair_offsets(VARIANT, MODE != kPairGroups, a.M, a.n_pad);
     const uint32_t kZero = 4u * (uint32_t)a.n_pad;
 #ifdef BPQ_DEBUG
     {
@@ -459,7 +462,7 @@ __global__ void __launch_bounds__(1024, 1) decode_pair_kernel(const DecodeArgs a
         for (int n = 0; n < 4; ++n) {
             if (sl[n] == kNoSlot || !BPQ_IN_BOUNDS(sl[n], kZero, a.work + 1)) sl[n] = kZero;
         }
-        if (ONE)
+        if (MODE != kPairGroups)
             reinterpret_cast<uint4 *>(smem + o.idx)[i] = make_uint4(8u * sl[0], 8u * sl[1], 8u * sl[2], 8u * sl[3]);
         else
             reinterpret_cast<uint2 *>(smem + o.idx)[i] = make_uint2(sl[0] | (sl[1] << 16), sl[2] | (sl[3] << 16));
@@ -488,16 +491,18 @@ __global__ void __launch_bounds__(1024, 1) decode_pair_kernel(const DecodeArgs a
         for (uint32_t s = (FULL ? kZero : 0u) + tg; s <= kZero; s += T) slots[s] = make_float2(0.f, 0.f);
     }
     __syncthreads();
-    decode_pairs<VARIANT, FULL, ONE>(a, m, T, tg, G, bar_id, grp_shot + 2 * group);
+    decode_pairs<VARIANT, FULL, MODE>(a, m, T, tg, G, bar_id, grp_shot + 2 * group);
 }
 
 }  // namespace dk
 
 // The two-shots-per-thread kernels of one variant (split tables; FULL for
-// tables without padding); one: one shot group per CTA.
+// tables without padding), by PairMode.
 #define BPQ_DEFINE_PICK_PAIR(NAME, V, FULLV)                                             \
-    DecodeKernelFn NAME(bool one) {                                                      \
-        return one ? dk::decode_pair_kernel<V, FULLV, true> : dk::decode_pair_kernel<V, FULLV, false>; \
+    DecodeKernelFn NAME(int mode) {                                                      \
+        return mode == kPairOne     ? dk::decode_pair_kernel<V, FULLV, kPairOne>         \
+               : mode == kPairWarps ? dk::decode_pair_kernel<V, FULLV, kPairWarps>       \
+                                    : dk::decode_pair_kernel<V, FULLV, kPairGroups>;     \
     }
 
 }  // namespace bpq
