@@ -201,10 +201,12 @@ __device__ __forceinline__ void check_node(const TrainArgs &a, const Adj &d, con
     }
 }
 
-// Lambda_H of one Pauli type H with the other two a, b.
+// Lambda_H of one Pauli type H with the other two a, b.  Prior probabilities of
+// 0 make Q infinite: with Qa = Qb = inf (noise of one Pauli only) the ratio has no
+// denominator and Lambda_H is inf; the minimum turns the NaN of inf - inf into 0.
 __device__ __forceinline__ float lambda_type(float QH, float Qa, float Qb) {
     const float lc = __fadd_rn(fmaxf(0.f, -QH), log1pf(expf(-fabsf(QH))));
-    const float la = __fadd_rn(fmaxf(-Qa, -Qb), log1pf(expf(-fabsf(__fsub_rn(Qa, Qb)))));
+    const float la = __fadd_rn(fmaxf(-Qa, -Qb), log1pf(expf(fminf(-fabsf(__fsub_rn(Qa, Qb)), 0.f))));
     return __fsub_rn(lc, la);
 }
 

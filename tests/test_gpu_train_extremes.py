@@ -1,0 +1,43 @@
+"""Training losses and gradients where the channel or the code is extreme:
+noise of one Pauli only (two of a qubit's prior probabilities are 0, so two of
+its log-likelihoods are infinite)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import unrolled
+from test_gpu_train import oracle_inputs, params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bpq():
+    import paper_2407_11523_gb300 as bpq
+    return bpq
+
+
+# The reference has 1e-30 in place of 0: log-likelihoods of 66 and more instead of infinity, beyond the
+# clip of 30 in every message, and probabilities that change no sum of fp32 or of the bars below (those of
+# the planar d = 9 tests; losses under 1e-9, where every qubit is certain, count as equal).  The gradient for alpha multiplies an infinite prior by 0 and is no number.
+@pytest.mark.parametrize("kind,d", [("planar", 5), ("toric", 4), ("xzzx", 5)])
+@pytest.mark.parametrize("ch", [(0.06, 0.0, 0.0), (0.0, 0.06, 0.0), (0.0, 0.0, 0.06), (0.04, 0.0, 0.03)])
+@pytest.mark.parametrize("kind_of_loss", ["posterior", "coset"])
+def test_noise_of_some_paulis_only(bpq, kind, d, ch, kind_of_loss):
+    T, B = 6, 16
+    t = bpq.Tanner(kind, d)
+    err, syn = bpq.sample(t, *ch, seed=5, shot0=0, B=B)
+    prior = bpq.prior_tensor(t, *ch)
+    H, s, e, pri = oracle_inputs(t, err, syn, np.maximum(ch, 1e-30))
+    Lg = t.logicals()
+    a, b, w = params(T, t.E, 6, spread=0.1)
+    ts = [torch.tensor(x, device="cuda", dtype=torch.float32, requires_grad=True) for x in (a, b, w)]
+    kw = dict(loss="coset", logicals=Lg) if kind_of_loss == "coset" else {}
+    L = bpq.unrolled_loss(t, syn, err, prior, *ts, T=T, ckpt_every=4, **kw)
+    L.backward()
+    kw = dict(kind="coset", logicals=Lg) if kind_of_loss == "coset" else {}
+    ref = unrolled.loss_and_grads(H, s, e, pri, a, b, w, T, **kw)
+    assert L.item() == pytest.approx(ref[0], rel=2e-4, abs=1e-9)
+    for x, r in zip(ts[1:], ref[2:]):
+        g = x.grad.cpu().numpy().astype(np.float64)
+        assert np.abs(g - r).max() <= 2e-3 * np.abs(r).max() + 1e-7, (np.abs(g - r).max(), np.abs(r).max())
