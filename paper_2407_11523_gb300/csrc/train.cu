@@ -476,7 +476,8 @@ __global__ void __launch_bounds__(1024, 1) train_forward_kernel(const TrainArgs 
     if (COSET) {
         check_terms();
         logical_terms(a.n_log - ((a.n_log - 1) % chunk + 1), (a.n_log - 1) % chunk + 1);
-        loss = (loss / (float)a.M + loss_log / (float)a.n_log) / (float)a.T;
+        // (a code without checks has no check terms)
+        loss = ((a.M ? loss / (float)a.M : 0.f) + loss_log / (float)a.n_log) / (float)a.T;
     } else if (qubit) {
         // cross-entropy of the final posterior against the true error; the
         // largest term enters through log1p, so that a small loss keeps its

@@ -1,6 +1,6 @@
 """Training losses and gradients where the channel or the code is extreme:
 noise of one Pauli only (two of a qubit's prior probabilities are 0, so two of
-its log-likelihoods are infinite)."""
+its log-likelihoods are infinite), no checks."""
 import numpy as np
 import pytest
 import torch
@@ -41,3 +41,24 @@ def test_noise_of_some_paulis_only(bpq, kind, d, ch, kind_of_loss):
     for x, r in zip(ts[1:], ref[2:]):
         g = x.grad.cpu().numpy().astype(np.float64)
         assert np.abs(g - r).max() <= 2e-3 * np.abs(r).max() + 1e-7, (np.abs(g - r).max(), np.abs(r).max())
+
+
+# A code without checks: every posterior is the prior, the coset loss has no check terms, and -log P of the
+# logical operator Z on qubit 0 is that of its X and Y errors.  rel 1e-6: a few roundings of fp32.
+def test_code_without_checks(bpq):
+    import ctypes
+
+    t = bpq.Tanner(H=np.zeros((0, 3), np.uint8)).upload()
+    prior = torch.tensor([[0.03, 0.02, 0.05], [0.1, 0.2, 0.1], [0.2, 0.1, 0.3]], device="cuda")
+    err = torch.tensor([[0, 1, 2], [1, 0, 0]], dtype=torch.uint8, device="cuda")
+    some = torch.full((4,), 0.5, device="cuda")  # weights of each of the T = 2 iterations; unused syndromes and edges
+    lg = torch.tensor([[3, 0, 0]], dtype=torch.uint8, device="cuda")
+    nbytes = bpq.lib().bpq_train_workspace_bytes(t.handle, 0, 2, 2, 1)
+    work, loss = torch.empty(nbytes, dtype=torch.uint8, device="cuda"), torch.empty(1, device="cuda")
+    p = lambda x: ctypes.c_void_p(x.data_ptr())
+    ld = bpq._binding.TrainLoss(1, lg.data_ptr(), 1)
+    rc = bpq.lib().bpq_train_forward(t.handle, 0, p(some), p(err), p(prior), 2, 2, 1, p(some), p(some), None, p(some),
+                                     30.0, ctypes.byref(ld), p(loss), None, p(work), nbytes,
+                                     ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0, bpq.lib().bpq_last_error()
+    assert loss.item() == pytest.approx(-(np.log(0.95) + np.log(0.05)) / 2, rel=1e-6)
