@@ -160,8 +160,10 @@ __device__ __forceinline__ void prior_llr(const TrainArgs &a, int x, float (&P)[
 
 // a [+] b = (1 + a)(1 + b) - 1.
 __device__ __forceinline__ float boxsum(float a, float b) { return __fmaf_rn(a, b, __fadd_rn(a, b)); }
-// Divisions by denominators below 2^126 (which all are here): __fdividef is
-// within 2 ulp and a fifth of the instructions of the rounded one.
+// Divisions: __fdividef is within 2 ulp and a fifth of the instructions of the
+// rounded one, for denominators of at most 2^126 (above, it gives 0).  expm1 of a
+// message is the one denominator that can be larger (messages above 87.3, with a
+// msg_clip that allows them); it goes in as its quarter.
 // h(y) = y (y + 2) / (y + 1).
 __device__ __forceinline__ float hfun(float y) { return __fmul_rn(y, __fadd_rn(1.f, __fdividef(1.f, __fadd_rn(y, 1.f)))); }
 
@@ -181,7 +183,7 @@ __device__ __forceinline__ void check_node(const TrainArgs &a, const Adj &d, con
         c.q[n] = 0.f;
         if (d.sl[n] != kNoSlot) {
             const float m = v[d.sl[n]];
-            c.q[n] = fminf(__fdividef(2.0f, expm1f(fabsf(m))), 1e12f);
+            c.q[n] = fminf(__fdividef(0.5f, 0.25f * expm1f(fabsf(m))), 1e12f);
             c.neg |= (m < 0.f ? 1u : 0u) << n;
         }
     }

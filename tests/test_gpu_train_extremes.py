@@ -1,6 +1,7 @@
 """Training losses and gradients where the channel or the code is extreme:
 noise of one Pauli only (two of a qubit's prior probabilities are 0, so two of
-its log-likelihoods are infinite), no checks."""
+its log-likelihoods are infinite), no checks, messages near the top of their
+range."""
 import numpy as np
 import pytest
 import torch
@@ -62,3 +63,23 @@ def test_code_without_checks(bpq):
                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert rc == 0, bpq.lib().bpq_last_error()
     assert loss.item() == pytest.approx(-(np.log(0.95) + np.log(0.05)) / 2, rel=1e-6)
+
+
+# Messages of 88.0 (both anticommuting Paulis of an edge have probability 3e-39), for which expm1 is above
+# 2^126: one iteration of checks of degree 2, 3 and 4 with weights of 1/2 against float64.  Bar: the largest
+# sum is about 260, of which fp32 holds 1.5e-5; expm1 and log1p are within a few such steps.
+def test_messages_near_the_top_of_the_range(bpq):
+    H = np.zeros((3, 7), np.uint8)
+    H[0, [0, 1]] = H[1, [1, 2, 3]] = H[2, [3, 4, 5, 6]] = 3
+    t = bpq.Tanner(H=H)
+    prior = np.full((7, 3), 3e-39, dtype=np.float32)
+    syn = np.array([[0], [5], [7]], np.int32)
+    a, b, w = np.full(1, 0.5), np.zeros(1), np.full(t.E, 0.5)
+    dev = lambda x, dt=torch.float32: torch.tensor(x, dtype=dt, device="cuda")
+    Q, _ = bpq.unrolled_posterior(t, dev(syn, torch.int32), torch.zeros((3, 7), dtype=torch.uint8, device="cuda"),
+                                  torch.from_numpy(prior).cuda(), dev(a), dev(b), dev(w), T=1, ckpt_every=1,
+                                  msg_clip=88.5)
+    s = (syn >> np.arange(3)) & 1
+    ref = unrolled.forward(unrolled.Graph(H), s, prior.astype(np.float64), *map(torch.tensor, (a, b, w)), T=1,
+                           clip=88.5).numpy()
+    assert np.abs(Q.cpu().numpy() - ref).max() <= 2e-4
