@@ -50,12 +50,17 @@ SerialShape serial_shape(const bpq_tanner *t, int variant, int mode) {
     r.off_qb = r.off_syn + (uint32_t)(((t->M + 31) / 32 + 3) & ~3);
     r.off_dec = r.off_qb + n_pad / 4;
     r.shot_words = r.off_dec + (sk::serial_state_arrays(variant) ? 0u : n_pad / 4);
-    // the shots of a warp: `lanes` banks apart
-    if (r.lanes < 32) r.shot_words += (uint32_t)(r.lanes - (int)(r.shot_words % 32) + 32) % 32;
+    const size_t limit = 227 * 1024;
+    auto warp_bytes = [&](uint32_t words) { return (32 / r.lanes) * 4 * (size_t)words; };
+    if (r.lanes < 32) {
+        // the shots of a warp `lanes` banks apart, unless that keeps the only warp out
+        const uint32_t spread = r.shot_words + (uint32_t)(r.lanes - (int)(r.shot_words % 32) + 32) % 32;
+        if (r.fixed + warp_bytes(spread) <= limit) r.shot_words = spread;
+    }
     r.shot_bytes = 4 * (size_t)r.shot_words;
-    const size_t limit = 227 * 1024, warp_bytes = (32 / r.lanes) * r.shot_bytes;
-    r.warps = r.fixed + warp_bytes > limit
-                  ? 0 : (int)std::min<size_t>(sk::serial_max_warps(r.lanes), (limit - r.fixed) / warp_bytes);
+    r.warps = r.fixed + warp_bytes(r.shot_words) > limit
+                  ? 0
+                  : (int)std::min<size_t>(sk::serial_max_warps(r.lanes), (limit - r.fixed) / warp_bytes(r.shot_words));
     return r;
 }
 
