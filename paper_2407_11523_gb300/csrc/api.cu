@@ -190,6 +190,11 @@ __global__ void sample_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli
     for (int k = threadIdx.x; k < cnt * W; k += blockDim.x) syn[b0 * W + k] = words[k];
 }
 
+// Bytes of shared memory of sample_kernel (W words of 32 checks): grows with N and W.
+constexpr size_t sample_smem(int N, int W) {
+    return 4 * (size_t)32 * (((N + 3) / 4) | 1) + 8 * (size_t)N + 4 * (size_t)32 * W;
+}
+
 // Four codes, one per byte; values above 3 (no Pauli code) count as I.
 __device__ __forceinline__ uint32_t valid_codes(uint32_t v) {
     const uint32_t bad = v & 0xFCFCFCFCu;
@@ -198,6 +203,12 @@ __device__ __forceinline__ uint32_t valid_codes(uint32_t v) {
     for (int l = 0; l < 4; ++l)
         if (!((bad >> (8 * l)) & 0xFFu)) r |= v & (0xFFu << (8 * l));
     return r;
+}
+
+constexpr int check_logical_stride(int N) { return N % 4 ? N : 4 * ((N / 4) | 1); }
+// (no N below kMaxNodes = 2048 takes more than 2048 does)
+constexpr size_t check_logical_smem(int N) {
+    return (((size_t)32 * check_logical_stride(N) + 7) & ~size_t(7)) + 8 * (size_t)N + 8;
 }
 
 // Classification of 32 consecutive shots per CTA: residual R = E^ E; 1 if R
@@ -616,10 +627,10 @@ int bpq_sample(const bpq_tanner *t, double px, double py, double pz, uint64_t se
     if (!err_dev || !syn_dev) return fail(BPQ_EINVAL, "NULL output");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nblk = (t->N + 3) / 4, W = (t->M + 31) / 32;
-    const size_t smem = 4 * (size_t)32 * (nblk | 1) + 8 * (size_t)t->N + 4 * (size_t)32 * W;
+    const size_t smem = bpq::sample_smem(t->N, W);
     if (smem > 48 * 1024) {
-        rc = bpq::cuda_check(cudaFuncSetAttribute(bpq::sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem), "sample attribute");
+        rc = bpq::allow_smem(bpq::sample_kernel, bpq::sample_smem(bpq::kMaxNodes, bpq::kMaxNodes / 32),
+                             "sample attribute");
         if (rc) return rc;
     }
     bpq::sample_kernel<<<bpq::launch_grid(B, 32), 32 * bpq::tile_warps(t, B, nblk), smem, st>>>(
@@ -859,11 +870,10 @@ int bpq_check_logical(const bpq_tanner *t, const uint8_t *err_dev, const uint8_t
     if (B == 0) return BPQ_OK;
     if (!err_dev || !est_dev || !fail_dev) return fail(BPQ_EINVAL, "NULL argument");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int stride = t->N % 4 ? t->N : 4 * ((t->N / 4) | 1);
-    const size_t smem = (((size_t)32 * stride + 7) & ~size_t(7)) + 8 * (size_t)t->N + 8;
+    const int stride = bpq::check_logical_stride(t->N);
+    const size_t smem = bpq::check_logical_smem(t->N);
     if (smem > 48 * 1024) {
-        rc = bpq::cuda_check(cudaFuncSetAttribute(bpq::check_logical_kernel,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        rc = bpq::allow_smem(bpq::check_logical_kernel, bpq::check_logical_smem(bpq::kMaxNodes),
                              "check_logical attribute");
         if (rc) return rc;
     }

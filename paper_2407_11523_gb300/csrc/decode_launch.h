@@ -165,6 +165,14 @@ void batch_start_items(const std::vector<double> &weight, int ctas, int *start);
 // Shared host helpers (api.cu).
 int need_uploaded(const bpq_tanner *t);
 int cuda_check(cudaError_t e, const char *what);
+// Lets a kernel take `most` bytes of dynamic shared memory.  The limit belongs to
+// the kernel and not to a launch, and all threads share it, so every caller
+// passes what the largest code takes: one that passed its own code's need would
+// lower it between another thread's call and launch.
+template <typename Fn>
+inline int allow_smem(Fn *fn, size_t most, const char *what) {
+    return cuda_check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most), what);
+}
 int cuda_set_device(int device);
 int fill_decode_args(const bpq_tanner *t, const uint32_t *syn, const float *prior, int variant,
                      const bpq_params *params, int max_iter, int B, void *work, DecodeArgs &a);

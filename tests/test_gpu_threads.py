@@ -1,0 +1,56 @@
+"""Calls from several host threads at once, each thread on a code, a stream
+and buffers of its own."""
+import ctypes
+import threading
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def in_threads(calls, rounds):
+    """calls: one list of (entry point, arguments) per thread, made over and
+    over; returns the error codes that are not 0 with their messages."""
+    import paper_2407_11523_gb300 as bpq
+
+    failures, go = set(), threading.Barrier(len(calls))
+
+    def loop(mine):
+        go.wait()
+        for _ in range(rounds):
+            for f, args in mine:
+                rc = f(*args)
+                if rc:
+                    failures.add((rc, bpq.lib().bpq_last_error()))
+
+    ts = [threading.Thread(target=loop, args=(c,)) for c in calls]
+    for th in ts:
+        th.start()
+    for th in ts:
+        th.join()
+    torch.cuda.synchronize()
+    return failures
+
+
+def p(x):
+    return ctypes.c_void_p(x.data_ptr())
+
+
+# Codes whose needs of shared memory differ, all above the 48 KB that a launch gets without asking
+def test_sample_and_check_logical_of_two_large_codes():
+    import paper_2407_11523_gb300 as bpq
+
+    calls, kept = [], []
+    for kind, d in [("planar", 26), ("toric", 32)] * 2:
+        t, stream = bpq.Tanner(kind, d).upload(), torch.cuda.Stream()
+        err, syn = bpq.sample(t, 0.02, 0.02, 0.02, seed=1, shot0=0, B=40)
+        out = [torch.empty_like(err), torch.empty_like(syn), torch.empty(40, dtype=torch.uint8, device="cuda")]
+        s, c = ctypes.c_void_p(stream.cuda_stream), ctypes.c_double(0.02)
+        kept.append((t, stream, err, syn, out))
+        calls.append([(bpq.lib().bpq_sample, (t.handle, c, c, c, 1, 0, 40, p(out[0]), p(out[1]), s)),
+                      (bpq.lib().bpq_check_logical, (t.handle, p(out[0]), p(out[0]), 40, p(out[2]), s))])
+    torch.cuda.synchronize()
+    assert not in_threads(calls, 10000)
+    for t, stream, err, syn, out in kept:
+        assert torch.equal(out[0], err) and torch.equal(out[1], syn) and not out[2].any()
