@@ -209,11 +209,12 @@ int bpq_decode_host(const bpq_tanner *t, const uint32_t *syn_host, const float *
  * (cudaGetSymbolAddress) and caches it; make that first call before any
  * stream capture.  The cached address does not survive a cudaDeviceReset:
  * resetting a device after that first call is not supported.  With CUDA's
- * default lazy module loading, the first launch of each decode kernel (one
- * per variant and message layout, see bpq_tanner_layout) loads its module,
- * and the driver may allocate device memory for it: make one warm-up call
- * per variant and code family before the loop that must not allocate, or
- * run with CUDA_MODULE_LOADING=EAGER.  All calls share the one array, which
+ * default lazy loading a kernel is loaded when it is first used, and the driver
+ * may allocate device memory for it.  Which kernel decodes depends on the
+ * variant, the message layout (bpq_tanner_layout), the code's size and the batch,
+ * so the first call of each variant and layout loads all of theirs: make one
+ * warm-up call, of any size, per variant and layout before the loop that must
+ * not allocate, or run with CUDA_MODULE_LOADING=EAGER.  All calls share the one array, which
  * keeps the last call's contents (the shot queue is reset on every call):
  * calls that may overlap on the GPU (other streams, other host threads) race
  * and must be serialised by the caller.  Arguments and errors otherwise as

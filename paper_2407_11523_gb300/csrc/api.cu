@@ -698,6 +698,9 @@ int bpq_decode_host_noalloc(const bpq_tanner *t, const uint32_t *syn_host, const
     void *scratch = nullptr;
     rc = bpq::noalloc_scratch(t->device, &scratch);
     if (rc) return rc;
+    // so that the first call of a variant and layout covers every batch size
+    rc = bpq::decode_preload(t, variant);
+    if (rc) return rc;
     return bpq::decode_host_impl(t, syn_host, prior_host, variant, params, max_iter, B, est_host, conv_host,
                                  iters_host, scratch, bpq::kNoAllocBytes, stream, false);
 }

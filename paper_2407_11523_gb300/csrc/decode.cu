@@ -3,7 +3,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <vector>
 
 #include "bpq_internal.h"
 #include "decode_launch.h"
@@ -241,6 +243,36 @@ bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t 
 constexpr long kOneNodeShotsPerGroup = 3;
 
 }  // namespace
+
+// Every kernel that decode_launch can pick for this variant and table layout,
+// whatever the batch and the stored shape.  The runtime loads a kernel when it is
+// first asked about it (CUDA's lazy loading), so asking about all of them leaves
+// no load, and no allocation for one, to a later call of another batch size.
+int decode_preload(const bpq_tanner *t, int variant) {
+    if (variant < BPQ_PLAIN || variant > BPQ_AEWA) return BPQ_OK;  // refused later
+    const int layout = t->full ? 2 : t->split ? 1 : 0;
+    static std::atomic<uint32_t> loaded[kMaxPreloadDevices];  // bit per (checked, layout, variant)
+    const uint32_t bit = 1u << ((t->debug_checks ? 15 : 0) + 5 * layout + variant);
+    std::atomic<uint32_t> *done = t->device < kMaxPreloadDevices ? &loaded[t->device] : nullptr;
+    if (done && (done->load(std::memory_order_acquire) & bit)) return BPQ_OK;
+    const bool pairs = layout && variant != BPQ_AEWA;
+    std::vector<const void *> fns;
+    auto add = [&](auto *fn) {
+        if (fn) fns.push_back(reinterpret_cast<const void *>(fn));
+    };
+    for (int npt = 1; npt <= 3; ++npt)  // three and more: one kernel
+        add(t->debug_checks ? pick_debug(variant, npt, false, 0, layout) : pick(variant, npt, false, layout));
+    for (int mode = kPairGroups; pairs && mode <= kPairWarps; ++mode)
+        add(t->debug_checks ? pick_debug(variant, 1, true, mode, layout) : pick_pair(variant, mode, layout));
+    for (int lanes = 1; layout && !t->debug_checks && lanes <= 4; lanes *= 2) add(pick_small(variant, lanes));
+    for (const void *fn : fns) {
+        cudaFuncAttributes attr;
+        const int rc = cuda_check(cudaFuncGetAttributes(&attr, fn), "kernel load");
+        if (rc) return rc;
+    }
+    if (done) done->fetch_or(bit, std::memory_order_release);
+    return BPQ_OK;
+}
 
 int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out) {
     int small_rc = BPQ_OK;

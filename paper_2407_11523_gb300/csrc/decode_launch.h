@@ -177,5 +177,8 @@ int cuda_set_device(int device);
 int fill_decode_args(const bpq_tanner *t, const uint32_t *syn, const float *prior, int variant,
                      const bpq_params *params, int max_iter, int B, void *work, DecodeArgs &a);
 int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out);
+// Loads every kernel that decode_launch can pick for this variant and table layout.
+int decode_preload(const bpq_tanner *t, int variant);
+constexpr int kMaxPreloadDevices = 64;
 
 }  // namespace bpq
