@@ -282,12 +282,13 @@ int bpq_set_debug_checks(bpq_tanner *t, int on);
 
 /* Autotuner of the launch shape (an addition; the paper has no GPU design):
  * times bpq_decode on the caller's sample batch (same arguments as
- * bpq_decode) for every candidate shape - one or two shots per thread, 1..4
- * nodes per thread (1..2 with two shots per thread), 1..32 shot groups per
- * CTA - and stores the fastest in the handle (as bpq_set_launch and
- * bpq_set_shots_per_thread would).  Synchronizes `stream`; the outputs are
- * those of the last trial.  Reports the chosen shape and its time per
- * launch (any output pointer may be NULL).  Errors: as bpq_decode, plus
+ * bpq_decode) for the automatic choice and every candidate shape - one or two
+ * shots per thread, 1..4 nodes per thread (1..2 with two shots per thread),
+ * 1..32 shot groups per CTA - and stores the fastest in the handle (as
+ * bpq_set_launch and bpq_set_shots_per_thread would).  Synchronizes `stream`;
+ * the outputs are those of the last trial.  Reports the chosen shape (0 and 0:
+ * the automatic choice) and its time per launch (any output pointer may be
+ * NULL).  Errors: as bpq_decode, plus
  * EINVAL when B < 1 or no shape fits the code; on an error the handle keeps
  * its previous shape. */
 int bpq_autotune(bpq_tanner *t, const uint32_t *syn_dev, const float *prior_dev, int variant,

@@ -263,8 +263,9 @@ class Tanner:
 
 
 def autotune(tanner: Tanner, syn, prior, variant="ewainit", params=None, max_iter=100, stream=None, **param_kw):
-    """Time every candidate launch shape on this sample batch and keep the
-    fastest in the handle; returns (threads_per_shot, shots_per_cta, ms)."""
+    """Time the automatic choice and every candidate launch shape on this
+    sample batch and keep the fastest in the handle; returns (threads_per_shot,
+    shots_per_cta, ms), 0 and 0 for the automatic choice."""
     tanner.upload()
     v = VARIANTS.get(variant, variant)
     p = params if params is not None else make_params(v, **param_kw)

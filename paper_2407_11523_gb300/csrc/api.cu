@@ -785,16 +785,42 @@ int bpq_autotune(bpq_tanner *t, const uint32_t *syn_dev, const float *prior_dev,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nodes = t->N > t->M ? t->N : t->M;
     const int old_t = t->threads_per_shot, old_s = t->shots_per_cta, old_k = t->shots_per_thread;
-    int best_T = 0, best_S = 0, best_K = 1;
+    int best_T = 0, best_S = 0, best_K = 0;
+    bool found = false;
     float best = 1e30f;
     cudaEvent_t e0, e1;
     rc = bpq::cuda_check(cudaEventCreate(&e0), "cudaEventCreate");
     if (rc) return rc;
     rc = bpq::cuda_check(cudaEventCreate(&e1), "cudaEventCreate");
     if (rc) { cudaEventDestroy(e0); return rc; }
-    // candidate shapes: one or (split tables, not AEWA-BP) two shots per
-    // thread; 1..4 nodes per thread (1..2 with two shots per thread); 1..32
-    // shot groups per CTA
+    auto time_shape = [&](int T, int S, int K) {
+        t->threads_per_shot = T;
+        t->shots_per_cta = S;
+        t->shots_per_thread = K;
+        float ms = 0.f;
+        for (int rep = 0; rep < 3 && !rc; ++rep) {  // one warm-up, two timed
+            if (rep == 1) rc = bpq::cuda_check(cudaEventRecord(e0, st), "cudaEventRecord");
+            if (!rc)
+                rc = bpq_decode(t, syn_dev, prior_dev, variant, params, max_iter, B, est_dev, conv_dev, iters_dev,
+                                work_dev, stream);
+        }
+        if (!rc) rc = bpq::cuda_check(cudaEventRecord(e1, st), "cudaEventRecord");
+        if (!rc) rc = bpq::cuda_check(cudaEventSynchronize(e1), "cudaEventSynchronize");
+        if (!rc) rc = bpq::cuda_check(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
+        if (!rc && ms / 2 < best) {
+            best = ms / 2;
+            best_T = T;
+            best_S = S;
+            best_K = K;
+            found = true;
+        }
+    };
+    // candidate shapes: the automatic choice, which small batches need (a stored
+    // shape keeps to the queue kernels: 150 planar d = 9 Momentum shots at p =
+    // 0.06 27 us automatic, 34 with the best stored shape); one or (split tables,
+    // not AEWA-BP) two shots per thread; 1..4 nodes per thread (1..2 with two
+    // shots per thread); 1..32 shot groups per CTA
+    time_shape(0, 0, 0);
     const bool can_pair = t->split && variant >= BPQ_PLAIN && variant <= BPQ_EWAINIT;
     for (int K = 1; K <= (can_pair ? 2 : 1) && !rc; ++K)
     for (int npt = 1; npt <= (K == 2 ? 2 : bpq::kMaxNodesPerThread) && !rc; ++npt) {
@@ -810,27 +836,12 @@ int bpq_autotune(bpq_tanner *t, const uint32_t *syn_dev, const float *prior_dev,
             bpq::LaunchShape shape;
             if (K == 2 ? bpq::decode_pair_shape(t, variant, &shape) : bpq::decode_launch_shape(t, variant, &shape))
                 continue;
-            float ms = 0.f;
-            for (int rep = 0; rep < 3 && !rc; ++rep) {  // one warm-up, two timed
-                if (rep == 1) rc = bpq::cuda_check(cudaEventRecord(e0, st), "cudaEventRecord");
-                if (!rc)
-                    rc = bpq_decode(t, syn_dev, prior_dev, variant, params, max_iter, B, est_dev, conv_dev,
-                                    iters_dev, work_dev, stream);
-            }
-            if (!rc) rc = bpq::cuda_check(cudaEventRecord(e1, st), "cudaEventRecord");
-            if (!rc) rc = bpq::cuda_check(cudaEventSynchronize(e1), "cudaEventSynchronize");
-            if (!rc) rc = bpq::cuda_check(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
-            if (!rc && ms / 2 < best) {
-                best = ms / 2;
-                best_T = T;
-                best_S = S;
-                best_K = K;
-            }
+            if (!rc) time_shape(T, S, K);
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc || best_T == 0) {
+    if (rc || !found) {
         t->threads_per_shot = old_t;
         t->shots_per_cta = old_s;
         t->shots_per_thread = old_k;
