@@ -214,7 +214,7 @@ namespace {
 // 640 threads of them; one lane per node pays (no queue reset, no table
 // staging) while every shot has a CTA of its own.
 bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t st, int *rc) {
-    if (a.split == 0 || t->debug_checks || t->threads_per_shot || t->shots_per_cta || t->shots_per_thread) return false;
+    if (a.split == 0 || t->threads_per_shot || t->shots_per_cta || t->shots_per_thread) return false;
     const int nodes = t->N > t->M ? t->N : t->M;
     const long shots_per_sm = ((long)a.B + t->num_sms - 1) / t->num_sms;
     if (nodes > 1024 || shots_per_sm > 32) return false;
@@ -227,8 +227,13 @@ bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t 
     if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess ||
         shots_per_sm > per_sm)
         return false;
+    if (t->debug_checks && !(fn = pick_debug_small(variant, lanes))) return false;
     a.n_pad = (t->N + 3) & ~3;
     const bool unclipped = a.split == 2 && variant != BPQ_ADAGRAD;
+    if (t->debug_checks) {  // the checked copy does not reset the error word, which any CTA may set
+        *rc = cuda_check(cudaMemsetAsync(a.work, 0, 8, st), "workspace reset");
+        if (*rc) return true;
+    }
     fn<<<(unsigned)a.B, threads, smem, st>>>(a, variant == BPQ_AEWA ? 11 : 1, unclipped ? INFINITY : a.clip2);
     *rc = cuda_check(cudaGetLastError(), "decode launch");
     return true;
@@ -264,7 +269,8 @@ int decode_preload(const bpq_tanner *t, int variant) {
         add(t->debug_checks ? pick_debug(variant, npt, false, 0, layout) : pick(variant, npt, false, layout));
     for (int mode = kPairGroups; pairs && mode <= kPairWarps; ++mode)
         add(t->debug_checks ? pick_debug(variant, 1, true, mode, layout) : pick_pair(variant, mode, layout));
-    for (int lanes = 1; layout && !t->debug_checks && lanes <= 4; lanes *= 2) add(pick_small(variant, lanes));
+    for (int lanes = 1; layout && lanes <= 4; lanes *= 2)
+        add(t->debug_checks ? pick_debug_small(variant, lanes) : pick_small(variant, lanes));
     for (const void *fn : fns) {
         cudaFuncAttributes attr;
         const int rc = cuda_check(cudaFuncGetAttributes(&attr, fn), "kernel load");

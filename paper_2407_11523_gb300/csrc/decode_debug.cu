@@ -1,11 +1,12 @@
 // Bounds-checked copies of the one-code decode kernels (one and two shots per
-// thread; plain, Momentum, AdaGrad and EWAInit BP; one or two nodes per
-// thread; every table layout), compiled with BPQ_DEBUG into namespace
+// thread and small batches; plain, Momentum, AdaGrad and EWAInit BP; one or two
+// nodes per thread; every table layout), compiled with BPQ_DEBUG into namespace
 // bpq::dk_debug.  bpq_set_debug_checks selects them.
 #define BPQ_DEBUG 1
 #define dk dk_debug
 #include "decode_kernel.cuh"
 #include "decode_pair.cuh"
+#include "decode_small.cuh"
 #undef dk
 
 namespace bpq {
@@ -42,6 +43,27 @@ DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int mode, int layout
         case BPQ_MOMENTUM: return pick_debug_v<BPQ_MOMENTUM>(npt, pairs, mode, layout);
         case BPQ_ADAGRAD: return pick_debug_v<BPQ_ADAGRAD>(npt, pairs, mode, layout);
         case BPQ_EWAINIT: return pick_debug_v<BPQ_EWAINIT>(npt, pairs, mode, layout);
+    }
+    return nullptr;
+}
+
+namespace {
+
+template <int V>
+SmallKernelFn pick_debug_lanes(int lanes) {
+    return lanes == 4   ? dk_debug::decode_small_kernel<V, 4>
+           : lanes == 2 ? dk_debug::decode_small_kernel<V, 2>
+                        : dk_debug::decode_small_kernel<V, 1>;
+}
+
+}  // namespace
+
+SmallKernelFn pick_debug_small(int variant, int lanes) {
+    switch (variant) {
+        case BPQ_PLAIN: return pick_debug_lanes<BPQ_PLAIN>(lanes);
+        case BPQ_MOMENTUM: return pick_debug_lanes<BPQ_MOMENTUM>(lanes);
+        case BPQ_ADAGRAD: return pick_debug_lanes<BPQ_ADAGRAD>(lanes);
+        case BPQ_EWAINIT: return pick_debug_lanes<BPQ_EWAINIT>(lanes);
     }
     return nullptr;
 }

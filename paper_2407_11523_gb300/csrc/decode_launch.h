@@ -116,6 +116,7 @@ SmallKernelFn pick_small(int variant, int lanes);
 // {1, 2} with one shot per thread, pairs on split layouts (mode: PairMode);
 // nullptr where none is compiled.
 DecodeKernelFn pick_debug(int variant, int npt, bool pairs, int mode, int layout);
+SmallKernelFn pick_debug_small(int variant, int lanes);  // not AEWA-BP
 
 int decode_launch_shape(const bpq_tanner *t, int variant, LaunchShape *s);
 // Whether bpq_decode runs the two-shots-per-thread kernel for this graph and
