@@ -154,10 +154,10 @@ int bpq_batch_plan(const bpq_batch_item *items, int n_items, int variant, const 
 
     bpq::BatchKernelFn fn = bpq::pick_batch_kernel(variant, generic);
     if (!fn) return fail(BPQ_EINVAL, "no batched kernel for this shape");
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+    rc = bpq::allow_smem(fn, bpq::kMaxDynamicSmem, "cudaFuncSetAttribute");
+    if (rc) return rc;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, bpq::kBatchThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, bpq::kBatchThreads, smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "batched kernel does not fit on an SM");
     long ctas = (long)per_sm * items[0].tanner->num_sms;
     ctas = std::min<long>({ctas, std::max(1L, useful_ctas), (long)bpq::kMaxBatchCtas});

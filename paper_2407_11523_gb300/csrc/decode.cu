@@ -307,7 +307,7 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         int per_sm = 0;
         DecodeKernelFn f1 = nullptr;
         if (decode_launch_shape(t, variant, &one) == BPQ_OK && (f1 = pick(variant, one.npt, false, a.split)) &&
-            cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one.smem) == cudaSuccess &&
+            allow_smem(f1, kMaxDynamicSmem, "cudaFuncSetAttribute") == BPQ_OK &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
             decode_pair_shape(t, variant, &s) == BPQ_OK &&
@@ -326,10 +326,10 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         fn = pairs ? pick_pair(variant, s.pair_mode, a.split) : pick(variant, s.npt, trace, a.split);
     }
     if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant (AEWA-BP has no trace mode)");
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
-    if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+    rc = allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute");
+    if (rc) return rc;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
     const int nodes = t->N > t->M ? t->N : t->M;
     if (!pairs && !trace && s.npt == 2 && !t->threads_per_shot && !t->shots_per_cta && nodes <= kMaxThreadsPerShot &&
@@ -340,8 +340,8 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         s.init_bytes = 0;
         fn = t->debug_checks ? pick_debug(variant, s.npt, false, 0, a.split) : pick(variant, s.npt, false, a.split);
         if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant");
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
-        if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+        rc = allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute");
+        if (rc) return rc;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
         if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
     }

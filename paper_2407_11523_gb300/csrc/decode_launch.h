@@ -169,7 +169,9 @@ int cuda_check(cudaError_t e, const char *what);
 // Lets a kernel take `most` bytes of dynamic shared memory.  The limit belongs to
 // the kernel and not to a launch, and all threads share it, so every caller
 // passes what the largest code takes: one that passed its own code's need would
-// lower it between another thread's call and launch.
+// lower it between another thread's call and launch, or a plan's making and its
+// launch.
+constexpr size_t kMaxDynamicSmem = 227 * 1024;  // of a kernel without static shared memory
 template <typename Fn>
 inline int allow_smem(Fn *fn, size_t most, const char *what) {
     return cuda_check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most), what);

@@ -166,10 +166,10 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
                             : mode == kSerial16 ? sk::pick_serial16(variant, t->split)
                                                 : sk::pick_serial8(variant, t->split);
     if (!fn) return fail(BPQ_EINVAL, "no serial kernel for this variant");
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+    rc = allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute");
+    if (rc) return rc;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "serial kernel does not fit on an SM");
     long ctas = (long)per_sm * t->num_sms;
     const long per_cta = warps * per_warp;

@@ -469,10 +469,10 @@ int bpq_server_create(const bpq_tanner *const *codes, const float *const *priors
             free_server(s);
             return fail(BPQ_EINVAL, "no batched kernel for these codes");
         }
-        cudaError_t e = cudaFuncSetAttribute(s->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem);
+        rc = bpq::allow_smem(s->fn, bpq::kMaxDynamicSmem, "cudaFuncSetAttribute");
         int per_sm = 0;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, s->fn, bpq::kBatchThreads, s->smem);
-        if (e != cudaSuccess || per_sm < 1) rc = fail(BPQ_ECUDA, "batched kernel does not fit on an SM");
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, s->fn, bpq::kBatchThreads, s->smem);
+        if (!rc && (e != cudaSuccess || per_sm < 1)) rc = fail(BPQ_ECUDA, "batched kernel does not fit on an SM");
         s->ctas = per_sm * s->codes[0]->num_sms;
     }
     const size_t lane_bytes = lane_device_bytes(n_codes, max_batch, s->Wmax, s->Nmax);
@@ -777,11 +777,12 @@ int bpq_server_create_slots(const bpq_tanner *const *codes, const float *const *
     }
     if (!rc) {
         R.fn = bpq::pick_serve_kernel(variant);
-        cudaError_t e = cudaFuncSetAttribute(R.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem);
+        cudaFuncAttributes fa;  // (for its static shared memory, which counts against the same 227 KB)
+        rc = bpq::cuda_check(cudaFuncGetAttributes(&fa, R.fn), "serving kernel attributes");
+        if (!rc) rc = bpq::allow_smem(R.fn, bpq::kMaxDynamicSmem - fa.sharedSizeBytes, "cudaFuncSetAttribute");
         int per_sm = 0;
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, R.fn, bpq::kBatchThreads, s->smem);
-        if (e != cudaSuccess || per_sm < 1) rc = fail(BPQ_ECUDA, "serving kernel does not fit on an SM");
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, R.fn, bpq::kBatchThreads, s->smem);
+        if (!rc && (e != cudaSuccess || per_sm < 1)) rc = fail(BPQ_ECUDA, "serving kernel does not fit on an SM");
         R.grid = per_sm * s->codes[0]->num_sms;
     }
     if (!rc) rc = bpq::cuda_check(cudaStreamCreateWithFlags(&R.st, cudaStreamNonBlocking), "server stream");

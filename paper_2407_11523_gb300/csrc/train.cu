@@ -988,8 +988,9 @@ int bpq_train_forward(const bpq_tanner *t, int model, const uint32_t *syn_dev, c
     using namespace bpq::tr;
     void (*fn)(const TrainArgs) = mom ? (coset ? train_forward_kernel<kMomentum, true> : train_forward_kernel<kMomentum, false>)
                                       : (coset ? train_forward_kernel<kEWAInit, true> : train_forward_kernel<kEWAInit, false>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("train forward attribute: ") + cudaGetErrorString(e));
+    // what a code of 1024 nodes takes with the coset loss
+    rc = bpq::allow_smem(fn, sizeof(float) * (12 * 1024 + 4 * 32), "train forward attribute");
+    if (rc) return rc;
     fn<<<B, threads, smem, st>>>(a);
     // per-shot sums: over qubits (posterior loss) or already normalised (coset loss)
     bpq::tr::launch_reduce(a.loss_shot, B, 1, {{loss_dev}, {1}},
@@ -1014,14 +1015,14 @@ int bpq_train_backward(const bpq_tanner *t, int model, const uint32_t *syn_dev, 
     const size_t smem = sizeof(float) * bpq::tr::backward_floats(a.n_pad, a.K, mom, a.n_log, threads / 32);
     if (smem > 227 * 1024) return fail(BPQ_EINVAL, "checkpoint interval too long for shared memory");
     void (*fn)(const bpq::tr::TrainArgs) = bpq::tr::pick_backward(mom, a.loss_kind == BPQ_TRAIN_LOSS_COSET, threads);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("train backward attribute: ") + cudaGetErrorString(e));
+    rc = bpq::allow_smem(fn, bpq::kMaxDynamicSmem, "train backward attribute");
+    if (rc) return rc;
     fn<<<B, threads, smem, st>>>(a);
     // per-shot rows hold [alpha | beta | w | gamma]
     bpq::tr::launch_reduce(a.rows, B, a.width,
                            {{grad_alpha_dev, grad_beta_dev, grad_w_dev, mom ? grad_gamma_dev : nullptr},
                             {T, 2 * T, 2 * T + t->E, a.width}}, 1.f, st);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(BPQ_ECUDA, std::string("train backward launch: ") + cudaGetErrorString(e));
     return BPQ_OK;
 }
