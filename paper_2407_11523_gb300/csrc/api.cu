@@ -190,6 +190,52 @@ __global__ void sample_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli
     for (int k = threadIdx.x; k < cnt * W; k += blockDim.x) syn[b0 * W + k] = words[k];
 }
 
+// The same for few shots: one CTA per shot, whose threads draw blocks of four
+// qubits and then test a check each.  sample_kernel gives a shot one lane, so few
+// shots leave most of the chip idle and a large code's blocks follow one another
+// (planar d = 31, 1 to 2000 shots: 36 us whatever the number).  Bound: the launch,
+// then the Philox chain.  Errors and syndromes, us a call, tile kernel / this:
+// planar d = 31, 40 shots 36 / 9.3, 1500 37 / 25.6, 2000 37 / 34, 3000 37 / 47;
+// planar d = 18, 300 15 / 8.7, 1500 15.4 / 12.8, 2000 15.4 / 15.3, 3000 15.4 /
+// 21; codes of up to 200 qubits the same up to 3000 shots (8.5).
+__global__ void sample_shot_kernel(const uint16_t *chk_slot, const uint8_t *chk_pauli, int N, int M, int W,
+                                   uint64_t seed, uint64_t shot0, uint64_t tx, uint64_t ty, uint64_t tz, uint8_t *err,
+                                   uint32_t *syn) {
+    __shared__ uint32_t codes[kMaxNodes / 4];  // one code per byte
+    const int nblk = (N + 3) / 4;
+    const PhiloxShot ps = philox_shot(shot0 + blockIdx.x, seed);
+    for (int blk = threadIdx.x; blk < nblk; blk += blockDim.x) {
+        uint64_t u[4];
+        philox_block(ps, (uint64_t)blk, seed, u);
+        uint32_t word = 0;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) word |= (u[l] < tx ? 1u : u[l] < ty ? 2u : u[l] < tz ? 3u : 0u) << (8 * l);
+        codes[blk] = word;
+    }
+    __syncthreads();
+    const uint8_t *code = reinterpret_cast<const uint8_t *>(codes);
+    uint8_t *e = err + (size_t)blockIdx.x * N;
+    for (int j = threadIdx.x; j < N; j += blockDim.x) e[j] = code[j];
+    for (int i0 = threadIdx.x & ~31; i0 < M; i0 += blockDim.x) {
+        const int i = i0 + (threadIdx.x & 31);
+        uint32_t odd = 0;
+        if (i < M) {
+            const uint32_t cp = chk_pauli[i];
+            const uint2 s = *reinterpret_cast<const uint2 *>(chk_slot + 4 * i);
+            const uint32_t sl[4] = {s.x & 0xFFFFu, s.x >> 16, s.y & 0xFFFFu, s.y >> 16};
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                const uint32_t p = (cp >> (2 * n)) & 3u;  // the mask of anti_word: 2, 1, 3 for X, Y, Z
+                if (sl[n] != kNoSlot) odd ^= __popc(code[sl[n] >> 2] & (p == 3u ? 3u : 3u - p));
+            }
+        }
+        const uint32_t word = __ballot_sync(0xffffffffu, odd & 1u);
+        if ((threadIdx.x & 31) == 0) syn[(size_t)blockIdx.x * W + (i0 >> 5)] = word;
+    }
+}
+// Batches of at most this many shots per SM (1824 on a GB300) take it.
+constexpr long kSampleShotsPerSm = 12;
+
 // Bytes of shared memory of sample_kernel (W words of 32 checks): grows with N and W.
 constexpr size_t sample_smem(int N, int W) {
     return 4 * (size_t)32 * (((N + 3) / 4) | 1) + 8 * (size_t)N + 4 * (size_t)32 * W;
@@ -627,6 +673,16 @@ int bpq_sample(const bpq_tanner *t, double px, double py, double pz, uint64_t se
     if (!err_dev || !syn_dev) return fail(BPQ_EINVAL, "NULL output");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nblk = (t->N + 3) / 4, W = (t->M + 31) / 32;
+    const uint16_t *chk_slot = reinterpret_cast<const uint16_t *>(t->d_table);
+    const uint8_t *chk_pauli = t->d_table + t->off_chk_pauli;
+    const uint64_t tx = bpq::threshold(cx), ty = bpq::threshold(cy), tz = bpq::threshold(cz);
+    if (B <= bpq::kSampleShotsPerSm * t->num_sms) {
+        // a block a thread and two checks a thread, where 512 threads reach that
+        const int threads = std::min(512, (std::max(nblk, t->M / 2) / 32 + 1) * 32);
+        bpq::sample_shot_kernel<<<(unsigned)B, threads, 0, st>>>(chk_slot, chk_pauli, t->N, t->M, W, seed, shot0, tx,
+                                                                 ty, tz, err_dev, syn_dev);
+        return bpq::cuda_check(cudaGetLastError(), "sample launch");
+    }
     const size_t smem = bpq::sample_smem(t->N, W);
     if (smem > 48 * 1024) {
         rc = bpq::allow_smem(bpq::sample_kernel, bpq::sample_smem(bpq::kMaxNodes, bpq::kMaxNodes / 32),
@@ -634,8 +690,7 @@ int bpq_sample(const bpq_tanner *t, double px, double py, double pz, uint64_t se
         if (rc) return rc;
     }
     bpq::sample_kernel<<<bpq::launch_grid(B, 32), 32 * bpq::tile_warps(t, B, nblk), smem, st>>>(
-        reinterpret_cast<const uint16_t *>(t->d_table), t->d_table + t->off_chk_pauli, t->N, t->M, W, B, seed, shot0,
-        bpq::threshold(cx), bpq::threshold(cy), bpq::threshold(cz), err_dev, syn_dev);
+        chk_slot, chk_pauli, t->N, t->M, W, B, seed, shot0, tx, ty, tz, err_dev, syn_dev);
     return bpq::cuda_check(cudaGetLastError(), "sample launch");
 }
 
