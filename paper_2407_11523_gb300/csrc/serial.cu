@@ -30,6 +30,8 @@ namespace {
 enum SerialMode { kSerial32 = 0, kSerial16 = 1, kSerial8 = 2 };
 constexpr int kModeLanes[3] = {32, 16, 8}, kModeTable[3] = {0, 0, 1};
 
+constexpr int kSerialStageWarps = 16;  // within every kernel's serial_max_warps
+
 // Shared memory of a launch.
 struct SerialShape {
     int lanes, warps;        // warps: that fit (0: not even one)
@@ -162,6 +164,14 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     const long per_warp = 32 / shape.lanes, wave = per_warp * t->num_sms;
     const int warps = (int)std::min<long>(shape.warps, (B + wave - 1) / wave);
     const size_t smem = shape.smem(warps);
+    // with few decoding warps, further ones share the staging of the prior and the
+    // initial messages (three logarithms and the message rule per qubit), which
+    // one warp takes a qubit per lane at a time.  One shot, EWAInit, us, without /
+    // with: toric d = 27 128 / 103, d = 20 77 / 63, planar d = 25 130 / 110, d = 11
+    // 19.6 / 16.4; staging on the sweep's own arrays before (one warp, no initial
+    // messages) 105, 67, 113, 18.2
+    a.warps = warps;
+    const int threads = 32 * std::max(warps, std::min(kSerialStageWarps, (t->N + 31) / 32));
     sk::SerialKernelFn fn = mode == kSerial32   ? sk::pick_serial32(variant, trace, t->split)
                             : mode == kSerial16 ? sk::pick_serial16(variant, t->split)
                                                 : sk::pick_serial8(variant, t->split);
@@ -169,7 +179,7 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     rc = allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute");
     if (rc) return rc;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "serial kernel does not fit on an SM");
     long ctas = (long)per_sm * t->num_sms;
     const long per_cta = warps * per_warp;
@@ -177,7 +187,7 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     if (ctas > need) ctas = need;
     rc = cuda_check(cudaMemsetAsync(work, 0, 8, st), "workspace reset");
     if (rc) return rc;
-    fn<<<(unsigned)std::max(1L, ctas), warps * 32, smem, st>>>(a);
+    fn<<<(unsigned)std::max(1L, ctas), threads, smem, st>>>(a);
     return cuda_check(cudaGetLastError(), "serial decode launch");
 }
 

@@ -86,6 +86,7 @@ struct SerialArgs {
     uint8_t *tr_dec;
     int N, M, E, W, B, max_iter;
     int n_pad;             // N rounded up to 4 (per-qubit array stride)
+    int warps;             // warps that decode; further warps of the CTA only stage the tables
     uint32_t zero_slot;    // message slots: [0, zero_slot) edges, then zero, no information, trash
     uint32_t shot_words;   // shared memory of one shot: messages | state | syndrome | qubit bytes
     uint32_t off_state, off_syn, off_qb, off_dec;  // word offsets inside it
@@ -486,7 +487,8 @@ __global__ void __launch_bounds__(32 * serial_max_warps(LANES), 1) serial_kernel
     constexpr int K = 32 / LANES;  // shots per warp
     SerialTab tab;
     uint32_t *mem;
-    if (!stage_serial<VARIANT, SPLIT>(a, smem, K * (int)(blockDim.x >> 5), tab, &mem)) return;
+    if (!stage_serial<VARIANT, SPLIT>(a, smem, K * a.warps, tab, &mem)) return;
+    if ((int)(threadIdx.x >> 5) >= a.warps) return;  // (no CTA barrier below)
     const int lane = threadIdx.x & 31, g = lane / LANES, ln = lane % LANES;
     const int h = ln % Q, pos = ln / Q;
     ShotMem m;
