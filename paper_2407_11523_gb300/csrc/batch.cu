@@ -53,17 +53,23 @@ void batch_start_items(const std::vector<double> &weight, int ctas, int *start) 
 
 namespace {
 // The batched kernel's threads that an item's shot groups leave over form one
-// more, smaller group (its shots take longer: more nodes per thread) where they
-// are at least half a group's and shared memory has room (planar d = 25: 416 of
-// 1024 threads, idle otherwise), and an item's initial messages take a table of
-// their own where shared memory has room for that: both once the batch holds
-// this many CTA loads of shots per SM, since a smaller batch ends with its
-// slowest shots and does not repay the table.  Without and with both, ten codes
-// in turn (us): plain, p = 0.03, 1146 shots (2 loads) 258 / 269, 4000 (6) 631 /
-// 630, 10000 (16) 1437 / 1327, 30000 (47) 4028 / 3709; EWAInit, p = 0.06, 4000
-// shots 479 / 510, 10000 1007 / 988, 30000 2765 / 2581; 262144 shots 24.7 / 21.2
-// ms.
+// more, smaller group where they are at least half a group's and shared memory has
+// room (planar d = 25: 416 of 1024 threads, idle otherwise), and an item's initial
+// messages take a table of their own where shared memory has room for that: both
+// once the batch holds this many CTA loads of shots per SM, since a smaller batch
+// ends with its slowest shots and does not repay the table.  Without and with both,
+// ten codes in turn (us): plain, p = 0.03, 1146 shots (2 loads) 258 / 269, 4000 (6)
+// 631 / 630, 10000 (16) 1437 / 1327, 30000 (47) 4028 / 3709; EWAInit, p = 0.06,
+// 4000 shots 479 / 510, 10000 1007 / 988, 30000 2765 / 2581; 262144 shots 24.7 /
+// 21.2 ms.
 constexpr long kManyLoads = 8;
+// A smaller group's shots take longer (more nodes per thread) and end last, so it
+// goes only with at most this many full groups, whose work it shares.  Without and
+// with it, EWAInit, p = 0.05, us: one group, planar d = 25, 30000 shots 5674 /
+// 4899; two, d = 19, 4000 402 / 409, 12000 990 / 942, 48000 3627 / 3329; three, d =
+// 17, 4000 283 / 325, 12000 670 / 699, 48000 2378 / 2333; four, d = 15, 6000 287 /
+// 318, 60000 1948 / 1969; ten, d = 7, 30000 131 / 162, 200000 643 / 656.
+constexpr int kRestGroups = 2;
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
@@ -140,7 +146,7 @@ int bpq_batch_plan(const bpq_batch_item *items, int n_items, int variant, const 
         bpq::DecodeArgs &a = desc[g];
         bpq::LaunchShape &s = shape[g];
         const int left = bpq::kBatchThreads - s.groups_per_cta * s.T;
-        if (many && s.groups_per_cta < 15 && 2 * left >= s.T && s.smem + s.group_bytes <= 227 * 1024) {
+        if (many && s.groups_per_cta <= bpq::kRestGroups && 2 * left >= s.T && s.smem + s.group_bytes <= 227 * 1024) {
             a.rest_warps = left / 32;
             s.smem += s.group_bytes;
         }
