@@ -62,19 +62,28 @@ int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     const size_t one_smem = pair_offsets(variant, true, t->M, n_pad).groups + group_bytes;
     int T = t->threads_per_shot, gpc = t->shots_per_cta;
     if (T <= 0) {
-        // Automatic.  Two nodes per thread, except that a code of at most 96
-        // nodes takes one warp per group (no barrier, warp votes only: planar
-        // d = 7, 10^6 shots, EWAInit 2.97 ms against 3.29 with two warps, d = 6
-        // 0.94 against 1.07; d = 8, four nodes per lane, 1.61 against 1.49), and
-        // a code of more than 512 nodes takes 256 threads where shared memory
-        // holds two such CTAs (more nodes per thread but more shots per SM:
-        // plain BP on planar d = 25, 30001 shots, 18.9 ms against 23.0, d = 21
-        // 11.9 against 13.7; with one CTA per SM it is slower: EWAInit on
-        // planar d = 25, 5.8 against 5.0).  One group per CTA but for the
-        // one-warp groups (planar d = 11 with 128 threads: 4.41 against 4.56).
+        // Automatic.  Two nodes per thread, except that
+        //  * a code of at most 96 nodes takes one warp per group (no barrier, warp
+        //    votes only: planar d = 7, 10^6 shots, EWAInit 2.97 ms against 3.29 with
+        //    two warps, d = 6 0.94 against 1.07; d = 8, four nodes per lane, 1.61
+        //    against 1.49);
+        //  * above 512 nodes 256 threads where shared memory holds two such CTAs
+        //    (more nodes per thread but more shots per SM: plain BP on planar d =
+        //    25, 30001 shots, 18.9 ms against 23.0, d = 21 11.9 against 13.7); with
+        //    variant state, which leaves room for fewer shots, only up to three
+        //    nodes for most threads (60000 shots, EWAInit at p = 0.08, two nodes /
+        //    256 threads: d = 18 7.02 / 6.72, toric d = 18 6.57 / 5.82, d = 20 8.32 /
+        //    8.36, planar d = 20 9.22 / 9.37; Momentum at p = 0.03, toric d = 20 5.76 /
+        //    6.08);
+        //  * above 1536 nodes three per thread, as the one CTA per SM has more than
+        //    768 threads otherwise (planar d = 31, 20000 shots, p = 0.03, two / three
+        //    nodes: Momentum 12.4 / 12.0, EWAInit 4.50 / 4.26, AdaGrad 16.0 / 15.3).
+        // One group per CTA but for the one-warp groups (planar d = 11 with 128
+        // threads: 4.41 against 4.56).
         T = (((nodes + 1) / 2 + 31) / 32) * 32;
         if (nodes <= 96) T = 32;
-        else if (nodes > 512 && 2 * (one_smem + 1024) <= 228 * 1024) T = 256;
+        else if (nodes > 512 && (nstate == 0 || nodes <= 672) && 2 * (one_smem + 1024) <= 228 * 1024) T = 256;
+        else if (nodes > 1536) T = (((nodes + 2) / 3 + 31) / 32) * 32;
         if (gpc <= 0) gpc = T == 32 ? 8 : 1;
     } else if ((nodes + T - 1) / T > 2) {
         return fail(BPQ_EINVAL, "two shots per thread take at most two nodes per thread");
@@ -93,13 +102,24 @@ int decode_pair_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
     s->n_pad = n_pad;
     s->slots_floats = slots;
     s->group_bytes = (uint32_t)group_bytes;
-    // one-warp groups too take the table of byte offsets, and have their size
-    // at compile time (planar d = 5, 10^6 shots, plain 4.68 -> 4.34 ms; d = 7,
-    // 500000 shots, Momentum 5.82 -> 5.53, EWAInit 1.82 -> 1.75)
+    // The table of byte offsets for one group per CTA and for one-warp groups
+    // (these have their size at compile time: planar d = 5, 10^6 shots, plain 4.68 ->
+    // 4.34 ms; d = 7, 500000 shots, Momentum 5.82 -> 5.53, EWAInit 1.82 -> 1.75),
+    // unless the 16-bit table, half its size, brings a third more CTAs onto an SM
+    // (64 registers a thread: 1024 threads).  Byte offsets / 16 bits, 60000 shots,
+    // p = 0.08, EWAInit, ms: planar d = 18 (2 / 3 CTAs of 256) 7.39 / 6.72, toric d =
+    // 18 (2 / 3) 6.30 / 5.82, planar d = 22 (1 / 2 of 480) 16.1 / 13.4, toric d = 22
+    // 13.6 / 11.0; d = 16 (3 / 4) 4.67 / 4.62; but with the same or nearly the same
+    // number toric d = 15 3.31 / 3.48, planar d = 11 Momentum (7 / 8 of 128), 150000
+    // shots, p = 0.03, 2.61 / 3.08.
     const size_t wide = one_smem + (size_t)(gpc - 1) * group_bytes;
-    s->pair_mode = wide > 227 * 1024 ? kPairGroups : gpc == 1 ? kPairOne : T == 32 ? kPairWarps : kPairGroups;
-    s->smem = s->pair_mode != kPairGroups
-                  ? wide : pair_offsets(variant, false, t->M, n_pad).groups + (size_t)gpc * group_bytes;
+    const size_t narrow = pair_offsets(variant, false, t->M, n_pad).groups + (size_t)gpc * group_bytes;
+    auto resident = [&](size_t smem) {
+        return std::min<size_t>(std::max(1, 1024 / (T * gpc)), 228 * 1024 / (smem + 1024));
+    };
+    const bool offsets = (gpc == 1 || T == 32) && wide <= 227 * 1024 && 3 * resident(narrow) < 4 * resident(wide);
+    s->pair_mode = !offsets ? kPairGroups : gpc == 1 ? kPairOne : kPairWarps;
+    s->smem = offsets ? wide : narrow;
     if (s->smem > 227 * 1024) return fail(BPQ_EINVAL, "shared memory of the launch shape exceeds 227 KB");
     return BPQ_OK;
 }
@@ -280,6 +300,20 @@ int decode_preload(const bpq_tanner *t, int variant) {
     return BPQ_OK;
 }
 
+namespace {
+// Threads of a kernel's launch shape that an SM holds at once.  Automatic pairs need
+// more than half of the one-shot kernel's: planar d = 23, one CTA of 512 threads
+// against two, 20000 shots at p = 0.03, one / two shots per thread: Momentum 4.01 /
+// 4.97 ms, EWAInit 1.47 / 1.95; p = 0.08 12.5 / 15.2, 4.70 / 5.79.
+int resident_threads(DecodeKernelFn fn, const LaunchShape &s) {
+    int per_sm = 0;
+    if (!fn || allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute") != BPQ_OK ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem) != cudaSuccess)
+        return 0;
+    return per_sm * s.T * s.groups_per_cta;
+}
+}  // namespace
+
 int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out) {
     int small_rc = BPQ_OK;
     if (!trace && launch_small(t, a, variant, st, &small_rc)) return small_rc;
@@ -311,7 +345,8 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
             decode_pair_shape(t, variant, &s) == BPQ_OK &&
-            (long)a.B < pair_shots_per_group(variant, s.T, one.T) * (long)per_sm * t->num_sms * one.groups_per_cta)
+            ((long)a.B < pair_shots_per_group(variant, s.T, one.T) * (long)per_sm * t->num_sms * one.groups_per_cta ||
+             2 * resident_threads(pick_pair(variant, s.pair_mode, a.split), s) <= per_sm * one.T * one.groups_per_cta))
             pairs = false;
     }
     int rc = pairs ? decode_pair_shape(t, variant, &s) : decode_launch_shape(t, variant, &s);

@@ -28,8 +28,8 @@
 //    place of packed indices in registers.  That also frees the registers that
 //    tied a thread to two nodes: a thread loops over any number of nodes, so
 //    large codes can take small groups, more of which fit an SM.
-//    With several larger groups per CTA (kPairGroups) the table holds 16-bit
-//    slot indices, half the size, for codes that the other would not fit.
+//    kPairGroups (several larger groups per CTA, or one where the smaller table
+//    brings a third more CTAs onto an SM): 16-bit slot indices, half the size.
 //  * a syndrome bit enters as one word whose bits 31 (sign) and 0 (parity)
 //    are both the bit; a register per lane is rotated from check to check.
 //  * the decision is kept as its two anticommutation bits, which the messages

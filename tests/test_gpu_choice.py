@@ -41,6 +41,21 @@ def decoding(bpq, t, syn, prior, variant):
     return out, lambda: bpq.decode(t, syn, prior, variant, max_iter=100, out=out, work=work)
 
 
+# Against one shot per thread
+@pytest.mark.parametrize("kind,d,variant,p,B,bar", [
+    ("planar", 22, "ewainit", 0.08, 40000, 1.12),   # 1.22: the table of byte offsets left one CTA per SM
+    ("planar", 23, "momentum", 0.03, 20000, 1.12),  # 1.24: one CTA per SM against two
+])
+def test_pairs_against_one_shot(bpq, kind, d, variant, p, B, bar):
+    t, syn, prior = inputs(bpq, kind, d, p, B)
+    out, call = decoding(bpq, t, syn, prior, variant)
+    ref = [x.clone() for x in out]
+    ms = milliseconds(call)
+    t.set_shots_per_thread(1)
+    assert ms <= bar * milliseconds(call)
+    assert all(torch.equal(x, y) for x, y in zip(ref, out))
+
+
 # A plan just above eight CTA loads per SM against one just below, per shot: the ones above form a group of
 # the threads left over where there are one or two full groups
 @pytest.mark.parametrize("d,groups,bar", [(7, 10, 1.12), (15, 4, 1.08)])  # 1.31, 1.13
