@@ -255,10 +255,12 @@ int bpq_get_launch(const bpq_tanner *t, int *threads_per_shot, int *shots_per_ct
  * next shot from the queue as soon as its own shot stops (split table layout
  * only, see bpq_tanner_layout; plain, Momentum, AdaGrad and EWAInit BP; not
  * the trace, serial, batched or AEWA-BP paths); 0 = automatic (2 where it
- * applies and the batch holds enough shots per resident one-shot shot group: 64
- * for plain and Momentum BP (128 for codes of at most 96 nodes), for EWAInit and
- * AdaGrad BP 64 for codes of more than 320 nodes, e.g. 38912 toric d = 15 shots
- * on a GB300, else 200, or 2000 for codes of at most 64 nodes: a pair's
+ * applies, an SM holds more than half as many threads of it as with 1, and the
+ * batch holds enough shots per resident one-shot group: for codes of more than
+ * 320 nodes 64 with plain, Momentum and (without padding) EWAInit BP, e.g. 38912
+ * toric d = 15 shots on a GB300, else 128; for smaller codes 128 with plain and
+ * Momentum BP, else 200; codes whose groups are one warp either way, up to 64
+ * nodes, or 32 with Momentum BP, keep 1: a pair's
  * iteration does two shots' work, so smaller batches, whose time is set by
  * their slowest shots, finish sooner with one shot per thread).  Per-shot
  * results are the same bit for bit either way.  bpq_get_shots_per_thread

@@ -325,18 +325,23 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // once each resident one-shot group would decode many shots.
         // Measured on GB300, one shot per thread against two (ms; shots per
         // resident one-shot group).  Plain and Momentum BP, whose shots mostly
-        // run long, cross early: planar d = 9 plain 60000 (39) 1.43 / 1.45, 120000
-        // (79) 2.79 / 2.73; planar d = 11 plain 100000 (82) 4.22 / 4.12; planar
-        // d = 25 plain 10000 (66) 6.00 / 5.97; one-warp pair groups: planar d = 7
-        // Momentum 500000 (205) 6.39 / 5.53, d = 5 10^6 (205) 5.14 / 5.02.  EWAInit
-        // and AdaGrad converge in few iterations, so that the slowest shots weigh
-        // more: planar d = 11 EWAInit 100000 (82) 1.50 / 1.56, d = 13 100000 (110)
-        // 2.71 / 2.73, d = 9 200000 (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38;
-        // planar d = 7 300000 (123) 0.957 / 1.011, 500000 (205) 1.85 / 1.75; large
-        // codes again earlier: toric d = 15, p = 0.08, 40000 (66) 2.41 / 2.36,
-        // p = 0.06, 20000 (33) 0.877 / 0.923.  A code whose one-shot group is one
-        // warp too gains nothing for them: planar d = 5 EWAInit 10^6 (205) 1.48 /
-        // 1.60, AdaGrad 5.74 / 5.84.
+        // run long, cross early: planar d = 13 Momentum 60000 (79), p = 0.08 and
+        // 0.03, 8.94 / 8.38 and 1.92 / 1.95, d = 25 plain 10000 (66) 6.00 / 5.97;
+        // small codes later: d = 11, p = 0.03, 150000 (123) plain 2.83 / 2.98,
+        // Momentum 2.52 / 2.61; toric d = 8 Momentum 200000 (66) 0.95 / 1.03;
+        // one-warp pair groups: planar d = 7 Momentum 500000 (205) 6.39 / 5.53.  EWAInit and AdaGrad converge in few
+        // iterations, so that the slowest shots weigh more: planar d = 11 EWAInit
+        // 100000 (82) 1.50 / 1.56, d = 13 100000 (110) 2.71 / 2.73, d = 9 200000
+        // (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38; d = 7 300000 (123) 0.957 /
+        // 1.011, 500000 (205) 1.85 / 1.75; large codes again earlier, without
+        // padding above all: toric d = 15, 60000 (99), p = 0.08 3.45 / 3.31, p = 0.03
+        // 1.21 / 1.24; planar d = 15, 60000 (79) 4.01 / 3.95 and 1.23 / 1.32; AdaGrad,
+        // 60000, p = 0.08 and 0.03: toric d = 15 13.7 / 13.5 and 3.23 / 3.44, d = 13
+        // 9.27 / 9.16 and 2.15 / 2.34, planar d = 15 17.4 / 16.8 and 3.91 / 4.05.  A
+        // code whose one-shot group is one warp too gains nothing, 10^6 shots (205):
+        // planar d = 4 plain 0.75 / 0.96, Momentum 1.57 / 1.83, d = 5 plain 1.58 /
+        // 1.86, EWAInit 1.75 / 1.91, AdaGrad 2.25 / 2.66; but Momentum with two nodes
+        // per lane at p = 0.08: d = 5 8.52 / 8.08, d = 6 10.8 / 10.2.
         LaunchShape one;
         int per_sm = 0;
         DecodeKernelFn f1 = nullptr;
@@ -345,7 +350,7 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
             decode_pair_shape(t, variant, &s) == BPQ_OK &&
-            ((long)a.B < pair_shots_per_group(variant, s.T, one.T) * (long)per_sm * t->num_sms * one.groups_per_cta ||
+            ((long)a.B < pair_shots_per_group(variant, s.T, one.T, std::max(t->N, t->M), t->full) * (long)per_sm * t->num_sms * one.groups_per_cta ||
              2 * resident_threads(pick_pair(variant, s.pair_mode, a.split), s) <= per_sm * one.T * one.groups_per_cta))
             pairs = false;
     }
