@@ -222,7 +222,7 @@ int decode_batch_shape(const bpq_tanner *t, int variant, LaunchShape *s) {
 namespace {
 
 // Launch of a small batch (decode_small.cu): one CTA per shot, `lanes` lanes
-// per node, every shot resident at once.  Returns false if the batch, the code
+// per node, every shot resident at once (or in two rounds).  Returns false if the batch, the code
 // or the handle's launch preferences call for the queue kernels.
 //
 // Measured (kernel and launch, EWAInit or Momentum, us), against one node per
@@ -237,15 +237,27 @@ bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t 
     if (a.split == 0 || t->threads_per_shot || t->shots_per_cta || t->shots_per_thread) return false;
     const int nodes = t->N > t->M ? t->N : t->M;
     const long shots_per_sm = ((long)a.B + t->num_sms - 1) / t->num_sms;
-    if (nodes > 1024 || shots_per_sm > 32) return false;
     int lanes = 4;
     while (lanes > 1 && lanes * nodes * shots_per_sm > 640) lanes /= 2;
+    // AdaGrad on a large code fills the SM's issue slots with fewer threads (304
+    // shots, us, this / one node per thread in the queue kernel: toric d = 15 (900
+    // nodes of an SM) 162 / 124, planar d = 15 (842) 111 / 144)
+    if (variant == BPQ_ADAGRAD && nodes > 256 && nodes * shots_per_sm > 864) return false;
+    // Large codes, whose CTAs nearly fill an SM, take two rounds of them: 304 shots,
+    // us, this / one node per thread in the queue kernel / two: Momentum at p = 0.05
+    // planar d = 18 105 / 126 / 172, toric d = 20 134 / 158 / 195, planar d = 22 228 /
+    // 261 / 236; EWAInit at p = 0.08 97 / 110 / 157, 127 / 133 / 178, 153 / 165 / 215.
+    // So do the tiniest, whose CTAs are over first where the queue kernel starts its
+    // CTAs and tables: 7000 shots of Momentum, this / queue: planar d = 2 62 / 85, d =
+    // 3 42 / 60, d = 4 58 / 69
+    const int rounds = nodes <= 32 || (nodes > 512 && variant != BPQ_ADAGRAD && variant != BPQ_AEWA) ? 2 : 1;
+    if (nodes > 1024 || shots_per_sm > 32 * rounds) return false;
     const int threads = (lanes * nodes + 31) / 32 * 32;
     const size_t smem = 16 * (size_t)((t->N + 3) & ~3);
     SmallKernelFn fn = pick_small(variant, lanes);
     int per_sm = 0;
     if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess ||
-        shots_per_sm > per_sm)
+        shots_per_sm > rounds * per_sm)
         return false;
     if (t->debug_checks && !(fn = pick_debug_small(variant, lanes))) return false;
     a.n_pad = (t->N + 3) & ~3;
@@ -260,12 +272,22 @@ bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t 
 }
 
 // One node per thread instead of the automatic two for batches of fewer than
-// this many shots per resident two-node group: they are bound by their slowest
-// shots, whose iterations are shorter then (kernel and launch, ms, two nodes
-// against one: planar d = 9 Momentum 1000 shots 0.139 / 0.112, 5000 (3.3 per
-// group) 0.209 / 0.183; toric d = 15 1000 (1.6 per group) 0.175 / 0.158, 5000
-// (8.2 per group) 0.407 / 0.447).
-constexpr long kOneNodeShotsPerGroup = 3;
+// this many half shots per resident two-node group: they are bound by their slowest
+// shots, whose iterations are shorter then (kernel and launch, us, two nodes against
+// one, p = 0.05: planar d = 9 Momentum 1000 shots 139 / 112, 5000 (3.3 per group)
+// 209 / 183; toric d = 15 Momentum 912 (1.2) 198 / 168, 1520 (2) 234 / 225, 2432
+// (3.2) 293 / 308).  But once an SM is full a shot of one node per thread costs it
+// more, so the line is lower the larger the code, for plain and Momentum BP above
+// all, which run most shots to the end: Momentum at p = 0.08 toric d = 15, 1500 shots
+// (2) 353 / 391, d = 20, 300 (0.7) 193 / 225, planar d = 18, 300 (0.5) 173 / 191, 700
+// (1.2) 344 / 384; EWAInit, p = 0.08: toric d = 20 608 (1.3) 207 / 197, 912 (2) 232 /
+// 250; AdaGrad, p = 0.03: planar d = 18 912 (2) 324 / 221.
+constexpr long one_node_half_shots(int variant, int nodes) {
+    const bool long_runs = variant == BPQ_PLAIN || variant == BPQ_MOMENTUM;
+    if (nodes <= 256 || variant == BPQ_ADAGRAD || variant == BPQ_AEWA) return 6;
+    if (nodes <= 512) return long_runs ? 3 : 6;
+    return long_runs ? 0 : 4;
+}
 
 }  // namespace
 
@@ -372,8 +394,9 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
     if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
     const int nodes = t->N > t->M ? t->N : t->M;
+    const long groups = (long)per_sm * t->num_sms * s.groups_per_cta;
     if (!pairs && !trace && s.npt == 2 && !t->threads_per_shot && !t->shots_per_cta && nodes <= kMaxThreadsPerShot &&
-        (long)a.B < kOneNodeShotsPerGroup * per_sm * t->num_sms * s.groups_per_cta) {
+        2L * a.B < one_node_half_shots(variant, nodes) * groups) {
         rc = one_shot_shape(t, variant, (nodes + 31) / 32 * 32, 0, &s);
         if (rc) return rc;
         s.smem -= s.init_bytes;  // too few shots per group to repay the table

@@ -66,6 +66,23 @@ def test_when_pairs_start(bpq, kind, d, variant, p, B, bar):
     test_pairs_against_one_shot(bpq, kind, d, variant, p, B, bar)
 
 
+# Against two nodes per thread
+@pytest.mark.parametrize("kind,d,variant,p,B,bar", [
+    ("planar", 18, "momentum", 0.08, 700, 1.06),    # 1.11: one node per thread
+    ("toric", 15, "momentum", 0.08, 1500, 1.06),    # 1.11
+    ("toric", 15, "adagrad", 0.03, 300, 1.02),      # 1.05: one CTA per shot
+])
+def test_small_batches_against_two_nodes_per_thread(bpq, kind, d, variant, p, B, bar):
+    t, syn, prior = inputs(bpq, kind, d, p, B)
+    out, call = decoding(bpq, t, syn, prior, variant)
+    ref = [x.clone() for x in out]
+    ms = milliseconds(call)
+    t.set_shots_per_thread(1)
+    t.set_launch((max(t.N, t.M) + 63) // 64 * 32, 0)
+    assert ms <= bar * milliseconds(call)
+    assert all(torch.equal(x, y) for x, y in zip(ref, out))
+
+
 # A plan just above eight CTA loads per SM against one just below, per shot: the ones above form a group of
 # the threads left over where there are one or two full groups
 @pytest.mark.parametrize("d,groups,bar", [(7, 10, 1.12), (15, 4, 1.08)])  # 1.31, 1.13
