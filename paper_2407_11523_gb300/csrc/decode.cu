@@ -334,6 +334,8 @@ int resident_threads(DecodeKernelFn fn, const LaunchShape &s) {
         return 0;
     return per_sm * s.T * s.groups_per_cta;
 }
+constexpr long kInitShotsPerGroup = 8;
+
 }  // namespace
 
 int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out) {
@@ -399,14 +401,20 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         2L * a.B < one_node_half_shots(variant, nodes) * groups) {
         rc = one_shot_shape(t, variant, (nodes + 31) / 32 * 32, 0, &s);
         if (rc) return rc;
-        s.smem -= s.init_bytes;  // too few shots per group to repay the table
-        s.init_bytes = 0;
         fn = t->debug_checks ? pick_debug(variant, s.npt, false, 0, a.split) : pick(variant, s.npt, false, a.split);
         if (!fn) return fail(BPQ_EINVAL, "no kernel for this variant");
         rc = allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute");
         if (rc) return rc;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.T * s.groups_per_cta, s.smem);
         if (e != cudaSuccess || per_sm < 1) return fail(BPQ_ECUDA, "launch shape does not fit on an SM");
+    }
+    // The initial messages' table, made by every CTA, pays from some shots per group
+    // on (kernel and launch, us, with / without it, p = 0.03): toric d = 20 EWAInit,
+    // 1500 shots (3.3 per group) 153 / 137; d = 3, 8000 (1.3) 26.3 / 25.4; planar d = 2
+    // plain, 8000, p = 0.08 92.5 / 87.8; d = 9 and 11, 8 per group, the same.
+    if (!pairs && !trace && (long)a.B < kInitShotsPerGroup * per_sm * t->num_sms * s.groups_per_cta) {
+        s.smem -= s.init_bytes;
+        s.init_bytes = 0;
     }
     const int threads = s.T * s.groups_per_cta;
     long ctas = (long)per_sm * t->num_sms;
