@@ -273,8 +273,8 @@ int bpq_get_shots_per_thread(const bpq_tanner *t, int variant, int *shots_per_th
 
 /* Bounds-checked decoding (a test aid; the paper has no counterpart): with
  * on != 0, bpq_decode and bpq_decode_host run copies of the decode kernels
- * compiled with checks on every shared-memory layout, slot index, table
- * offset and output index.  A failed check sets the device error word that
+ * (small batches' too) compiled with checks on every shared-memory layout, slot
+ * index, table offset and output index.  A failed check sets the device error word that
  * bpq_decode_status reads (value 5), substitutes a safe index and carries on
  * (or, for a layout that does not fit, makes the CTA return before its first
  * barrier); nothing traps.  Results are those of the unchecked kernels when

@@ -710,7 +710,7 @@ int bpq_decode(const bpq_tanner *t, const uint32_t *syn_dev, const float *prior_
     a.conv = conv_dev;
     a.iters = iters_dev;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return bpq::decode_launch(t, a, variant, false, st, nullptr);
+    return bpq::decode_launch(t, a, variant, false, st);
 }
 
 int bpq_decode_status(const void *work_dev, void *stream, int *device_error) {
@@ -785,7 +785,7 @@ int bpq_decode_trace(const bpq_tanner *t, const uint32_t *syn_dev, const float *
     a.tr_Q = Q_dev;
     a.tr_dec = dec_dev;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return bpq::decode_launch(t, a, variant, true, st, nullptr);
+    return bpq::decode_launch(t, a, variant, true, st);
 }
 
 int bpq_set_launch(bpq_tanner *t, int threads_per_shot, int shots_per_cta) {

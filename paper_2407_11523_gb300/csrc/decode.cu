@@ -146,7 +146,7 @@ int one_shot_shape(const bpq_tanner *t, int variant, int T, int gpc, LaunchShape
     s->npt = npt;
     s->groups_per_cta = gpc;
     s->n_pad = (t->N + 3) & ~3;
-    // message slots (+ zero and trash slots), state
+    // message slots (+ the zero slot, padded), state
     s->slots_floats = (uint32_t)(4 * s->n_pad + 4);
     const int nstate = state_arrays(variant < 0 ? BPQ_MOMENTUM : variant);
     s->group_bytes = (uint32_t)(4 * s->slots_floats + 4 * nstate * s->n_pad);
@@ -155,7 +155,7 @@ int one_shot_shape(const bpq_tanner *t, int variant, int T, int gpc, LaunchShape
     // the initial messages, unless they cost a resident CTA (48 registers a
     // thread: 1280 threads per SM).  Without and with them: AdaGrad on xzzx
     // d = 7, 5.7 iterations a shot, 200000 shots, 1.30 and 1.24 ms; AEWA on planar
-    // d = 11, 11.3 iterations, 10^5 shots, 11.3 and 11.2
+    // d = 11, 11.3 iterations in a shot's last run, 10^5 shots, 11.3 and 11.2
     const size_t init = 16 * (size_t)s->n_pad, by_threads = std::max(1, 1280 / (T * gpc));
     auto resident = [&](size_t smem) { return std::min<size_t>(by_threads, 228 * 1024 / (smem + 1024)); };
     s->init_bytes = 0;
@@ -338,7 +338,7 @@ constexpr long kInitShotsPerGroup = 8;
 
 }  // namespace
 
-int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st, int *ctas_out) {
+int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, cudaStream_t st) {
     int small_rc = BPQ_OK;
     if (!trace && launch_small(t, a, variant, st, &small_rc)) return small_rc;
     LaunchShape s;
@@ -353,8 +353,9 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // 0.03, 8.94 / 8.38 and 1.92 / 1.95, d = 25 plain 10000 (66) 6.00 / 5.97;
         // small codes later: d = 11, p = 0.03, 150000 (123) plain 2.83 / 2.98,
         // Momentum 2.52 / 2.61; toric d = 8 Momentum 200000 (66) 0.95 / 1.03;
-        // one-warp pair groups: planar d = 7 Momentum 500000 (205) 6.39 / 5.53.  EWAInit and AdaGrad converge in few
-        // iterations, so that the slowest shots weigh more: planar d = 11 EWAInit
+        // one-warp pair groups: planar d = 7 Momentum 500000 (205) 6.39 / 5.53.
+        // EWAInit and AdaGrad converge in few iterations, so that the slowest shots
+        // weigh more: planar d = 11 EWAInit
         // 100000 (82) 1.50 / 1.56, d = 13 100000 (110) 2.71 / 2.73, d = 9 200000
         // (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38; d = 7 300000 (123) 0.957 /
         // 1.011, 500000 (205) 1.85 / 1.75; large codes again earlier, without
@@ -374,7 +375,8 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
             decode_pair_shape(t, variant, &s) == BPQ_OK &&
-            ((long)a.B < pair_shots_per_group(variant, s.T, one.T, std::max(t->N, t->M), t->full) * (long)per_sm * t->num_sms * one.groups_per_cta ||
+            ((long)a.B < pair_shots_per_group(variant, s.T, one.T, std::max(t->N, t->M), t->full) * (long)per_sm *
+                             t->num_sms * one.groups_per_cta ||
              2 * resident_threads(pick_pair(variant, s.pair_mode, a.split), s) <= per_sm * one.T * one.groups_per_cta))
             pairs = false;
     }
@@ -427,7 +429,6 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     a.slots_floats = s.slots_floats;
     a.group_bytes = s.group_bytes;
     a.init_bytes = pairs ? 0 : s.init_bytes;
-    if (ctas_out) *ctas_out = (int)ctas;
     rc = cuda_check(cudaMemsetAsync(a.work, 0, 8, st), "workspace reset");  // the shot queue, the error word
     if (rc) return rc;
     fn<<<(unsigned)ctas, threads, s.smem, st>>>(a);

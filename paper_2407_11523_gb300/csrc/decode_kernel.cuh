@@ -54,7 +54,7 @@
 // Specialisations: SPLIT (tables whose qubits have at most two X and two Z
 // edges: the edge type is fixed by its position, so no per-edge Pauli
 // selects) and FULL (split tables without padding, e.g. the toric codes: no
-// zero/trash slot choice, no unused positions, no check-side clip).
+// test for the zero slot, no unused positions, no check-side clip).
 //
 // Bounds-checked build: with BPQ_DEBUG defined (decode_debug_*.cu compile
 // these headers a second time, into namespace dk_debug), every CTA checks its
@@ -166,11 +166,6 @@ __device__ __forceinline__ int group_any(int G, int bar_id, int pred) {
         : "r"(pred), "r"(bar_id), "r"(G * 32)
         : "memory");
     return r;
-}
-
-// <A, B> for single-qubit Pauli codes (0 = I, 1 = X, 2 = Y, 3 = Z).
-__device__ __forceinline__ uint32_t anti(uint32_t a, uint32_t b) {
-    return (a != 0u) & (b != 0u) & (a != b);
 }
 
 constexpr float kLog2e = 1.4426950408889634f;

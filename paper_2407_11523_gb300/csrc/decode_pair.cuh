@@ -90,7 +90,7 @@ struct PairPrior {
 // Shared memory of the CTA: header | idx (int4 or ushort4 per check) | used
 // positions of each qubit (bytes) | Pi [3][n_pad] | initial messages
 // [4 n_pad] | groups.  A group: two vote words (16 bytes), the float2 message
-// slots (4 n_pad + the zero slot + the trash slot, padded to 4 n_pad + 4) and
+// slots (4 n_pad + the zero slot, padded to 4 n_pad + 4) and
 // the variant state (float2 [arrays][n_pad]).
 struct PairMem {
     const uint8_t *idx, *used;
