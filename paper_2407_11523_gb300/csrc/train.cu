@@ -66,8 +66,8 @@
 // Training step (Momentum, coset loss, planar d = 9, T = 25, 4096 shots), with
 // phi, its inverse, lambda and their derivatives evaluated per edge: 932 us
 // forward, 3590 us backward, gradients 1.4e-6 off float64; so arranged: 652 us,
-// 2018 us, 1.8e-7; with adjacency in registers and approximate divisions 601 us,
-// 1597 us, 2.9e-7.
+// 2018 us, 1.8e-7; with adjacency in registers and approximate divisions 635 us,
+// 1604 us, 2.9e-7.
 #include <cuda_runtime.h>
 
 #include <algorithm>
