@@ -164,14 +164,10 @@ int serial_launch(const bpq_tanner *t, const uint32_t *syn, const float *prior, 
     const long per_warp = 32 / shape.lanes, wave = per_warp * t->num_sms;
     const int warps = (int)std::min<long>(shape.warps, (B + wave - 1) / wave);
     const size_t smem = shape.smem(warps);
-    // with few decoding warps, further ones share the staging of the prior and the
-    // initial messages (three logarithms and the message rule per qubit), which
-    // one warp takes a qubit per lane at a time.  One shot, EWAInit, us, without /
-    // with: toric d = 27 128 / 103, d = 20 77 / 63, planar d = 25 130 / 110, d = 11
-    // 19.6 / 16.4; staging on the sweep's own arrays before (one warp, no initial
-    // messages) 105, 67, 113, 18.2
+    // the further warps of SerialHelpers
     a.warps = warps;
-    const int threads = 32 * std::max(warps, std::min(kSerialStageWarps, (t->N + 31) / 32));
+    const int threads =
+        32 * (variant == BPQ_ADAGRAD ? warps : std::max(warps, std::min(kSerialStageWarps, (t->N + 31) / 32)));
     sk::SerialKernelFn fn = mode == kSerial32   ? sk::pick_serial32(variant, trace, t->split)
                             : mode == kSerial16 ? sk::pick_serial16(variant, t->split)
                                                 : sk::pick_serial8(variant, t->split);

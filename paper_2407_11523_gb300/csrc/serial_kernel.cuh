@@ -86,12 +86,12 @@ struct SerialArgs {
     uint8_t *tr_dec;
     int N, M, E, W, B, max_iter;
     int n_pad;             // N rounded up to 4 (per-qubit array stride)
-    int warps;             // warps that decode; further warps of the CTA only stage the tables
     uint32_t zero_slot;    // message slots: [0, zero_slot) edges, then zero, no information, trash
     uint32_t shot_words;   // shared memory of one shot: messages | state | syndrome | qubit bytes
     uint32_t off_state, off_syn, off_qb, off_dec;  // word offsets inside it
     float alpha, gamma, eps, clip, clip2, delta_clip, phi_clip;
     int ada_from1;
+    int warps;             // warps that decode (SerialHelpers)
 };
 
 namespace sk {
@@ -105,6 +105,18 @@ __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 __host__ __device__ constexpr int serial_state_arrays(int variant) {
     return variant == BPQ_PLAIN ? 0 : variant == BPQ_EWAINIT ? 3 : 6;
 }
+
+// Whether a launch of few shots has further warps, which share the staging of the
+// prior and the initial messages (three logarithms and the message rule per
+// qubit: one warp takes a qubit per lane at a time) and get no shot.  One shot,
+// EWAInit, us, without / with: toric d = 27 128 / 103, d = 20 77 / 63, planar d = 25
+// 130 / 110, d = 11 19.6 / 16.4; staging on the sweep's own arrays before (one warp,
+// no initial messages) 105, 67, 113, 18.2.  Not for AdaGrad, whose sweeps the
+// compiler's code for it slows (toric d = 15, 30000 shots, 5.95 ms against 5.52).
+template <int VARIANT>
+struct SerialHelpers {
+    static constexpr bool value = VARIANT != BPQ_ADAGRAD;
+};
 
 // The four edge Paulis of a qubit one per byte (anti_bytes' format).
 __device__ __forceinline__ uint32_t pauli_bytes(uint32_t pauli) {
@@ -487,7 +499,8 @@ __global__ void __launch_bounds__(32 * serial_max_warps(LANES), 1) serial_kernel
     constexpr int K = 32 / LANES;  // shots per warp
     SerialTab tab;
     uint32_t *mem;
-    if (!stage_serial<VARIANT, SPLIT>(a, smem, K * a.warps, tab, &mem)) return;
+    constexpr bool HELPERS = SerialHelpers<VARIANT>::value;
+    if (!stage_serial<VARIANT, SPLIT>(a, smem, K * (HELPERS ? a.warps : (int)(blockDim.x >> 5)), tab, &mem)) return;
     const int lane = threadIdx.x & 31, g = lane / LANES, ln = lane % LANES;
     const int h = ln % Q, pos = ln / Q;
     ShotMem m;
@@ -508,8 +521,8 @@ __global__ void __launch_bounds__(32 * serial_max_warps(LANES), 1) serial_kernel
             // a warp that only staged the tables: no shot, and it ends here.  (A return
             // above the loop costs every warp of it: toric d = 15, 10^5 shots, EWAInit
             // 3.26 ms against 3.16.)
-            int s = a.B;
-            if (start && ln == 0 && (int)(threadIdx.x >> 5) < a.warps) s = (int)atomicAdd(a.work, 1u);
+            int s = HELPERS ? a.B : 0;
+            if (start && ln == 0 && (!HELPERS || (int)(threadIdx.x >> 5) < a.warps)) s = (int)atomicAdd(a.work, 1u);
             s = __shfl_sync(0xffffffffu, s, g * LANES);
             if (start) {
                 shot = s;
