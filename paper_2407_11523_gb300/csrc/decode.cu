@@ -324,9 +324,11 @@ int decode_preload(const bpq_tanner *t, int variant) {
 
 namespace {
 // Threads of a kernel's launch shape that an SM holds at once.  Automatic pairs need
-// more than half of the one-shot kernel's: planar d = 23, one CTA of 512 threads
-// against two, 20000 shots at p = 0.03, one / two shots per thread: Momentum 4.01 /
-// 4.97 ms, EWAInit 1.47 / 1.95; p = 0.08 12.5 / 15.2, 4.70 / 5.79.
+// more than half of the one-shot kernel's if they are one group, all of which waits
+// at its barriers: planar d = 23, one CTA of 512 threads against two, 20000 shots at p
+// = 0.03, one / two shots per thread: Momentum 4.01 / 4.97 ms, EWAInit 1.47 / 1.95; p
+// = 0.08 12.5 / 15.2, 4.70 / 5.79.  Two groups are ahead with fewer: planar d = 25
+// plain, two of 256 threads against two of 608, 30001 shots at p = 0.06 19.4 / 18.9.
 int resident_threads(DecodeKernelFn fn, const LaunchShape &s) {
     int per_sm = 0;
     if (!fn || allow_smem(fn, kMaxDynamicSmem, "cudaFuncSetAttribute") != BPQ_OK ||
@@ -374,11 +376,15 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
             allow_smem(f1, kMaxDynamicSmem, "cudaFuncSetAttribute") == BPQ_OK &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f1, one.T * one.groups_per_cta, one.smem) ==
                 cudaSuccess &&
-            decode_pair_shape(t, variant, &s) == BPQ_OK &&
-            ((long)a.B < pair_shots_per_group(variant, s.T, one.T, std::max(t->N, t->M), t->full) * (long)per_sm *
-                             t->num_sms * one.groups_per_cta ||
-             2 * resident_threads(pick_pair(variant, s.pair_mode, a.split), s) <= per_sm * one.T * one.groups_per_cta))
-            pairs = false;
+            decode_pair_shape(t, variant, &s) == BPQ_OK) {
+            const int one_threads = per_sm * one.T * one.groups_per_cta;
+            pairs = (long)a.B >= pair_shots_per_group(variant, s.T, one.T, std::max(t->N, t->M), t->full) *
+                                     (long)per_sm * t->num_sms * one.groups_per_cta;
+            if (pairs) {
+                const int threads = resident_threads(pick_pair(variant, s.pair_mode, a.split), s);
+                pairs = threads > s.T || 2 * threads > one_threads;
+            }
+        }
     }
     int rc = pairs ? decode_pair_shape(t, variant, &s) : decode_launch_shape(t, variant, &s);
     if (rc) return rc;

@@ -569,10 +569,11 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const Owned<NPT>
     const float *PiS = m.PiS;
     const uint2 *chk = reinterpret_cast<const uint2 *>(m.tab);  // four 16-bit slots per check
     const uint8_t *vps = m.tab + a.off_var_pauli;
-    // owned nodes of thread 0.  The loops over them that run once a shot are
-    // unrolled too: counted at run time they cost codes of one node per thread,
+    // owned nodes of thread 0.  The loops over them that run once a shot end after
+    // the first with one node per thread: counted at run time they cost such codes,
     // whose shots take few iterations, 5 % (10^6 shots, ms: planar d = 2 plain 1.71
-    // and 1.59, d = 4 Momentum 1.66 and 1.57)
+    // and 1.59, d = 4 Momentum 1.66 and 1.57).  (With two, unrolled loops take 64
+    // registers, not 56: planar d = 25 plain, 8000 shots, 3.47 ms against 3.07)
     const int nk = NPT ? NPT : ((M > N ? M : N) + T - 1) / T;
 
     // syndrome bits of the owned checks: that of the k-th is at bits 31 (sign)
@@ -580,22 +581,17 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const Owned<NPT>
     uint32_t syn = 0;
     {
         const uint32_t *src = a.syn + (size_t)shot * a.W;
-#pragma unroll (NPT ? NPT : 1)
-        for (int k = 0; k < nk; ++k) {
-            const int i = k * T + tg;
-            if (i >= M) break;
+        for (int i = tg, k = 0; i < M; i += T, k += 2) {
             const uint32_t w = STAGED ? *reinterpret_cast<const volatile uint32_t *>(src + (i >> 5)) : __ldg(src + (i >> 5));
-            if ((w >> (i & 31)) & 1u) syn |= __funnelshift_r(0x80000001u, 0x80000001u, 2 * k);
+            if ((w >> (i & 31)) & 1u) syn |= __funnelshift_r(0x80000001u, 0x80000001u, k);
+            if (NPT == 1) break;
         }
     }
 
     // eq. (init): lambda(Pi^(0)), i.e. the variable pass with Q = Pi^(0)
     // and no incoming messages; Q^(0) = Pi^(0), g^(0) = G^(0) = 0; EWAInit
     // starts from Pi^(1) = Pi^(0) and keeps alpha Pi^(0)
-#pragma unroll (NPT ? NPT : 1)
-    for (int k = 0; k < nk; ++k) {
-        const int j = k * T + tg;
-        if (j >= N) break;
+    for (int j = tg; j < N; j += T) {
         if (StateArrays<VARIANT>::n >= 3) {
 #pragma unroll
             for (int w = 0; w < 3; ++w) {
@@ -616,6 +612,7 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const Owned<NPT>
             emit_v2c<TRACE, SPLIT, PHI, true, FULL>(a, sp, slots, j, 0, shot, vps[j], PiS[j], PiS[Np + j],
                                                     PiS[2 * Np + j], z4, 0u);
         }
+        if (NPT == 1) break;
     }
     group_sync(G, bar_id);
 
@@ -789,14 +786,12 @@ __device__ __forceinline__ int decode_shot(const DecodeArgs &a, const Owned<NPT>
 
     // ---- outputs ----
     if (!TRACE || a.est) {
-        int sh = NPT == 1 ? 2 : NPT == 2 ? (tg + T < N ? 4 : 2) : 2 * ((N - tg + T - 1) / T);
-#pragma unroll (NPT ? NPT : 1)
-        for (int k = 0; k < nk; ++k) {
-            const int j = k * T + tg;
-            if (j >= N) break;
+        int sh = NPT == 1 ? 2 : 2 * ((N - tg + T - 1) / T);
+        for (int j = tg; j < N; j += T) {
             sh -= 2;
             if (BPQ_IN_BOUNDS((size_t)shot * N + j, (size_t)a.B * N, a.work + 1))
                 a.est[(size_t)shot * N + j] = (uint8_t)decision_code<SPLIT>((dec >> sh) & 3u);
+            if (NPT == 1) break;
         }
     }
     if (tg == 0 && (!TRACE || a.conv) && BPQ_IN_BOUNDS(shot, a.B, a.work + 1)) {
