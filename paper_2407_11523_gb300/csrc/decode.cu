@@ -271,22 +271,20 @@ bool launch_small(const bpq_tanner *t, DecodeArgs &a, int variant, cudaStream_t 
     return true;
 }
 
-// One node per thread instead of the automatic two for batches of fewer than
-// this many half shots per resident two-node group: they are bound by their slowest
-// shots, whose iterations are shorter then (kernel and launch, us, two nodes against
-// one, p = 0.05: planar d = 9 Momentum 1000 shots 139 / 112, 5000 (3.3 per group)
-// 209 / 183; toric d = 15 Momentum 912 (1.2) 198 / 168, 1520 (2) 234 / 225, 2432
-// (3.2) 293 / 308).  But once an SM is full a shot of one node per thread costs it
-// more, so the line is lower the larger the code, for plain and Momentum BP above
-// all, which run most shots to the end: Momentum at p = 0.08 toric d = 15, 1500 shots
-// (2) 353 / 391, d = 20, 300 (0.7) 193 / 225, planar d = 18, 300 (0.5) 173 / 191, 700
-// (1.2) 344 / 384; EWAInit, p = 0.08: toric d = 20 608 (1.3) 207 / 197, 912 (2) 232 /
-// 250; AdaGrad, p = 0.03: planar d = 18 912 (2) 324 / 221.
+// One node per thread instead of the automatic two for batches of fewer than three
+// shots per resident two-node group: they are bound by their slowest shots, whose
+// iterations are shorter then (kernel and launch, us, two nodes against one:
+// planar d = 9 Momentum, p = 0.05, 1000 shots 139 / 112, 5000 (3.3 per group) 209 /
+// 183; toric d = 15 Momentum 912 (1.2) 198 / 168, 1520 (2) 234 / 225, 2432 (3.2) 293 /
+// 308; at p = 0.03 planar d = 18, 700 (1.2) plain 213 / 160, Momentum 220 / 158,
+// planar d = 15 Momentum 1500 211 / 164; EWAInit toric d = 20 700 126 / 109).  Once
+// an SM is full a shot of one node per thread costs it more, so where most shots run
+// long two nodes are ahead on large codes: Momentum at p = 0.08 toric d = 15, 1500,
+// 353 / 391, d = 20, 700 391 / 440, planar d = 18, 700 344 / 384; but the prior is
+// not the host's to read.  Plain BP, most of whose shots run long at p = 0.03 too,
+// takes two nodes above 700 (toric d = 20, 700 shots 186 / 215).
 constexpr long one_node_half_shots(int variant, int nodes) {
-    const bool long_runs = variant == BPQ_PLAIN || variant == BPQ_MOMENTUM;
-    if (nodes <= 256 || variant == BPQ_ADAGRAD || variant == BPQ_AEWA) return 6;
-    if (nodes <= 512) return long_runs ? 3 : 6;
-    return long_runs ? 0 : 4;
+    return variant == BPQ_PLAIN && nodes > 700 ? 0 : 6;
 }
 
 }  // namespace

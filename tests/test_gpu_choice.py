@@ -68,8 +68,7 @@ def test_when_pairs_start(bpq, kind, d, variant, p, B, bar):
 
 # Against two nodes per thread
 @pytest.mark.parametrize("kind,d,variant,p,B,bar", [
-    ("planar", 18, "momentum", 0.08, 700, 1.06),    # 1.11: one node per thread
-    ("toric", 15, "momentum", 0.08, 1500, 1.06),    # 1.11
+    ("toric", 20, "plain", 0.03, 700, 1.06),        # 1.14: one node per thread
     ("toric", 15, "adagrad", 0.03, 300, 1.02),      # 1.05: one CTA per shot
 ])
 def test_small_batches_against_two_nodes_per_thread(bpq, kind, d, variant, p, B, bar):
