@@ -334,7 +334,7 @@ int resident_threads(DecodeKernelFn fn, const LaunchShape &s) {
         return 0;
     return per_sm * s.T * s.groups_per_cta;
 }
-constexpr long kInitShotsPerGroup = 8;
+constexpr long kInitShotsPerGroup = 4;
 
 }  // namespace
 
@@ -416,8 +416,9 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
     }
     // The initial messages' table, made by every CTA, pays from some shots per group
     // on (kernel and launch, us, with / without it, p = 0.03): toric d = 20 EWAInit,
-    // 1500 shots (3.3 per group) 153 / 137; d = 3, 8000 (1.3) 26.3 / 25.4; planar d = 2
-    // plain, 8000, p = 0.08 92.5 / 87.8; d = 9 and 11, 8 per group, the same.
+    // 1500 shots (3.3 per group) 151 / 145; d = 3, 8000 (1.3) 26.3 / 25.4; planar d = 2
+    // plain, 8000, p = 0.08 92.5 / 87.8; planar d = 5 Momentum, 20000 (4.1) 132 / 146, d =
+    // 13 EWAInit, 4800 (5.2) 145 / 151.
     if (!pairs && !trace && (long)a.B < kInitShotsPerGroup * per_sm * t->num_sms * s.groups_per_cta) {
         s.smem -= s.init_bytes;
         s.init_bytes = 0;
