@@ -255,17 +255,16 @@ int bpq_get_launch(const bpq_tanner *t, int *threads_per_shot, int *shots_per_ct
  * next shot from the queue as soon as its own shot stops (split table layout
  * only, see bpq_tanner_layout; plain, Momentum, AdaGrad and EWAInit BP; not
  * the trace, serial, batched or AEWA-BP paths); 0 = automatic (2 where it
- * applies, an SM holds more than half as many threads of it as with 1, and the
- * batch holds enough shots per resident one-shot group: for codes of more than
- * 320 nodes 64 with plain, Momentum and (without padding) EWAInit BP, e.g. 38912
- * toric d = 15 shots on a GB300, else 128; for smaller codes 128 with plain and
- * Momentum BP, else 200; codes whose groups are one warp either way, up to 64
- * nodes, or 32 with Momentum BP, keep 1: a pair's
- * iteration does two shots' work, so smaller batches, whose time is set by
- * their slowest shots, finish sooner with one shot per thread).  Per-shot
- * results are the same bit for bit either way.  bpq_get_shots_per_thread
- * reports what bpq_decode
- * will use for `variant` on large batches.
+ * applies, an SM holds two groups of it or more than half as many threads as
+ * with 1, and the batch holds enough shots per resident one-shot group: 64 with
+ * plain and Momentum BP, 128 up to 96 nodes; with EWAInit and AdaGrad BP 200 up to
+ * 320 nodes, 128 above, or 64 with EWAInit without padding, e.g. 38912 toric d = 15
+ * shots on a GB300; codes whose groups are one warp either way, up to 64 nodes, or
+ * 32 with Momentum BP, keep 1: a pair's iteration does two shots' work, so
+ * smaller batches, whose time is set by their slowest shots, finish sooner with
+ * one shot per thread).  Per-shot results are the same bit for bit either way.
+ * bpq_get_shots_per_thread reports what bpq_decode will use for `variant` on
+ * large batches.
  * Errors: EINVAL (value outside 0..2, 2 on a table without the split
  * layout, a stored launch shape that does not fit). */
 int bpq_set_shots_per_thread(bpq_tanner *t, int shots_per_thread);

@@ -350,16 +350,15 @@ int decode_launch(const bpq_tanner *t, DecodeArgs &a, int variant, bool trace, c
         // Measured on GB300, one shot per thread against two (ms; shots per
         // resident one-shot group).  Plain and Momentum BP, whose shots mostly
         // run long, cross early: planar d = 13 Momentum 60000 (79), p = 0.08 and
-        // 0.03, 8.94 / 8.38 and 1.92 / 1.95, d = 25 plain 10000 (66) 6.00 / 5.97;
-        // small codes later: d = 11, p = 0.03, 150000 (123) plain 2.83 / 2.98,
-        // Momentum 2.52 / 2.61; toric d = 8 Momentum 200000 (66) 0.95 / 1.03;
-        // one-warp pair groups: planar d = 7 Momentum 500000 (205) 6.39 / 5.53.
-        // EWAInit and AdaGrad converge in few iterations, so that the slowest shots
-        // weigh more: planar d = 11 EWAInit
-        // 100000 (82) 1.50 / 1.56, d = 13 100000 (110) 2.71 / 2.73, d = 9 200000
-        // (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38; d = 7 300000 (123) 0.957 /
-        // 1.011, 500000 (205) 1.85 / 1.75; large codes again earlier, without
-        // padding above all: toric d = 15, 60000 (99), p = 0.08 3.45 / 3.31, p = 0.03
+        // 0.03, 8.94 / 8.38 and 1.92 / 1.95, toric d = 8 Momentum 200000 (66) 3.78 /
+        // 3.60 and 0.95 / 1.03, planar d = 11 plain 100000 (82) 4.22 / 4.12, at p =
+        // 0.03 150000 (123) 2.83 / 2.98, d = 25 plain 10000 (66) 6.00 / 5.97; one-warp
+        // pair groups: planar d = 7 Momentum 500000 (205) 6.39 / 5.53.  EWAInit and
+        // AdaGrad converge in few iterations, so that the slowest shots weigh more:
+        // planar d = 11 EWAInit 100000 (82) 1.50 / 1.56, d = 13 100000 (110) 2.71 /
+        // 2.73, d = 9 200000 (132) 1.75 / 1.77, 400000 (263) 3.43 / 3.38; d = 7 300000
+        // (123) 0.957 / 1.011, 500000 (205) 1.85 / 1.75; large codes again earlier,
+        // without padding above all: toric d = 15, 60000 (99), p = 0.08 3.45 / 3.31, p = 0.03
         // 1.21 / 1.24; planar d = 15, 60000 (79) 4.01 / 3.95 and 1.23 / 1.32; AdaGrad,
         // 60000, p = 0.08 and 0.03: toric d = 15 13.7 / 13.5 and 3.23 / 3.44, d = 13
         // 9.27 / 9.16 and 2.15 / 2.34, planar d = 15 17.4 / 16.8 and 3.91 / 4.05.  A

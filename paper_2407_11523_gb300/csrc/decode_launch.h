@@ -155,8 +155,8 @@ __host__ __device__ inline PairOffsets pair_offsets(int variant, bool wide, int 
 // group, nodes: max(N, M), full: a table without padding); measured in decode_launch.
 constexpr long pair_shots_per_group(int variant, int T, int one_T, int nodes, bool full) {
     const long never = 2000;  // one-warp groups either way: pairs gain nothing
-    if (variant == BPQ_PLAIN) return T > 160 ? 64 : one_T > 32 ? 128 : never;
-    if (variant == BPQ_MOMENTUM) return T > 160 ? 64 : nodes > 32 ? 128 : never;
+    if (variant == BPQ_PLAIN) return T > 32 ? 64 : one_T > 32 ? 128 : never;
+    if (variant == BPQ_MOMENTUM) return T > 32 ? 64 : nodes > 32 ? 128 : never;
     if (T > 160) return variant == BPQ_EWAINIT && full ? 64 : 128;
     return one_T > 32 ? 200 : never;
 }

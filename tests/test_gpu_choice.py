@@ -60,7 +60,6 @@ def test_pairs_against_one_shot(bpq, kind, d, variant, p, B, bar):
     ("planar", 4, "plain", 0.03, 1000000, 1.08),    # 1.18: one-warp groups either way
     ("toric", 13, "adagrad", 0.03, 60000, 1.04),    # 1.09: 64 shots per group
     ("planar", 16, "ewainit", 0.03, 60000, 1.05),   # 1.12: 64 shots per group
-    ("toric", 8, "momentum", 0.03, 200000, 1.04),   # 1.09: 64 shots per group
 ])
 def test_when_pairs_start(bpq, kind, d, variant, p, B, bar):
     test_pairs_against_one_shot(bpq, kind, d, variant, p, B, bar)
